@@ -20,7 +20,9 @@ BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libfehmm.so")
 SOURCES = ["rve2d.cu",
            "rve2d_k_mixed_mg_nh.cu",
+           "rve2d_k_mixed_mg_nh_small.cu",
            "rve2d_k_mixed_mg_svk.cu",
+           "rve2d_k_mixed_mg_svk_small.cu",
            "rve2d_k_mixed_bj_nh.cu",
            "rve2d_k_mixed_bj_svk.cu",
            "rve2d_k_fp64_mg_nh.cu",

@@ -40,9 +40,19 @@ struct fehmm_ctx {
   void* d_x_cur = nullptr;  // kept tangent-transfer solutions (fehmm_options.transfer_warm)
   void* d_x_comm = nullptr;
   size_t x_bytes = 0;
-  int32_t* d_queue = nullptr;
+  int32_t* d_queue = nullptr;  // [kMaxClasses] work counters
   void* d_scratch = nullptr;
   size_t scratch_bytes = 0;
+  // 2D: the points of one grid size, a launch of their own with a block shaped for that grid (a
+  // contiguous range of d_order); 3D: one class with every point
+  struct SizeClass {
+    int n, first, count, blocks;
+    size_t scratch_off;
+  };
+  std::vector<SizeClass> classes;
+  std::vector<cudaStream_t> side;  // the classes after the first run beside it
+  std::vector<cudaEvent_t> joined;
+  cudaEvent_t fork = nullptr;
   // macro mesh
   bool has_macro = false;
   MacroArgs macro{};
@@ -61,6 +71,9 @@ struct fehmm_ctx {
 };
 
 namespace {
+
+constexpr int kMaxClasses = 16;  // 2D grid sizes: even, 2..32
+constexpr int kMaxSide = 7;
 
 template <typename T>
 void dfree(T*& p) {
@@ -129,7 +142,7 @@ int fehmm_create(fehmm_ctx** out, const fehmm_options* opt) {
     delete c;
     return FEHMM_ERR_CUDA;
   }
-  if (cudaMalloc((void**)&c->d_queue, sizeof(int32_t) * 4) != cudaSuccess) {
+  if (cudaMalloc((void**)&c->d_queue, sizeof(int32_t) * kMaxClasses) != cudaSuccess) {
     cudaGetLastError();
     delete c;
     return FEHMM_ERR_OOM;
@@ -152,6 +165,9 @@ int fehmm_destroy(fehmm_ctx* c) {
   if (c->d_x_cur) cudaFree(c->d_x_cur);
   if (c->d_x_comm) cudaFree(c->d_x_comm);
   dfree(c->d_queue);
+  for (cudaStream_t t : c->side) cudaStreamDestroy(t);
+  for (cudaEvent_t e : c->joined) cudaEventDestroy(e);
+  if (c->fork) cudaEventDestroy(c->fork);
   if (c->d_scratch) cudaFree(c->d_scratch);
   dfree(c->d_rowptr);
   dfree(c->d_col);
@@ -284,9 +300,41 @@ int fehmm_bind_qps(fehmm_ctx* c, int n_qp, const int32_t* rve_of_qp) {
       return FEHMM_ERR_CUDA;
     c->x_bytes = xb;
   }
-  const int blocks = std::min(n_qp, c->num_sms);
   const bool mixed = c->opt.precision == FEHMM_PREC_MIXED;
-  const size_t sb = d == 2 ? rve2d_scratch_bytes(nn_max, mixed, blocks) : rve3d_scratch_bytes(nn_max, mixed, blocks);
+  std::vector<fehmm_ctx::SizeClass> classes;
+  size_t sb = 0;
+  if (d == 3) {
+    const int blocks = std::min(n_qp, c->num_sms);
+    classes.push_back({0, 0, n_qp, blocks, 0});
+    sb = rve3d_scratch_bytes(nn_max, mixed, blocks);
+  } else {
+    for (int first = 0; first < n_qp;) {  // order is sorted by size
+      const int nn = nodes[order[first]];
+      int end = first;
+      while (end < n_qp && nodes[order[end]] == nn) ++end;
+      const int blocks = std::min(end - first, c->num_sms * rve2d_blocks_per_sm(nn, mixed));
+      classes.push_back({c->rve_n[rve_of_qp[order[first]]], first, end - first, blocks, sb});
+      sb += (rve2d_scratch_bytes(nn, mixed, blocks) + 255) & ~size_t(255);
+      first = end;
+    }
+    while (c->side.size() < std::min<size_t>(classes.size() - 1, kMaxSide)) {
+      cudaStream_t t = nullptr;
+      cudaEvent_t e = nullptr;
+      if ((!c->fork && cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess) ||
+          cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaGetLastError();
+        c->n_qp = 0;
+        return FEHMM_ERR_CUDA;
+      }
+      c->side.push_back(t);
+      if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        c->n_qp = 0;
+        return FEHMM_ERR_CUDA;
+      }
+      c->joined.push_back(e);
+    }
+  }
   if (sb > c->scratch_bytes) {
     if (c->d_scratch) cudaFree(c->d_scratch);
     c->d_scratch = nullptr;
@@ -298,6 +346,7 @@ int fehmm_bind_qps(fehmm_ctx* c, int n_qp, const int32_t* rve_of_qp) {
     }
     c->scratch_bytes = sb;
   }
+  c->classes = classes;
   c->n_qp = n_qp;
   c->nn_max = nn_max;
   c->w_total = total;
@@ -365,15 +414,52 @@ static int rve_solve_impl(fehmm_ctx* c, const double* F, double* P, double* A, d
   a.law = c->opt.law;
   a.mg_omega = (float)c->opt.mg_omega;
   a.mg_reuse = c->opt.mg_reuse;
-  a.scratch_stride = c->opt.dim == 2 ? rve2d_scratch_stride(c->nn_max, mixed) : 0;
-  if (cudaMemsetAsync(c->d_queue, 0, sizeof(int32_t), s) != cudaSuccess) return FEHMM_ERR_CUDA;
-  const int blocks = std::min(c->n_qp, c->num_sms);
-  const cudaError_t err = c->opt.dim == 2 ? rve2d_launch(a, mixed, blocks, s) : rve3d_launch(a, mixed, blocks, s);
+  if (cudaMemsetAsync(c->d_queue, 0, sizeof(int32_t) * kMaxClasses, s) != cudaSuccess) return FEHMM_ERR_CUDA;
+  if (c->opt.dim == 3) {
+    if (rve3d_launch(a, mixed, c->classes[0].blocks, s) != cudaSuccess) {
+      cudaGetLastError();
+      return FEHMM_ERR_CUDA;
+    }
+    c->launches += 1;
+    return FEHMM_OK;
+  }
+  // One launch per grid size, the largest grid first on the caller's stream and the others beside it
+  // on the context's side streams: they are forked from the caller's stream and joined to it again,
+  // so the caller sees one ordered operation (and a capture records the fork).  Every launch walks
+  // its own range of the order; of a device list, which the host cannot split, every launch walks
+  // all items and solves those of its grid.
+  const int nc = (int)c->classes.size(), ns = std::min(nc - 1, (int)c->side.size());
+  cudaError_t err = cudaSuccess;
+  if (ns > 0) {
+    err = cudaEventRecord(c->fork, s);
+    for (int k = 0; k < ns && err == cudaSuccess; ++k) err = cudaStreamWaitEvent(c->side[k], c->fork, 0);
+  }
+  int started = 0;
+  for (int k = 0; k < nc && err == cudaSuccess; ++k) {
+    const fehmm_ctx::SizeClass& g = c->classes[k];
+    a.nn_max = g.n * g.n;
+    a.queue = c->d_queue + k;
+    a.scratch = static_cast<char*>(c->d_scratch) + g.scratch_off;
+    a.scratch_stride = rve2d_scratch_stride(a.nn_max, mixed);
+    if (list) {
+      a.only_n = nc > 1 ? g.n : 0;
+    } else {
+      a.order = c->d_order + g.first;
+      a.n_qp = g.count;
+    }
+    err = rve2d_launch(a, mixed, g.blocks, k == 0 ? s : c->side[(k - 1) % ns]);
+    if (err == cudaSuccess) ++started;
+  }
+  // joined even after a failed launch, so that nothing runs on unordered
+  for (int k = 0; k < ns; ++k) {
+    if (cudaEventRecord(c->joined[k], c->side[k]) != cudaSuccess || cudaStreamWaitEvent(s, c->joined[k], 0) != cudaSuccess)
+      err = err == cudaSuccess ? cudaErrorUnknown : err;
+  }
+  c->launches += started;
   if (err != cudaSuccess) {
     cudaGetLastError();
     return FEHMM_ERR_CUDA;
   }
-  c->launches += 1;
   return FEHMM_OK;
 }
 

@@ -51,7 +51,7 @@ __device__ __forceinline__ T warp_sum(T v) {
 }
 
 // Sum of NV values over the whole block; every thread receives the totals.
-// buf: shared memory with room for 32*NV values; blockDim.x must be a multiple of 32.
+// buf: shared memory with room for NV values per warp; blockDim.x must be a multiple of 32.
 // Contains one __syncthreads(); callers alternate buffers between consecutive calls.
 template <int NV, typename T>
 __device__ __forceinline__ void block_sum(T (&v)[NV], T* buf) {
@@ -60,14 +60,14 @@ __device__ __forceinline__ void block_sum(T (&v)[NV], T* buf) {
   for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
   if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) buf[k * 32 + warp] = v[k];
+    for (int k = 0; k < NV; ++k) buf[k * nw + warp] = v[k];
   }
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(lane < nw ? buf[k * 32 + lane] : T(0));
+  for (int k = 0; k < NV; ++k) v[k] = warp_sum(lane < nw ? buf[k * nw + lane] : T(0));
 }
 
-// Two inner products summed over a block of 16 warps, the block-level sum in FP64: each thread's
+// Two inner products summed over a block of up to 16 warps, the block-level sum in FP64: each thread's
 // partial and the warp's shuffle tree stay in T (FP32 in mixed mode), lane 0 of every warp
 // stores its warp sum as a double, and warp 0 adds the 16 warp sums of each product in FP64
 // (lanes 0-15 the first, lanes 16-31 the second, a 4-level shuffle tree in a fixed order, so

@@ -132,7 +132,8 @@ extern "C" int fehmm_rve2d_solve_fp64_noalloc(int n_qp, int grid_n, int phase_pe
     cudaGetLastError();
     return FEHMM_ERR_CUDA;
   }
-  const int blocks = std::min(std::min(n_qp, slots.num_sms), kNoallocMaxBlocks);
+  const size_t fit = kNoallocScratchDoubles / (size_t)a.scratch_stride;  // blocks that the static scratch holds
+  const int blocks = (int)std::min<size_t>(std::min(n_qp, slots.num_sms * rve2d_blocks_per_sm(a.nn_max, false)), fit);
   if (rve2d_launch_fixed_fp64(a, blocks, s) != cudaSuccess) {
     cudaGetLastError();
     return FEHMM_ERR_CUDA;

@@ -10,9 +10,16 @@
 // periodic responses to the unit macro gradients E_c; this is the paper's
 // k^H = omega/|K_delta| T^T K_T T (Eq. k-mac-element-6/7) written per unit gradient.
 //
-// GB300 layout (one RVE per SM, everything on chip):
-//  * 512 threads; thread (col, strip) owns the node pair (col, 2*strip), (col, 2*strip+1)
-//    and the two elements whose lower-left corners are those nodes.
+// GB300 layout (one RVE per block, everything on chip; 32 x 32: one block per SM, smaller grids more):
+//  * One thread per node pair (512 for 32 x 32): thread (col, strip) owns the node pair (col, 2*strip),
+//    (col, 2*strip+1) and the two elements whose lower-left corners are those nodes.  The points of each
+//    grid size are a launch of their own, so the block is no larger than its grid needs.  Measured on a
+//    GB300, mixed precision, one pass from a committed state, against 512 threads for every grid: 2000
+//    RVEs of 8 x 8 5.27 -> 2.18 ms, 1000 of 16 x 16 4.82 -> 2.54 ms, 400 of 10 x 10 2.47 -> 0.72 ms.
+//  * The six grids with a multigrid hierarchy are compiled with their size as a constant (kernel template
+//    parameter N): the V-cycle's coarse levels (40 % of the time at 32 x 32) were bound by the index
+//    arithmetic between their barriers (divisions by run-time sizes, level offsets, generic addresses),
+//    about 1100 cycles a phase.  4096 RVEs of 32 x 32: 31.2 -> 24.5 ms; 1000 of 16 x 16 2.54 -> 1.59 ms.
 //  * w (FP64) lives in shared memory; the residual is evaluated per element in FP64 and the
 //    element forces are staged in shared memory, then gathered per node (no atomics).
 //  * Mixed precision (TA = float): element tangents are staged in the block's global scratch
@@ -41,13 +48,35 @@ namespace fehmm {
 
 namespace {
 
-constexpr int kThreads2D = 512;
+constexpr int kThreads2D = 512;  // largest block: n = 32
+// Threads of a block that solves RVEs of n^2 = nn nodes: one per node pair, whole warps, and as many
+// such blocks on an SM as its registers hold.  (With 512 threads for every grid the idle warps of a small
+// one took part in every barrier and executed the vector operations on zeros.)  At least four warps: the
+// dense coarsest level spreads over them, and in FP64 each of the SM's four sub-partitions has a quarter of
+// its FP64 rate (8 x 8, 64 points, FP64: 3.63 ms with one warp, 2.64 ms with four, 3.41 ms with 16).
+template <typename TA>
+__host__ __device__ constexpr int threads2d(int nn) {
+  const int t = (nn / 2 + 31) / 32 * 32;
+  return t < 128 ? 128 : t;
+}
 
 __host__ __device__ constexpr int offx(int a) { return (a == 1 || a == 2) ? 1 : 0; }
 __host__ __device__ constexpr int offy(int a) { return a >= 2 ? 1 : 0; }
 // upper-triangle index of a symmetric 8x8 element matrix
 __host__ __device__ constexpr int tri8(int r, int c) {
   return r <= c ? r * 8 - (r * (r - 1)) / 2 + (c - r) : c * 8 - (c * (c - 1)) / 2 + (r - c);
+}
+
+// A grid size known when compiling must not be folded into the tangents' constants: folding rounds
+// every product where the run-time code contracts it into an FMA, and the results of one grid would
+// differ by the last bits from those of the general path.
+__device__ __forceinline__ float unfolded(float v) {
+  asm("" : "+f"(v));
+  return v;
+}
+__device__ __forceinline__ double unfolded(double v) {
+  asm("" : "+d"(v));
+  return v;
 }
 
 __device__ __forceinline__ double gauss01(int g) {
@@ -62,7 +91,7 @@ __device__ __forceinline__ double gauss01(int g) {
 constexpr int kMgMaxLevels = 4;  // coarse levels: 32 -> 16, 8, 4
 
 // Number of coarse levels (0: no multigrid for this grid).
-__host__ __device__ inline int mg_levels(int n) {
+__host__ __device__ constexpr int mg_levels(int n) {
   int l = 0, m = n;
   while (m > 4 && (m & 1) == 0) {
     m >>= 1;
@@ -73,7 +102,7 @@ __host__ __device__ inline int mg_levels(int n) {
 
 // Element counts (TA) of the fast region (stencils, inverted blocks, vectors, coarsest inverse)
 // and of the slow region (coarse element matrices) for grid n.
-__host__ __device__ inline long long mg_fast_elems(int n) {
+__host__ __device__ constexpr long long mg_fast_elems(int n) {
   const int L = mg_levels(n);
   if (!L) return 0;
   long long e = 0;
@@ -86,19 +115,19 @@ __host__ __device__ inline long long mg_fast_elems(int n) {
   // out-of-place Gauss-Jordan steps)
   return 2LL * n * n + e + 2 * 2 * nc + 2 * D * (D + 1);
 }
-__host__ __device__ inline long long mg_slow_elems(int n) {
+__host__ __device__ constexpr long long mg_slow_elems(int n) {
   const int L = mg_levels(n);
   long long e = 0;
   for (int l = 1; l <= L; ++l) e += 36LL * (n >> l) * (n >> l);
   return e;
 }
 // Largest region sizes over the grids a batch with n^2 <= nn_max may hold.
-__host__ __device__ inline long long mg_fast_max(int nn_max) {
+__host__ __device__ constexpr long long mg_fast_max(int nn_max) {
   long long m = 0;
   for (int n = 2; n * n <= nn_max; n += 2) m = mg_fast_elems(n) > m ? mg_fast_elems(n) : m;
   return m;
 }
-__host__ __device__ inline long long mg_slow_max(int nn_max) {
+__host__ __device__ constexpr long long mg_slow_max(int nn_max) {
   long long m = 0;
   for (int n = 2; n * n <= nn_max; n += 2) m = mg_slow_elems(n) > m ? mg_slow_elems(n) : m;
   return m;
@@ -111,24 +140,32 @@ struct Smem2D {
   vec2_t<TA>* p;     // [2][NN] PCG exchange vector (u = M^-1 r), two alternating buffers
   vec2_t<TA>* x;     // [NN] PCG solution (owned nodes written by their thread)
   unsigned char* stage;  // element forces / element tangents / condensation solutions
-  double* red;       // 2 x 512 doubles of reduction buffers
+  double* red;       // reduction buffers: two of red_n doubles, then the PCG's dot buffer (34)
+  int red_n;
   double* lame;      // [kMaxPhase][2]
   double* misc;      // [16]: Fbar (0..3), homogenised P and W (4..8)
 };
 
+// Byte offsets of the arrays in the block's shared memory (constants where the grid is one).
+struct Offsets2D {
+  size_t w, w32, p, x, stage, red, lame, misc, total;
+  int red_n;
+};
+
 template <typename TA>
-__host__ __device__ inline size_t smem2d_layout(int NN, Smem2D<TA>* s, unsigned char* base) {
+__host__ __device__ constexpr Offsets2D offsets2d(int NN) {
   constexpr bool REG = std::is_same<TA, float>::value;
+  Offsets2D o{};
   size_t off = 0;
-  auto take = [&](size_t bytes) {
-    size_t o = off;
+  const auto take = [&off](size_t bytes) {
+    const size_t at = off;
     off += (bytes + 15) & ~size_t(15);
-    return o;
+    return at;
   };
-  size_t o_w = take(sizeof(double2) * NN);
-  size_t o_w32 = REG ? take(sizeof(float2) * NN) : 0;
-  size_t o_p = take(2 * sizeof(vec2_t<TA>) * NN);
-  size_t o_x = take(sizeof(vec2_t<TA>) * NN);
+  o.w = take(sizeof(double2) * NN);
+  o.w32 = REG ? take(sizeof(float2) * NN) : 0;
+  o.p = take(2 * sizeof(vec2_t<TA>) * NN);
+  o.x = take(sizeof(vec2_t<TA>) * NN);
   size_t stage_bytes = sizeof(double) * 8 * NN;                               // element forces
   // condensation solutions X[4][NN] and right-hand sides L[4][NN]; in mixed mode followed by
   // the multigrid fast region of the RVE's grid (largest over the grids up to NN)
@@ -138,21 +175,28 @@ __host__ __device__ inline size_t smem2d_layout(int NN, Smem2D<TA>* s, unsigned 
       const size_t need = sizeof(vec2_t<TA>) * 8 * (size_t)m * m + sizeof(TA) * (size_t)mg_fast_elems(m);
       if (need > stage_bytes) stage_bytes = need;
     }
-  size_t o_stage = take(stage_bytes);
-  size_t o_red = take(sizeof(double) * 2 * 512);
-  size_t o_lame = take(sizeof(double) * 2 * kMaxPhase);
-  size_t o_misc = take(sizeof(double) * 16);
-  if (s) {
-    s->w = reinterpret_cast<double2*>(base + o_w);
-    s->w32 = REG ? reinterpret_cast<float2*>(base + o_w32) : nullptr;
-    s->p = reinterpret_cast<vec2_t<TA>*>(base + o_p);
-    s->x = reinterpret_cast<vec2_t<TA>*>(base + o_x);
-    s->stage = base + o_stage;
-    s->red = reinterpret_cast<double*>(base + o_red);
-    s->lame = reinterpret_cast<double*>(base + o_lame);
-    s->misc = reinterpret_cast<double*>(base + o_misc);
-  }
-  return off;
+  o.stage = take(stage_bytes);
+  o.red_n = 10 * (threads2d<TA>(NN) / 32);  // block_sum of up to 10 values
+  o.red = take(sizeof(double) * (2 * o.red_n + 34));
+  o.lame = take(sizeof(double) * 2 * kMaxPhase);
+  o.misc = take(sizeof(double) * 16);
+  o.total = off;
+  return o;
+}
+
+template <typename TA>
+__device__ __forceinline__ Smem2D<TA> smem2d(const Offsets2D& o, unsigned char* base) {
+  Smem2D<TA> s;
+  s.w = reinterpret_cast<double2*>(base + o.w);
+  s.w32 = std::is_same<TA, float>::value ? reinterpret_cast<float2*>(base + o.w32) : nullptr;
+  s.p = reinterpret_cast<vec2_t<TA>*>(base + o.p);
+  s.x = reinterpret_cast<vec2_t<TA>*>(base + o.x);
+  s.stage = base + o.stage;
+  s.red = reinterpret_cast<double*>(base + o.red);
+  s.red_n = o.red_n;
+  s.lame = reinterpret_cast<double*>(base + o.lame);
+  s.misc = reinterpret_cast<double*>(base + o.misc);
+  return s;
 }
 
 // Per-thread geometry of the owned node pair.
@@ -270,7 +314,7 @@ __device__ __forceinline__ void element_residual(int e, int n, const double2* w,
                                                  double& bad) {
   const int i = e % n, j = e / n, ip = (i + 1) % n, jp = (j + 1) % n;
   const double2 w0 = w[e], w1 = w[ip + n * j], w2 = w[ip + n * jp], w3 = w[i + n * jp];
-  const double ih = (double)n;
+  const double ih = unfolded((double)n);
   const double2 d10 = make_double2(w1.x - w0.x, w1.y - w0.y);
   const double2 d30 = make_double2(w3.x - w0.x, w3.y - w0.y);
   const double2 e1 = make_double2((w2.x - w3.x) - d10.x, (w2.y - w3.y) - d10.y);
@@ -341,7 +385,7 @@ __device__ __forceinline__ double element_energy(int e, int n, const double2* w,
                                                  double mu) {
   const int i = e % n, j = e / n, ip = (i + 1) % n, jp = (j + 1) % n;
   const double2 w0 = w[e], w1 = w[ip + n * j], w2 = w[ip + n * jp], w3 = w[i + n * jp];
-  const double ih = (double)n;
+  const double ih = unfolded((double)n);
   double acc = 0.0;
 #pragma unroll
   for (int gy = 0; gy < 2; ++gy) {
@@ -378,7 +422,7 @@ __device__ __forceinline__ void element_tangent(int e, int n, const vec2_t<TA>* 
                                                 TA* stage_k, int slot, int NN) {
   const int i = e % n, j = e / n, ip = (i + 1) % n, jp = (j + 1) % n;
   const vec2_t<TA> w0 = w[e], w1 = w[ip + n * j], w2 = w[ip + n * jp], w3 = w[i + n * jp];
-  const TA ih = (TA)n;
+  const TA ih = unfolded((TA)n);
   const TA d10x = w1.x - w0.x, d10y = w1.y - w0.y, d30x = w3.x - w0.x, d30y = w3.y - w0.y;
   const TA e1x = (w2.x - w3.x) - d10x, e1y = (w2.y - w3.y) - d10y;
   const TA e2x = (w2.x - w1.x) - d30x, e2y = (w2.y - w1.y) - d30y;
@@ -606,10 +650,15 @@ __device__ __forceinline__ void invert_block(const TA (&Kself)[4], bool pinned, 
 //    in the fast region (shared memory in mixed mode, block scratch in FP64 mode); coarse
 //    element matrices (needed only while building) in the block's global scratch.
 template <typename TA>
+struct alignas(16) Block2 {
+  TA xx, xy, yx, yy;
+};
+
+template <typename TA>
 struct MgLevel {
   int n, NN, bc;
-  TA* st;          // [36][NN]
-  TA* mi;          // [4][NN]
+  Block2<TA>* st;  // [9][NN]
+  Block2<TA>* mi;  // [NN]
   vec2_t<TA>* r;   // [NN]
   vec2_t<TA>* z;   // [NN]
   vec2_t<TA>* t;   // [NN]
@@ -641,13 +690,14 @@ struct MgCtx {
     v.bc = bc;
     v.ke = k;
     if (l < levels) {
-      v.st = f;
-      v.mi = f + 36 * v.NN;
+      v.st = reinterpret_cast<Block2<TA>*>(f);
+      v.mi = v.st + 9 * v.NN;
       v.r = reinterpret_cast<vec2_t<TA>*>(f + 40 * v.NN);
       v.z = v.r + v.NN;
       v.t = v.z + v.NN;
     } else {
-      v.st = v.mi = nullptr;
+      v.st = nullptr;
+      v.mi = nullptr;
       v.r = reinterpret_cast<vec2_t<TA>*>(f);
       v.z = v.r + v.NN;
       v.t = nullptr;
@@ -727,16 +777,16 @@ __device__ __forceinline__ vec2_t<TA> mg_apply(const MgLevel<TA>& L, const vec2_
 #pragma unroll
   for (int nb = 0; nb < 9; ++nb) {
     const vec2_t<TA> zn = z[rows[nb / 3] + cols[nb % 3]];
-    yx += L.st[(size_t)(nb * 4 + 0) * L.NN + v] * zn.x + L.st[(size_t)(nb * 4 + 1) * L.NN + v] * zn.y;
-    yy += L.st[(size_t)(nb * 4 + 2) * L.NN + v] * zn.x + L.st[(size_t)(nb * 4 + 3) * L.NN + v] * zn.y;
+    const Block2<TA> k = L.st[nb * L.NN + v];
+    yx += k.xx * zn.x + k.xy * zn.y;
+    yy += k.yx * zn.x + k.yy * zn.y;
   }
   return pinned2(i, j, L.bc) ? mk2<TA>(TA(0), TA(0)) : mk2<TA>(yx, yy);
 }
 
 template <typename TA>
-__device__ __forceinline__ vec2_t<TA> mg_smooth(const TA* mi, int NN, int v, vec2_t<TA> r, TA omega) {
-  const TA m0 = mi[v], m1 = mi[NN + v], m2 = mi[2 * NN + v], m3 = mi[3 * NN + v];
-  return mk2<TA>(omega * (m0 * r.x + m1 * r.y), omega * (m2 * r.x + m3 * r.y));
+__device__ __forceinline__ vec2_t<TA> mg_smooth(const Block2<TA>& m, vec2_t<TA> r, TA omega) {
+  return mk2<TA>(omega * (m.xx * r.x + m.xy * r.y), omega * (m.yx * r.x + m.yy * r.y));
 }
 
 // Full-weighting restriction (the transpose of bilinear prolongation) of the fine vector t
@@ -824,13 +874,11 @@ __device__ __forceinline__ void mg_build_part2(const MgCtx<TA>& mg) {
       for (int nb = 0; nb < 9; ++nb) {
         TA blk[4];
         mg_stencil_block<TA>(v.ke, v.n, i, j, nb, blk);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) v.st[(size_t)(nb * 4 + q) * v.NN + node] = blk[q];
+        v.st[nb * v.NN + node] = {blk[0], blk[1], blk[2], blk[3]};
         if (nb == 4) {
           TA m[4];
           invert_block<TA>(blk, pinned2(i, j, v.bc), m);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) v.mi[(size_t)q * v.NN + node] = m[q];
+          v.mi[node] = {m[0], m[1], m[2], m[3]};
         }
       }
     }
@@ -864,22 +912,22 @@ __device__ __forceinline__ void mg_build_part2(const MgCtx<TA>& mg) {
     }
   }
   __syncthreads();
-  // entries (i, j) of this thread: e and e + blockDim.x (D*D <= 1024 = 2 x 512)
-  const int e0 = tid, e1 = tid + blockDim.x;
-  const int i0 = e0 / D, j0 = e0 % D, i1 = e1 / D, j1 = e1 % D;
+  // one column per lane (D <= 32), the rows dealt to the warps
+  const int j = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   for (int k = 0; k < D; ++k) {  // SPD: no pivoting; D is even, so the result ends in A
     const TA* Ao = (k & 1) ? B : A;
     TA* An = (k & 1) ? A : B;
     const TA ip = TA(1) / Ao[(size_t)k * ld + k];
-    auto step = [&](int i, int j) {
-      const TA aik = Ao[(size_t)i * ld + k], akj = Ao[(size_t)k * ld + j];
-      TA v;
-      if (i == k) v = (j == k) ? ip : akj * ip;
-      else v = (j == k) ? -aik * ip : Ao[(size_t)i * ld + j] - aik * akj * ip;
-      An[(size_t)i * ld + j] = v;
-    };
-    if (e0 < D * D) step(i0, j0);
-    if (e1 < D * D) step(i1, j1);
+    if (j < D) {
+      const TA akj = Ao[(size_t)k * ld + j];
+      for (int i = warp; i < D; i += nw) {
+        const TA aik = Ao[(size_t)i * ld + k];
+        TA v;
+        if (i == k) v = (j == k) ? ip : akj * ip;
+        else v = (j == k) ? -aik * ip : Ao[(size_t)i * ld + j] - aik * akj * ip;
+        An[(size_t)i * ld + j] = v;
+      }
+    }
     __syncthreads();
   }
 }
@@ -892,7 +940,7 @@ __device__ __forceinline__ void mg_restrict_smooth(const MgCtx<TA>& mg, int l, c
   const MgLevel<TA> c = mg.level(l);
   const vec2_t<TA> r = mg_restrict<TA>(tf, nf, t % c.n, t / c.n, mg.bc);
   c.r[t] = r;
-  if (l < mg.levels) c.z[t] = mg_smooth<TA>(c.mi, c.NN, t, r, mg.omega);
+  if (l < mg.levels) c.z[t] = mg_smooth<TA>(c.mi[t], r, mg.omega);
 }
 
 // Where the corrected z of level l ends: the t vector of a smoothing level (free on the way
@@ -909,9 +957,10 @@ __device__ __forceinline__ const vec2_t<TA>* mg_result(const MgCtx<TA>& mg, int 
 // (Running the small levels in one warp with warp barriers was measured slower: the other warps
 // idle while one warp walks the level's nodes serially.)
 template <typename TA>
-__device__ void mg_coarse_cycle(const MgCtx<TA>& mg) {
+__device__ __forceinline__ void mg_coarse_cycle(const MgCtx<TA>& mg) {
   const int tid = threadIdx.x;
   const TA om = mg.omega;
+#pragma unroll
   for (int l = 1; l < mg.levels; ++l) {  // descend: residual, restrict (+ next pre-smoothing)
     const MgLevel<TA> v = mg.level(l);
     if (tid < v.NN) {
@@ -924,18 +973,22 @@ __device__ void mg_coarse_cycle(const MgCtx<TA>& mg) {
   }
   {  // coarsest: z = A^-1 r, 16 lanes per row (rows 0, 1 of the inverse: the pinned identity)
     const MgLevel<TA> c = mg.level(mg.levels);
-    const int D = 2 * c.NN, ld = D + 1, row = tid >> 4, l16 = tid & 15;
+    const int D = 2 * c.NN, ld = D + 1, l16 = tid & 15;
     const TA* A = mg.coarsest_inverse();
     const TA* r = reinterpret_cast<const TA*>(c.r);
-    TA zz = TA(0);
-    if (row < D)
-      for (int q = l16; q < D; q += 16) zz += A[(size_t)row * ld + q] * r[q];
+    for (int row0 = 0; row0 < D; row0 += blockDim.x >> 4) {  // whole warps stay in the loop
+      const int row = row0 + (tid >> 4);
+      TA zz = TA(0);
+      if (row < D)
+        for (int q = l16; q < D; q += 16) zz += A[(size_t)row * ld + q] * r[q];
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) zz += __shfl_xor_sync(0xffffffffu, zz, o);
-    if (row < D && l16 == 0)
-      reinterpret_cast<TA*>(c.z)[row] = pinned2((row >> 1) % c.n, (row >> 1) / c.n, c.bc) ? TA(0) : zz;
+      for (int o = 8; o > 0; o >>= 1) zz += __shfl_xor_sync(0xffffffffu, zz, o);
+      if (row < D && l16 == 0)
+        reinterpret_cast<TA*>(c.z)[row] = pinned2((row >> 1) % c.n, (row >> 1) / c.n, c.bc) ? TA(0) : zz;
+    }
     __syncthreads();
   }
+#pragma unroll
   for (int l = mg.levels - 1; l >= 1; --l) {  // ascend: prolong, post-smooth into t
     const MgLevel<TA> v = mg.level(l);
     const vec2_t<TA>* zc = mg_result<TA>(mg, l + 1);
@@ -947,7 +1000,7 @@ __device__ void mg_coarse_cycle(const MgCtx<TA>& mg) {
     __syncthreads();
     if (tid < v.NN) {
       const vec2_t<TA> kz = mg_apply<TA>(v, v.z, i, j), rr = v.r[tid], z = v.z[tid];
-      const vec2_t<TA> dz = mg_smooth<TA>(v.mi, v.NN, tid, mk2<TA>(rr.x - kz.x, rr.y - kz.y), om);
+      const vec2_t<TA> dz = mg_smooth<TA>(v.mi[tid], mk2<TA>(rr.x - kz.x, rr.y - kz.y), om);
       v.t[tid] = mk2<TA>(z.x + dz.x, z.y + dz.y);
     }
     __syncthreads();
@@ -1255,7 +1308,7 @@ __device__ __forceinline__ void element_transfer(int e, int n, const vec2_t<TA>*
   const int NN = n * n;
   const int i = e % n, j = e / n, ip = (i + 1) % n, jp = (j + 1) % n;
   const int nd[4] = {e, ip + n * j, ip + n * jp, i + n * jp};
-  const TA ih = (TA)n;
+  const TA ih = unfolded((TA)n);
   const vec2_t<TA> w0 = wsrc[nd[0]], w1 = wsrc[nd[1]], w2 = wsrc[nd[2]], w3 = wsrc[nd[3]];
   vec2_t<TA> x[4][4];  // [rhs][local node]
 #pragma unroll
@@ -1340,13 +1393,15 @@ __device__ __forceinline__ void element_transfer(int e, int n, const vec2_t<TA>*
 
 // kFixed: one grid size for the whole batch, arrays indexed arithmetically (qp -> RVE qp or 0,
 // fluctuation of qp at qp*2*n*n) instead of through the context's index tables.
-template <typename TA, bool kFixed, bool kMG, int LAW>
-__device__ void solve_item_2d(const Rve2dArgs& a, int qp, const Smem2D<TA>& sm, TA* gscr) {
+// N: the grid size of every item where it is known when compiling (0: read per item).
+template <typename TA, bool kFixed, bool kMG, int LAW, int N>
+__device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const Smem2D<TA>& sm, TA* gscr) {
   constexpr bool REG = std::is_same<TA, float>::value;
   const int tid = threadIdx.x;
   const int rv = kFixed ? (a.phase_per_qp ? qp : 0) : a.qp_rve[qp];
-  const int n = kFixed ? a.fixed_n : a.rve_n[rv];
+  const int n = N ? N : kFixed ? a.fixed_n : a.rve_n[rv];
   const int NN = n * n;
+  const int nn_max = N ? N * N : a.nn_max;
   const Own2D o = make_own(n, a.bc);
   const uint8_t* phase = a.phase + (kFixed ? (size_t)rv * n * n : (size_t)a.rve_phase_off[rv]);
   const size_t w_off = kFixed ? (size_t)qp * 2 * n * n : (size_t)a.qp_w_off[qp];
@@ -1386,17 +1441,22 @@ __device__ void solve_item_2d(const Rve2dArgs& a, int qp, const Smem2D<TA>& sm, 
   // block scratch
   MgCtx<TA> mg;
   mg.n = n;
-  mg.levels = (kMG && a.mg) ? mg_levels(n) : 0;
+  if constexpr (N > 0) {
+    constexpr int kLevels = kMG ? mg_levels(N) : 0;
+    mg.levels = kLevels;
+  } else {
+    mg.levels = kMG ? mg_levels(n) : 0;
+  }
   mg.bc = a.bc;
   mg.omega = (TA)a.mg_omega;
   if constexpr (REG) {
     mg.fast = reinterpret_cast<TA*>(sm.stage + 8 * (size_t)NN * sizeof(vec2_t<TA>));
-    mg.slow = reinterpret_cast<TA*>(a.scratch) + (size_t)blockIdx.x * a.scratch_stride + (size_t)36 * a.nn_max;
+    mg.slow = reinterpret_cast<TA*>(a.scratch) + (size_t)blockIdx.x * a.scratch_stride + (size_t)36 * nn_max;
   } else {
-    mg.fast = gscr + (size_t)72 * a.nn_max;
-    mg.slow = mg.fast + mg_fast_max(a.nn_max);
+    mg.fast = gscr + (size_t)72 * nn_max;
+    mg.slow = mg.fast + mg_fast_max(nn_max);
   }
-  double* redD = sm.red + 2 * 512 - 64;  // the PCG's FP64 dot buffer (34 doubles) at the end of red
+  double* redD = sm.red + 2 * sm.red_n;  // the PCG's FP64 dot buffer
   vec2_t<TA>* Xs = reinterpret_cast<vec2_t<TA>*>(sm.stage);  // [4][NN]
   vec2_t<TA>* Lb = Xs + 4 * NN;                               // [4][NN]
   TA Minv[2][4];
@@ -1447,7 +1507,7 @@ __device__ void solve_item_2d(const Rve2dArgs& a, int qp, const Smem2D<TA>& sm, 
         if (o.pin[1]) R[2] = R[3] = 0.0;
       }
       double v2[2] = {R[0] * R[0] + R[1] * R[1] + R[2] * R[2] + R[3] * R[3], bad};
-      block_sum<2, double>(v2, sm.red + (it & 1) * 512);
+      block_sum<2, double>(v2, sm.red + (it & 1) * sm.red_n);
       const double rn = sqrt(v2[0]);
       if (it == 0) r0 = rn;
       if ((v2[1] > 0.0 || !isfinite(rn)) && it > 0 && nhalf < kMaxStepHalvings) {
@@ -1583,7 +1643,7 @@ __device__ void solve_item_2d(const Rve2dArgs& a, int qp, const Smem2D<TA>& sm, 
     }
   }
   // the last residual norm used buffer (it & 1) and may still be read: use the other one
-  block_sum<5, double>(Pv, sm.red + ((it + 1) & 1) * 512);
+  block_sum<5, double>(Pv, sm.red + ((it + 1) & 1) * sm.red_n);
   if (tid == 0) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) sm.misc[4 + k] = Pv[k];
@@ -1669,7 +1729,7 @@ __device__ void solve_item_2d(const Rve2dArgs& a, int qp, const Smem2D<TA>& sm, 
         element_transfer<TA, LAW>(e, n, wsrc, X, Fb, (TA)sm.lame[2 * ph], (TA)sm.lame[2 * ph + 1], Q);
       }
     }
-    block_sum<10, double>(Q, sm.red + (it & 1) * 512);
+    block_sum<10, double>(Q, sm.red + (it & 1) * sm.red_n);
   }
 
   // ---- outputs
@@ -1709,11 +1769,17 @@ __device__ void solve_item_2d(const Rve2dArgs& a, int qp, const Smem2D<TA>& sm, 
   __syncthreads();
 }
 
-template <typename TA, bool kFixed, bool kMG, int LAW>
-__global__ void __launch_bounds__(kThreads2D, 1) rve2d_kernel(const Rve2dArgs a) {
+template <typename TA, bool kFixed, bool kMG, int LAW, int N>
+__global__ void __launch_bounds__(N ? threads2d<TA>(N * N) : kThreads2D, N ? 512 / threads2d<TA>(N * N) : 1)
+rve2d_kernel(const Rve2dArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Smem2D<TA> sm;
-  smem2d_layout<TA>(a.nn_max, &sm, smem_raw);
+  if constexpr (N > 0) {
+    constexpr Offsets2D off = offsets2d<TA>(N * N);
+    sm = smem2d<TA>(off, smem_raw);
+  } else {
+    sm = smem2d<TA>(offsets2d<TA>(a.nn_max), smem_raw);
+  }
   __shared__ int s_item;
   constexpr bool REG = std::is_same<TA, float>::value;
   TA* gscr = REG ? nullptr : reinterpret_cast<TA*>(a.scratch) + (size_t)blockIdx.x * a.scratch_stride;
@@ -1723,19 +1789,21 @@ __global__ void __launch_bounds__(kThreads2D, 1) rve2d_kernel(const Rve2dArgs a)
     const int item = s_item;
     __syncthreads();
     if (item >= (a.n_dev ? *a.n_dev : a.n_qp)) break;
-    solve_item_2d<TA, kFixed, kMG, LAW>(a, kFixed ? item : a.order[item], sm, gscr);
+    const int qp = kFixed ? item : a.order[item];
+    if (!kFixed && a.only_n && a.rve_n[a.qp_rve[qp]] != a.only_n) continue;  // another launch's grid
+    solve_item_2d<TA, kFixed, kMG, LAW, N>(a, qp, sm, gscr);
   }
 }
 
 }  // namespace
 
 // Launch of one instantiation (grid of n_blocks persistent blocks, smem dynamic shared bytes).
-template <typename TA, bool kFixed, bool kMG, int LAW>
+template <typename TA, bool kFixed, bool kMG, int LAW, int N = 0>
 inline cudaError_t rve2d_launch_instance(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream) {
-  const cudaError_t err = cudaFuncSetAttribute(rve2d_kernel<TA, kFixed, kMG, LAW>,
+  const cudaError_t err = cudaFuncSetAttribute(rve2d_kernel<TA, kFixed, kMG, LAW, N>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  rve2d_kernel<TA, kFixed, kMG, LAW><<<n_blocks, kThreads2D, smem, stream>>>(a);
+  rve2d_kernel<TA, kFixed, kMG, LAW, N><<<n_blocks, threads2d<TA>(a.nn_max), smem, stream>>>(a);
   return cudaGetLastError();
 }
 
