@@ -283,7 +283,7 @@ int fehmm_macro_update(fehmm_ctx* ctx, double* u, const double* du, void* stream
  *   K_vals device [nnz] (CSR order of fehmm_macro_csr), f device [n_rows], du device
  *   [n_rows] (output), info device double[3] (output): |f_free|_2 (the macro convergence
  *   measure, taken before the solve), CG iterations, status (0 converged, 1 cap,
- *   2 non-positive curvature).
+ *   2 non-positive curvature, 3 a thread block gave up waiting for another: du is not valid).
  */
 int fehmm_macro_solve(fehmm_ctx* ctx, const double* K_vals, const double* f, double* du, double* info,
                       double rtol, int max_it, void* stream);

@@ -59,6 +59,7 @@ struct fehmm_ctx {
   int32_t* d_rowptr = nullptr;
   int32_t* d_col = nullptr;
   int32_t* d_blk_base = nullptr;
+  double* d_grad = nullptr;
   int32_t* d_blk_stride = nullptr;
   int macro_rows = 0, macro_nnz = 0;
   uint8_t* d_fixed = nullptr;   // Dirichlet mask of the macro dofs
@@ -67,6 +68,11 @@ struct fehmm_ctx {
   double* d_dir_full = nullptr;  // [macro_rows]: the Dirichlet end values on their dofs, 0 elsewhere
   int n_fixed = 0;
   double* d_solve_work = nullptr;
+  MacroResident resident;  // the macro solve with rows in registers (lanes 0: mesh too large for it)
+  int32_t* d_halo_ptr = nullptr;
+  int32_t* d_halo = nullptr;
+  uint16_t* d_lcol = nullptr;
+  void* d_pub = nullptr;
   long long launches = 0;
 };
 
@@ -172,12 +178,17 @@ int fehmm_destroy(fehmm_ctx* c) {
   dfree(c->d_rowptr);
   dfree(c->d_col);
   dfree(c->d_blk_base);
+  dfree(c->d_grad);
   dfree(c->d_blk_stride);
   dfree(c->d_fixed);
   dfree(c->d_fixed_dofs);
   dfree(c->d_fixed_vals);
   dfree(c->d_dir_full);
   dfree(c->d_solve_work);
+  dfree(c->d_halo_ptr);
+  dfree(c->d_halo);
+  dfree(c->d_lcol);
+  if (c->d_pub) cudaFree(c->d_pub);
   delete c;
   return FEHMM_OK;
 }
@@ -584,6 +595,17 @@ int fehmm_macro_create(fehmm_ctx* c, const int32_t* n_el) {
       (rc = dupload(c->d_blk_base, blk_base.data(), blk_base.size())) ||
       (rc = dupload(c->d_blk_stride, blk_stride.data(), blk_stride.size())))
     return rc;
+  dfree(c->d_grad);
+  if (cudaMalloc((void**)&c->d_grad, sizeof(double) * m.nen * m.nq * d) != cudaSuccess) {
+    cudaGetLastError();
+    c->d_grad = nullptr;
+    return FEHMM_ERR_OOM;
+  }
+  if (macro_grad_launch(m, c->d_grad) != cudaSuccess || cudaStreamSynchronize(0) != cudaSuccess) {
+    cudaGetLastError();
+    return FEHMM_ERR_CUDA;
+  }
+  m.grad = c->d_grad;
   m.blk_base = c->d_blk_base;
   m.blk_stride = c->d_blk_stride;
   std::vector<uint8_t> nofix((size_t)nn * d, 0);
@@ -594,6 +616,23 @@ int fehmm_macro_create(fehmm_ctx* c, const int32_t* n_el) {
     cudaGetLastError();
     c->d_solve_work = nullptr;
     return FEHMM_ERR_OOM;
+  }
+  c->resident = MacroResident{};
+  if (c->d_pub) cudaFree(c->d_pub);
+  c->d_pub = nullptr;
+  MacroResident resident = macro_resident_plan(d, nn * d, c->num_sms);
+  std::vector<int32_t> halo_ptr, halo;
+  std::vector<uint16_t> lcol;
+  if (resident.lanes && macro_resident_columns(resident, d, nn * d, rowptr, col, halo_ptr, halo, lcol)) {
+    if ((rc = dupload(c->d_halo_ptr, halo_ptr.data(), halo_ptr.size())) ||
+        (rc = dupload(c->d_halo, halo.data(), halo.size())) || (rc = dupload(c->d_lcol, lcol.data(), lcol.size())))
+      return rc;
+    if (cudaMalloc(&c->d_pub, 16 * ((size_t)nn * d + 4 * resident.blocks)) != cudaSuccess) {
+      cudaGetLastError();
+      c->d_pub = nullptr;
+      return FEHMM_ERR_OOM;
+    }
+    c->resident = resident;
   }
   c->macro = m;
   c->macro_rows = nn * d;
@@ -701,7 +740,13 @@ int fehmm_macro_solve(fehmm_ctx* c, const double* K_vals, const double* f, doubl
   a.out = info;
   a.rtol = rtol;
   a.max_it = max_it;
-  if (macro_solve_launch(a, macro_solve_blocks(c->num_sms, c->macro_rows), (cudaStream_t)stream) != cudaSuccess) {
+  a.halo_ptr = c->d_halo_ptr;
+  a.halo = c->d_halo;
+  a.lcol = c->d_lcol;
+  a.pub = c->d_pub;
+  if ((c->resident.lanes
+           ? macro_solve_resident_launch(a, c->opt.dim, c->resident, (cudaStream_t)stream)
+           : macro_solve_launch(a, macro_solve_blocks(c->num_sms, c->macro_rows), (cudaStream_t)stream)) != cudaSuccess) {
     cudaGetLastError();
     return FEHMM_ERR_CUDA;
   }

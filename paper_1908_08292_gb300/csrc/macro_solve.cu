@@ -3,16 +3,29 @@
 // Eq. Assem_k_T_IK_mac).  Jacobi-preconditioned CG in FP64 over the CSR tangent.
 //
 // One cooperative launch, one block per SM at most, all co-resident.  The CG is the single-
-// reduction form of Chronopoulos and Gear: per iteration the vector updates and u = M^-1 r (one
-// thread per row), a grid barrier (u visible), the sparse product w = K u (8 lanes per row,
-// strided nonzeros per lane, shuffle sum) together with the partial inner products
-// gamma = r.u and delta = w.u, and a second grid barrier after which every block adds the block
-// partials in the same order — two grid barriers per iteration and identical decisions in
-// every block.  Fixed rows carry M^-1 = 0 and no product, which keeps their r, u, p, x at zero.
-// The first output is |f_free|_2, the macro convergence measure.
+// reduction form of Chronopoulos and Gear: per iteration the vector updates and u = M^-1 r, the
+// exchange of u, the sparse product w = K u together with the partial inner products gamma = r.u and
+// delta = w.u, and their sum over the blocks, added in the same order by every block: identical
+// decisions in every block.  Fixed rows carry M^-1 = 0 and no product, which keeps their r, u, p, x
+// at zero.  The first output is |f_free|_2, the macro convergence measure.
+//
+// Two kernels.  macro_pcg_resident_kernel (meshes whose rows fit the registers of one block per SM, up to
+// 128 rows a block) holds its rows of K and of every vector in registers for the whole solve; blocks
+// exchange only u at the block boundaries and the partial sums, both as 16-byte {value, sequence number}
+// words that the reader polls, so an exchange is one store and one load through the L2.  An iteration was
+// bound by its two grid barriers and by reading K again after each (9 us at 2178 rows); now by those two
+// hops (about 0.6 us each) and by the FP64 pipe (64 cycles per warp instruction on an SM sub-partition),
+// which the split of the rows over all SMs, the order of the updates (p and x beside the exchange) and
+// one lane per inner product keep short.  Per iteration on a GB300: 50 rows 9.0 -> 2.3 us, 2178 rows (2D)
+// 9.6 -> 3.5, 9894 rows (2D) 11.3 -> 3.9, 14739 rows (3D) 15.4 -> 8.0.  macro_pcg_kernel: any larger mesh,
+// vectors in global memory, two grid barriers per iteration.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdint.h>
+
+#include <algorithm>
+#include <vector>
 
 #include "rve_args.h"
 
@@ -23,7 +36,6 @@ namespace {
 
 constexpr int kSolveThreads = 256;
 constexpr int kRowLanes = 8;                              // lanes per matrix row in the product
-constexpr int kRowsPerWarp = 32 / kRowLanes;              // 4
 constexpr int kRowsPerBlock = kSolveThreads / kRowLanes;  // 32
 
 // Sum (a, b) over the grid: block sums -> partial[2*block], grid barrier, every block adds the
@@ -189,6 +201,223 @@ __global__ void __launch_bounds__(kSolveThreads) macro_pcg_kernel(const MacroSol
   }
 }
 
+// ------------------------------------------------------------------ rows resident in registers
+constexpr int kResMaxThreads = 256, kResMaxRows = 128;
+constexpr long long kSpinCycles = 1ll << 32;  // about 2 s: a block that never arrives
+
+// {value, sequence number} as one 16-byte word: a reader sees both or neither
+__device__ __forceinline__ void put(ulonglong2* p, double v, unsigned long long seq) {
+  asm volatile("{\n\t.reg .b128 q;\n\tmov.b128 q, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], q;\n\t}" ::"l"(p),
+               "l"(__double_as_longlong(v)), "l"(seq)
+               : "memory");
+}
+
+// Calls take(e, value) for e = t, t + blockDim.x, ... < count with the words at word(e) once they carry seq; four
+// loads are in flight at a time (one after the other their latencies add up).  False if a word never comes.
+template <typename Word, typename Take>
+__device__ __forceinline__ bool get_all(int count, unsigned long long seq, Word word, Take take) {
+  constexpr int M = 4;
+  bool ok = true;
+  for (int e0 = threadIdx.x; e0 < count; e0 += M * blockDim.x) {
+    unsigned long long b[M], s[M];
+    const long long t0 = clock64();
+    for (;;) {
+      bool all = true;
+#pragma unroll
+      for (int j = 0; j < M; ++j) {
+        const int e = e0 + j * blockDim.x;
+        s[j] = seq;
+        if (e < count)
+          asm volatile("{\n\t.reg .b128 q;\n\tld.relaxed.gpu.global.b128 q, [%2];\n\tmov.b128 {%0, %1}, q;\n\t}"
+                       : "=l"(b[j]), "=l"(s[j])
+                       : "l"(word(e))
+                       : "memory");
+      }
+#pragma unroll
+      for (int j = 0; j < M; ++j) all = all && s[j] == seq;
+      if (all) break;
+      if (clock64() - t0 > kSpinCycles) {
+        ok = false;
+        break;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+      if (e0 + j * blockDim.x < count) take(e0 + j * blockDim.x, __longlong_as_double((long long)b[j]));
+  }
+  return ok;
+}
+
+// 1 / x for positive normal x: the FP32 reciprocal of the mantissa refined by two Newton steps in FP64 (within an
+// ulp or so; a division takes about four times the FP64 instructions, and the iteration waits for this one).
+__device__ __forceinline__ double recip(double x) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (e == 0 || e > 2040 || hi < 0) return 1.0 / x;
+  const double m = __hiloint2double((hi & 0xfffff) | (1023 << 20), __double2loint(x));
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)m));
+  double q = (double)r;
+  q = fma(q, fma(-m, q, 1.0), q);
+  q = fma(q, fma(-m, q, 1.0), q);
+  return __hiloint2double(__double2hiint(q) + ((1023 - e) << 20), __double2loint(q));
+}
+
+// L lanes per row, at most PER nonzeros per lane.
+template <int L, int PER>
+__global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(const MacroSolveArgs a) {
+  cg::grid_group grid = cg::this_grid();
+  extern __shared__ __align__(16) double us[];  // u of this block's rows, then of the rows around them
+  __shared__ double part[2][32], total[4];      // total: alpha, beta, first sum, second sum
+  __shared__ int action;                        // 0: go on, 1: converged, 2: cap, 3: breakdown, 4: gave up
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5, nb = gridDim.x;
+  const int R = blockDim.x / L, lr = t / L, ll = t % L;
+  const int r0 = blockIdx.x * R, i = r0 + lr;
+  const bool mine = i < a.n;
+  const int h0 = a.halo_ptr[blockIdx.x], nh = a.halo_ptr[blockIdx.x + 1] - h0;
+  ulonglong2* pub = reinterpret_cast<ulonglong2*>(a.pub);
+  // Partial sums, two alternating buffers of 2 per block: a block may publish its next sums while a slower one
+  // still reads these, but the ones after that only when every block has read these (it needs their next).
+  // u needs one buffer: a block publishes its next u after sums that every reader of this u contributed to.
+  ulonglong2* slots = pub + a.n;  // [2][2 * nb]
+  // this lane's nonzeros, the row's diagonal and right-hand side
+  const bool fixed = !mine || a.fixed[i] != 0;
+  constexpr int PL = (PER + 1) / 2;
+  double k[PER], d = 0.0;
+  uint32_t lc[PL];  // two 16-bit places each
+  {
+    const int k0 = mine ? a.rowptr[i] : 0, k1 = mine ? a.rowptr[i + 1] : 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int e = k0 + ll + j * L;
+      const bool in = e < k1;
+      const uint32_t c = in ? a.lcol[e] : 0u;
+      k[j] = in ? a.K[e] : 0.0;
+      lc[j / 2] = (j & 1) ? lc[j / 2] | (c << 16) : c;
+      if (in && (int)c == lr) d = k[j];
+      if (fixed) k[j] = 0.0;
+    }
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+  }
+  const double di = fixed ? 0.0 : 1.0 / (d != 0.0 ? d : 1.0);
+  double r = fixed ? 0.0 : -a.f[i], u = r * di, x = 0.0, p = 0.0, s = 0.0, w = 0.0;
+  if (mine && ll == 0) pub[i] = make_ulonglong2(0ull, 0ull);
+  if (t < 4) slots[(t >> 1) * 2 * nb + 2 * blockIdx.x + (t & 1)] = make_ulonglong2(0ull, 0ull);
+  if (t == 0) action = 0;
+  grid.sync();  // every word carries sequence number 0
+  unsigned long long useq = 0, sseq = 0;
+  bool lost = false;
+
+  auto publish = [&]() {
+    ++useq;
+    if (ll == 0) {
+      us[lr] = u;
+      if (mine && nb > 1) put(pub + i, u, useq);
+    }
+  };
+  auto product = [&]() {  // the surrounding rows' u, then w = K u (the same in all lanes of a row)
+    lost |= !get_all(nh, useq, [&](int h) { return pub + a.halo[h0 + h]; }, [&](int h, double v) { us[R + h] = v; });
+    __syncthreads();
+    w = 0.0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) w = fma(k[j], us[(j & 1) ? lc[j / 2] >> 16 : lc[j / 2] & 0xffffu], w);
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  };
+  // Sums over the grid of the values v of lanes ll == 0 (first) and ll == 1 (second), the others zero, into
+  // total[2], total[3] of warp 0; `decide` runs in warp 0 with them before the closing barrier.
+  auto reduce = [&](double v, auto decide) {
+#pragma unroll
+    for (int o = L; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane < 2) part[0][2 * warp + lane] = v;
+    __syncthreads();
+    ++sseq;
+    ulonglong2* slot = slots + (sseq & 1) * 2 * nb;
+    double acc = 0.0;
+    if (warp == 0) {
+      acc = lane < 2 * nw ? part[0][lane] : 0.0;
+      for (int o = 2; o < 2 * nw; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane < 2 && nb > 1) put(slot + 2 * blockIdx.x + lane, acc, sseq);
+    }
+    if (nb > 1) {
+      acc = 0.0;
+      lost |= !get_all(2 * nb, sseq, [&](int e) { return slot + e; }, [&](int, double q) { acc += q; });
+#pragma unroll
+      for (int o = 2; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane < 2) part[1][2 * warp + lane] = acc;
+      if (__syncthreads_or(lost) && t == 0) action = 4;
+      if (warp == 0) {
+        acc = lane < 2 * nw ? part[1][lane] : 0.0;
+        for (int o = 2; o < 2 * nw; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      }
+    }
+    if (warp == 0) {
+      const double q0 = __shfl_sync(0xffffffffu, acc, 0), q1 = __shfl_sync(0xffffffffu, acc, 1);
+      __syncwarp();
+      if (lane == 0 && action == 0) decide(q0, q1);
+    }
+    __syncthreads();
+  };
+  // scalars of the iteration, thread 0 only
+  double gamma = 0.0, rgamma = 0.0, den = 0.0, stop = 0.0;
+  int it = 0;
+  reduce(ll < 2 ? r * (ll ? u : r) : 0.0, [&](double ff, double ru) {
+    a.out[0] = sqrt(ff);
+    gamma = ru;
+    stop = a.rtol * a.rtol * gamma;
+    if (!(gamma > 0.0)) action = 1;
+  });
+  if (action == 0) {
+    publish();
+    product();
+    reduce(ll == 1 ? w * u : 0.0, [&](double, double delta) {
+      if (!(delta > 0.0)) {
+        action = 3;
+        return;
+      }
+      den = delta;
+      total[0] = gamma * recip(delta);
+      total[1] = 0.0;
+    });
+  }
+  while (action == 0) {
+    const double alpha = total[0], beta = total[1], u_old = u;
+    s = fma(beta, s, w);
+    r = fma(-alpha, s, r);
+    u = r * di;
+    publish();
+    p = fma(beta, p, u_old);  // off the path of u: while it travels
+    x = fma(alpha, p, x);
+    if (t == 0) rgamma = recip(gamma);
+    product();
+    reduce(ll < 2 ? u * (ll ? w : r) : 0.0, [&](double g, double dl) {
+      ++it;
+      if (g <= stop) {
+        action = 1;
+        return;
+      }
+      if (it >= a.max_it) {
+        action = 2;
+        return;
+      }
+      const double b = g * rgamma;
+      den = fma(-b * b, den, dl);  // d - beta g / alpha, with alpha = gamma / (the last) den
+      if (!(den > 0.0)) {
+        action = 3;
+        return;
+      }
+      total[0] = g * recip(den);
+      total[1] = b;
+      gamma = g;
+    });
+  }
+  if (mine && ll == 0) a.du[i] = x;
+  if (blockIdx.x == 0 && t == 0) {
+    a.out[1] = (double)it;
+    a.out[2] = (double)(action - 1);  // 0 converged, 1 cap, 2 breakdown, 3 gave up waiting
+  }
+}
+
 }  // namespace
 
 size_t macro_solve_work_doubles(int n, int blocks) { return 6 * (size_t)n + 4 * (size_t)blocks; }
@@ -198,6 +427,79 @@ int macro_solve_blocks(int num_sms, long long n_rows) {
   long long b = (n_rows + kRowsPerBlock - 1) / kRowsPerBlock;
   if (b < 1) b = 1;
   return (int)(b < num_sms ? b : num_sms);
+}
+
+// Lanes per row, rows and blocks of the resident kernel for a mesh of n rows (0 lanes: not resident).  An FP64
+// warp instruction takes 64 cycles of an SM sub-partition however many of its lanes are active, so an iteration
+// counts (instructions of a warp) x (warps per sub-partition): with L lanes a row, 8 + nnz / L + ... instructions
+// and R L / 128 warps.  R <= 16 rows: 8 lanes fill the four sub-partitions with one warp each; up to 32 rows 4
+// lanes, above that 2.  A mesh of up to 128 rows (3D, with 81 nonzeros a row: 64) is solved by one block, which
+// exchanges nothing.
+MacroResident macro_resident_plan(int dim, int n, int num_sms) {
+  MacroResident m{};
+  const int rows = n <= (dim == 2 ? 128 : 64) ? n : std::max(16, (n + num_sms - 1) / num_sms);
+  if (rows > kResMaxRows) return m;
+  m.lanes = rows <= 16 ? 8 : rows <= 32 ? 4 : 2;
+  const int per_warp = 32 / m.lanes;
+  m.rows = (rows + per_warp - 1) / per_warp * per_warp;
+  m.blocks = (n + m.rows - 1) / m.rows;
+  return m;
+}
+
+// Per block the distinct columns outside its rows (in the order met), and per nonzero its column's place among the
+// block's rows and those.  The d rows of a node have the same columns.  False if a block needs more places than
+// the shared memory for u holds.
+bool macro_resident_columns(MacroResident& m, int dim, int n, const std::vector<int32_t>& rowptr,
+                            const std::vector<int32_t>& col, std::vector<int32_t>& halo_ptr, std::vector<int32_t>& halo,
+                            std::vector<uint16_t>& lcol) {
+  halo_ptr.assign(1, 0);
+  halo.clear();
+  lcol.resize(col.size());
+  std::vector<int32_t> block(n, -1);  // the block that last met this column
+  std::vector<uint16_t> place(n);
+  int most = 0;
+  for (int b = 0; b < m.blocks; ++b) {
+    const int r0 = b * m.rows, r1 = std::min(n, r0 + m.rows);
+    int places = m.rows;
+    for (int i = r0; i < r1; ++i) {
+      block[i] = b;
+      place[i] = (uint16_t)(i - r0);
+    }
+    for (int i = r0; i < r1; ++i) {
+      if (i > r0 && i % dim != 0) {
+        std::copy(lcol.begin() + rowptr[i - 1], lcol.begin() + rowptr[i], lcol.begin() + rowptr[i]);
+        continue;
+      }
+      for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
+        const int32_t c = col[e];
+        if (block[c] != b) {
+          block[c] = b;
+          place[c] = (uint16_t)places++;
+          halo.push_back(c);
+        }
+        lcol[e] = place[c];
+      }
+    }
+    if (places > 4096) return false;
+    most = std::max(most, places);
+    halo_ptr.push_back((int32_t)halo.size());
+  }
+  m.smem = sizeof(double) * most;
+  return true;
+}
+
+cudaError_t macro_solve_resident_launch(const MacroSolveArgs& a, int dim, const MacroResident& m, cudaStream_t stream) {
+  void* args[] = {(void*)&a};
+  const void* kernel;
+  if (dim == 2)
+    kernel = m.lanes == 8   ? (const void*)macro_pcg_resident_kernel<8, 3>
+             : m.lanes == 4 ? (const void*)macro_pcg_resident_kernel<4, 5>
+                            : (const void*)macro_pcg_resident_kernel<2, 9>;
+  else
+    kernel = m.lanes == 8   ? (const void*)macro_pcg_resident_kernel<8, 11>
+             : m.lanes == 4 ? (const void*)macro_pcg_resident_kernel<4, 21>
+                            : (const void*)macro_pcg_resident_kernel<2, 41>;
+  return cudaLaunchCooperativeKernel(kernel, dim3(m.blocks), dim3(m.rows * m.lanes), args, m.smem, stream);
 }
 
 cudaError_t macro_solve_launch(const MacroSolveArgs& a, int blocks, cudaStream_t stream) {

@@ -4,6 +4,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <vector>
+
 namespace fehmm {
 
 struct Rve2dArgs {
@@ -65,6 +67,7 @@ struct MacroArgs {
   const double* A;      // [n_qp][d^4]
   double* f;            // [n_nodes*dim]
   double* K;            // [nnz]
+  const double* grad;         // [nen][nq][dim] shape gradients at the Gauss points (the same in every element)
   const int32_t* blk_base;    // [n_el][nen][nen] CSR position of the (I,J) block's (0,0) entry
   const int32_t* blk_stride;  // [n_el][nen] row stride (entries) between the dim rows of node I
 };
@@ -81,7 +84,22 @@ struct MacroSolveArgs {
   double* out;              // [3]: |f_free|_2, iterations, status (0 ok, 1 cap, 2 breakdown)
   double rtol;
   int max_it;
+  // resident kernel only
+  const int32_t* halo_ptr;  // [blocks + 1]
+  const int32_t* halo;      // rows around each block's
+  const uint16_t* lcol;     // [nnz] column's place in the block's u
+  void* pub;                // 16-byte words: n of u, 4 per block of the partial sums
 };
+
+struct MacroResident {
+  int lanes = 0, rows = 0, blocks = 0;
+  size_t smem = 0;
+};
+MacroResident macro_resident_plan(int dim, int n, int num_sms);
+bool macro_resident_columns(MacroResident& m, int dim, int n, const std::vector<int32_t>& rowptr,
+                            const std::vector<int32_t>& col, std::vector<int32_t>& halo_ptr, std::vector<int32_t>& halo,
+                            std::vector<uint16_t>& lcol);
+cudaError_t macro_solve_resident_launch(const MacroSolveArgs& a, int dim, const MacroResident& m, cudaStream_t stream);
 
 size_t macro_solve_work_doubles(int n, int blocks);
 int macro_solve_blocks(int num_sms, long long n_rows);
@@ -93,6 +111,7 @@ cudaError_t macro_dirichlet_launch(double* u, double* du, int n, const int32_t* 
 cudaError_t macro_update_launch(double* u, const double* du, int n, cudaStream_t stream);
 cudaError_t macro_spmv_launch(const int32_t* rowptr, const int32_t* col, const double* K, const double* x,
                               double scale, double* y, int n, cudaStream_t stream);
+cudaError_t macro_grad_launch(const MacroArgs& m, double* grad);
 cudaError_t macro_assemble_launch(const MacroArgs& m, cudaStream_t stream, int* launches);
 
 }  // namespace fehmm
