@@ -43,10 +43,10 @@ struct fehmm_ctx {
   int32_t* d_queue = nullptr;  // [kMaxClasses] work counters
   void* d_scratch = nullptr;
   size_t scratch_bytes = 0;
-  // 2D: the points of one grid size, a launch of their own with a block shaped for that grid (a
-  // contiguous range of d_order); 3D: one class with every point
+  // the points of one grid size, a launch of their own with a block shaped for that grid (a contiguous
+  // range of d_order)
   struct SizeClass {
-    int n, first, count, blocks;
+    int n, first, count, blocks, per_sm;
     size_t scratch_off;
   };
   std::vector<SizeClass> classes;
@@ -78,7 +78,7 @@ struct fehmm_ctx {
 
 namespace {
 
-constexpr int kMaxClasses = 16;  // 2D grid sizes: even, 2..32
+constexpr int kMaxClasses = 16;  // grid sizes: 2D even, 2..32; 3D 2..16
 constexpr int kMaxSide = 7;
 
 template <typename T>
@@ -314,37 +314,33 @@ int fehmm_bind_qps(fehmm_ctx* c, int n_qp, const int32_t* rve_of_qp) {
   const bool mixed = c->opt.precision == FEHMM_PREC_MIXED;
   std::vector<fehmm_ctx::SizeClass> classes;
   size_t sb = 0;
-  if (d == 3) {
-    const int blocks = std::min(n_qp, c->num_sms);
-    classes.push_back({0, 0, n_qp, blocks, 0});
-    sb = rve3d_scratch_bytes(nn_max, mixed, blocks);
-  } else {
-    for (int first = 0; first < n_qp;) {  // order is sorted by size
-      const int nn = nodes[order[first]];
-      int end = first;
-      while (end < n_qp && nodes[order[end]] == nn) ++end;
-      const int blocks = std::min(end - first, c->num_sms * rve2d_blocks_per_sm(nn, mixed));
-      classes.push_back({c->rve_n[rve_of_qp[order[first]]], first, end - first, blocks, sb});
-      sb += (rve2d_scratch_bytes(nn, mixed, blocks) + 255) & ~size_t(255);
-      first = end;
+  for (int first = 0; first < n_qp;) {  // order is sorted by size
+    const int nn = nodes[order[first]];
+    int end = first;
+    while (end < n_qp && nodes[order[end]] == nn) ++end;
+    const int per_sm = d == 2 ? rve2d_blocks_per_sm(nn, mixed) : rve3d_blocks_per_sm(nn, mixed, end - first, c->num_sms);
+    const int blocks = std::min(end - first, c->num_sms * per_sm);
+    classes.push_back({c->rve_n[rve_of_qp[order[first]]], first, end - first, blocks, per_sm, sb});
+    sb += ((d == 2 ? rve2d_scratch_bytes(nn, mixed, blocks) : rve3d_scratch_bytes(nn, mixed, blocks)) + 255) & ~size_t(255);
+    first = end;
+  }
+  while (c->side.size() < std::min<size_t>(classes.size() - 1, kMaxSide)) {
+    cudaStream_t t = nullptr;
+    cudaEvent_t e = nullptr;
+    if ((!c->fork && cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess) ||
+        cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      c->n_qp = 0;
+      return FEHMM_ERR_CUDA;
     }
-    while (c->side.size() < std::min<size_t>(classes.size() - 1, kMaxSide)) {
-      cudaStream_t t = nullptr;
-      cudaEvent_t e = nullptr;
-      if ((!c->fork && cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess) ||
-          cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking) != cudaSuccess) {
-        cudaGetLastError();
-        c->n_qp = 0;
-        return FEHMM_ERR_CUDA;
-      }
-      c->side.push_back(t);
-      if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        c->n_qp = 0;
-        return FEHMM_ERR_CUDA;
-      }
-      c->joined.push_back(e);
+    if (cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaEventDestroy(e);
+      cudaGetLastError();
+      c->n_qp = 0;
+      return FEHMM_ERR_CUDA;
     }
+    c->side.push_back(t);
+    c->joined.push_back(e);
   }
   if (sb > c->scratch_bytes) {
     if (c->d_scratch) cudaFree(c->d_scratch);
@@ -426,14 +422,6 @@ static int rve_solve_impl(fehmm_ctx* c, const double* F, double* P, double* A, d
   a.mg_omega = (float)c->opt.mg_omega;
   a.mg_reuse = c->opt.mg_reuse;
   if (cudaMemsetAsync(c->d_queue, 0, sizeof(int32_t) * kMaxClasses, s) != cudaSuccess) return FEHMM_ERR_CUDA;
-  if (c->opt.dim == 3) {
-    if (rve3d_launch(a, mixed, c->classes[0].blocks, s) != cudaSuccess) {
-      cudaGetLastError();
-      return FEHMM_ERR_CUDA;
-    }
-    c->launches += 1;
-    return FEHMM_OK;
-  }
   // One launch per grid size, the largest grid first on the caller's stream and the others beside it
   // on the context's side streams: they are forked from the caller's stream and joined to it again,
   // so the caller sees one ordered operation (and a capture records the fork).  Every launch walks
@@ -448,17 +436,18 @@ static int rve_solve_impl(fehmm_ctx* c, const double* F, double* P, double* A, d
   int started = 0;
   for (int k = 0; k < nc && err == cudaSuccess; ++k) {
     const fehmm_ctx::SizeClass& g = c->classes[k];
-    a.nn_max = g.n * g.n;
+    a.nn_max = c->opt.dim == 2 ? g.n * g.n : g.n * g.n * g.n;
     a.queue = c->d_queue + k;
     a.scratch = static_cast<char*>(c->d_scratch) + g.scratch_off;
-    a.scratch_stride = rve2d_scratch_stride(a.nn_max, mixed);
+    a.scratch_stride = c->opt.dim == 2 ? rve2d_scratch_stride(a.nn_max, mixed) : 0;
     if (list) {
       a.only_n = nc > 1 ? g.n : 0;
     } else {
       a.order = c->d_order + g.first;
       a.n_qp = g.count;
     }
-    err = rve2d_launch(a, mixed, g.blocks, k == 0 ? s : c->side[(k - 1) % ns]);
+    cudaStream_t on = k == 0 ? s : c->side[(k - 1) % ns];
+    err = c->opt.dim == 2 ? rve2d_launch(a, mixed, g.blocks, on) : rve3d_launch(a, mixed, g.blocks, g.per_sm, on);
     if (err == cudaSuccess) ++started;
   }
   // joined even after a failed launch, so that nothing runs on unordered

@@ -9,19 +9,20 @@
 // omega/|K_delta| T^T K T, Eq. k-mac-element-6; the two are checked equal in the oracle tests).
 //
 // GB300 layout:
-//  * 512 threads per block, one block per SM.  Elements are processed thread-strided; the
-//    nodal unknowns live in per-block global scratch (L2 resident), except the vector the
-//    tangent is applied to and its product, which live in shared memory.
-//  * Residual in FP64 per element (edge differences of the fluctuation; P = mu F + hb F^-T),
-//    element forces staged in global scratch and gathered per node (deterministic sums).
-//  * Tangent apply matrix-free in TA (FP32 in mixed mode): per Gauss point the kernel stores
-//    F^-T, hb and lam J^2 (11 values); the apply computes dF = Grad p from edge differences,
-//    dP = mu dF - hb Fit dF^T Fit + gm (Fit:dF) Fit and adds the element's nodal results to
-//    shared memory with float atomics.
-//  * Preconditioner: geometric multigrid V(1,1)-cycle with Galerkin coarse levels where the
-//    grid halves down to 2 or 3 nodes per axis, else block-Jacobi with the 3x3 nodal diagonal
-//    blocks; PCG in the single-reduction form of Chronopoulos and Gear; truncated on negative
+//  * One block per RVE, 512 threads and one block per SM, or two of 256 (see rve3d_blocks_per_sm); the points of
+//    each grid size are a launch of their own.  The apply's vectors, in mixed mode also the FP32 fluctuation, the
+//    residual and the coarse vectors, live in shared memory; the other PCG vectors stream from per-block scratch.
+//  * Residual and tangent apply: two lanes per element, one for each plane of four Gauss points (Cell3).  The FP64
+//    residual stages element forces in global scratch and gathers them per node; the apply, matrix-free in TA
+//    (FP32 in mixed mode), evaluates F again and adds corner by corner without atomics (deterministic sums).
+//  * Preconditioner: geometric multigrid V(1,1)-cycle with Galerkin coarse levels (27-point stencils, several
+//    lanes per node) where the grid halves down to 2 or 3 nodes per axis, else block-Jacobi with the 3x3 nodal
+//    diagonal blocks; PCG in the single-reduction form of Chronopoulos and Gear; truncated on negative
 //    curvature for Newton corrections.
+//  * Measured on a GB300, mixed precision, one pass from a committed state, against stored Gauss-point data, shared
+//    atomics and element-block coarse operators: 152 RVEs of 8^3 18.2 -> 8.8 ms, 12^3 56.6 -> 28.7, 16^3
+//    141 -> 70.0; cycles of one application for 16^3 218 000 -> 125 000, of the coarse levels 313 000 -> 77 000, of
+//    a residual evaluation 4.6 -> 2.0 million.
 //  * Tangent transfer: L_c = apply of the element operator to the constant gradient E_c (the
 //    affine field), 9 PCG solves X_c = -K^-1 L_c, Abar = <A> + sym(L^T X), all sums in FP64.
 #include <cuda_runtime.h>
@@ -259,6 +260,166 @@ __device__ __forceinline__ void nat_scatter(const T (&S)[9], T c, T s, T t, T r,
   }
 }
 
+// ---------------------------------------------------------------- half an element per thread
+// The residual and the tangent apply give an element to two lanes (l and l + 16 of a warp), one for each plane of
+// four Gauss points zeta = r: a lane interpolates the field to its plane first (h, and the vertical differences
+// v), so the gradient costs 90 operations in place of 144 a component-wise evaluation shares between 8 points,
+// and its 24 + 24 values fit the registers beside the field's own (one thread per element needs 255 registers).
+// Element (i, j, k) of lane pair e: corners column q = ox + 2 oy, bottom (k) and top (k + 1).
+struct Cell3 {
+  int bot[4], top[4];  // nodes of the columns
+  bool in, upper;      // an element at all; this lane's plane
+  bool full;           // every lane of the block has one
+  int e;
+  bool pb[4], pt[4];   // pinned nodes
+};
+
+__device__ __forceinline__ int div_n(int x, int magic) { return (x * magic) >> 16; }  // x / n, x < 4096
+
+__device__ __forceinline__ Cell3 cell3(int pass, int n, int NE, int magic, int bc) {
+  Cell3 c;
+  const int lane = threadIdx.x & 31;
+  c.upper = lane >= 16;
+  c.e = pass * (blockDim.x / 2) + (threadIdx.x >> 5) * 16 + (lane & 15);
+  c.in = c.e < NE;
+  c.full = (pass + 1) * (int)(blockDim.x / 2) <= NE;
+  const int e = c.in ? c.e : 0;
+  const int jk = div_n(e, magic), i = e - n * jk, k = div_n(jk, magic), j = jk - n * k;
+  const int i1 = i + 1 == n ? 0 : i + 1, j1 = j + 1 == n ? 0 : j + 1, k1 = k + 1 == n ? 0 : k + 1;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int x = q & 1 ? i1 : i, y = q & 2 ? j1 : j;
+    c.bot[q] = x + n * (y + n * k);
+    c.top[q] = x + n * (y + n * k1);
+    c.pb[q] = bc ? (x == 0 || y == 0 || k == 0) : c.bot[q] == 0;
+    c.pt[q] = bc ? (x == 0 || y == 0 || k1 == 0) : c.top[q] == 0;
+  }
+  return c;
+}
+
+// natural-coordinate gradients of one component on the plane zeta = r: gx[eta point], gy[xi point],
+// gz[eta point][xi point]; b, t: the field at the bottom and top nodes of the four columns
+template <typename T>
+__device__ __forceinline__ void plane_grad(const T (&b)[4], const T (&t)[4], T r, T (&gx)[2], T (&gy)[2], T (&gz)[2][2]) {
+  const T s0 = (T)g01(0), s1 = (T)g01(1);
+  T h[4], v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    v[q] = t[q] - b[q];
+    h[q] = b[q] + r * v[q];
+  }
+  const T x0 = h[1] - h[0], x1 = h[3] - h[2], dx = x1 - x0;
+  gx[0] = x0 + s0 * dx;
+  gx[1] = x0 + s1 * dx;
+  const T y0 = h[2] - h[0], y1 = h[3] - h[1], dy = y1 - y0;
+  gy[0] = y0 + s0 * dy;
+  gy[1] = y0 + s1 * dy;
+  const T e0 = v[1] - v[0], e1 = v[3] - v[2];
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    const T s = p ? s1 : s0, lo = v[0] + s * e0, hi = v[2] + s * e1, d = hi - lo;
+    gz[0][p] = lo + s0 * d;
+    gz[1][p] = lo + s1 * d;
+  }
+}
+
+// the transpose: nodal values of one component from the stress columns summed on the plane
+template <typename T>
+__device__ __forceinline__ void plane_scatter(const T (&sx)[2], const T (&sy)[2], const T (&sz)[2][2], T r, T (&b)[4], T (&t)[4]) {
+  // q = 1 - s in T, not the other abscissa: the two differ in the last bit, and the gradient's weights are these
+  const T s0 = (T)g01(0), s1 = (T)g01(1), q0 = T(1) - s0, q1 = T(1) - s1;
+  const T x0 = q0 * sx[0] + q1 * sx[1], x1 = s0 * sx[0] + s1 * sx[1];
+  const T y0 = q0 * sy[0] + q1 * sy[1], y1 = s0 * sy[0] + s1 * sy[1];
+  const T h[4] = {-x0 - y0, x0 - y1, y0 - x1, x1 + y1};
+  T c0[2], c1[2];
+#pragma unroll
+  for (int p = 0; p < 2; ++p) {
+    c0[p] = q0 * sz[0][p] + q1 * sz[1][p];
+    c1[p] = s0 * sz[0][p] + s1 * sz[1][p];
+  }
+  const T v[4] = {q0 * c0[0] + q1 * c0[1], s0 * c0[0] + s1 * c0[1], q0 * c1[0] + q1 * c1[1], s0 * c1[0] + s1 * c1[1]};
+  const T q = T(1) - r;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    b[k] = q * h[k] - v[k];
+    t[k] = r * h[k] + v[k];
+  }
+}
+
+// out[comp * NN + node] += the element's nodal values, without atomics: the two lanes of an element exchange
+// halves (the lower keeps the bottom nodes, the upper the top ones), then one corner at a time, which is a
+// different node for every element, with a barrier between.  (Shared-memory float atomics are compare-and-swap
+// loops; neighbouring lanes share nodes.)  Where n divides 16 the lanes of a row hold all its elements: the two
+// corners of a node along x are added by a shuffle first, which halves the steps.  All threads call it; ends with
+// a barrier.
+template <typename T>
+__device__ __forceinline__ void add_corners(const Cell3& c, const T (&yb)[3][4], const T (&yt)[3][4], T* out, int NN, int n) {
+  T y[3][4];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const T send = c.upper ? yb[i][q] : yt[i][q];
+      y[i][q] = (c.upper ? yt[i][q] : yb[i][q]) + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+  const bool rows = (16 % n) == 0 && c.full;
+  if (rows) {  // node (i, ., .) gets corner 1 of element i - 1
+    const int lane = threadIdx.x & 31, src = (lane & (n - 1)) ? lane - 1 : lane + n - 1;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; q += 2) y[i][q] += __shfl_sync(0xffffffffu, y[i][q + 1], src);
+  }
+#pragma unroll
+  for (int ph = 0; ph < 8; ++ph) {
+    const int q = ph & 3;
+    if ((q & 1) && rows) continue;
+    const bool pin = ph < 4 ? c.pb[q] : c.pt[q];
+    if (c.in && !pin && c.upper == (ph >= 4)) {
+      const int v = ph < 4 ? c.bot[q] : c.top[q];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) out[i * NN + v] += y[i][q];
+    }
+    __syncthreads();
+  }
+}
+
+// cofactors c_iJ = dJ/dF_iJ; returns J = det F
+template <typename T>
+__device__ __forceinline__ T cofactors(const T (&F)[9], T (&c)[9]) {
+  c[0] = F[4] * F[8] - F[5] * F[7];
+  c[1] = F[5] * F[6] - F[3] * F[8];
+  c[2] = F[3] * F[7] - F[4] * F[6];
+  c[3] = F[2] * F[7] - F[1] * F[8];
+  c[4] = F[0] * F[8] - F[2] * F[6];
+  c[5] = F[1] * F[6] - F[0] * F[7];
+  c[6] = F[1] * F[5] - F[2] * F[4];
+  c[7] = F[2] * F[3] - F[0] * F[5];
+  c[8] = F[0] * F[4] - F[1] * F[3];
+  return F[0] * c[0] + F[1] * c[1] + F[2] * c[2];
+}
+
+// Neo-Hookean dP = mu dF - hb Fit dF^T Fit + gm (Fit:dF) Fit in terms of F alone: with c = cof F = J Fit,
+// a = c:dF and dc = d(cof F) (bilinear in F and dF), c dF^T c = a c - J dc, and gm / J^2 = lam, so
+//   dP = mu dF + (lam - b) a c + b J dc,   b = hb / J^2 = lam/2 - (lam/2 + mu) / J^2.
+template <typename T>
+__device__ __forceinline__ void nh_action(const T (&F)[9], const T (&d)[9], T lam, T mu, T (&dP)[9]) {
+  T c[9];
+  const T J = cofactors(F, c);
+  const T b = T(0.5) * lam - (T(0.5) * lam + mu) * recip_T(J * J);
+  T a = c[0] * d[0];
+#pragma unroll
+  for (int k = 1; k < 9; ++k) a += c[k] * d[k];
+  const T ca = (lam - b) * a, cb = b * J;
+  auto dcof = [&](int p, int q, int r, int t) {  // d(F_p F_q - F_r F_t)
+    return d[p] * F[q] + F[p] * d[q] - d[r] * F[t] - F[r] * d[t];
+  };
+  const T dc[9] = {dcof(4, 8, 5, 7), dcof(5, 6, 3, 8), dcof(3, 7, 4, 6), dcof(2, 7, 1, 8), dcof(0, 8, 2, 6),
+                   dcof(1, 6, 0, 7), dcof(1, 5, 2, 4), dcof(2, 3, 0, 5), dcof(0, 4, 1, 3)};
+#pragma unroll
+  for (int k = 0; k < 9; ++k) dP[k] = mu * d[k] + ca * c[k] + cb * dc[k];
+}
+
 template <typename TA>
 struct Scratch3 {
   // per-block global scratch, layout set by scratch3_layout
@@ -285,15 +446,17 @@ __host__ __device__ inline int mg3_levels(int n) {
   return (m <= 3 && l >= 1) ? l : 0;
 }
 // Elements (TA) of the multigrid region for grid n: per coarse level the element blocks
-// [36][9][NE], the inverted nodal blocks [6][NN] and r, z, t [3][NN]; then the coarsest
-// inverse (two buffers of D x (D + 1), D = 3 NN_c).
+// [36][9][NE], the inverted nodal blocks [6][NN], r, z, t [3][NN] and (smoothing levels, reserved on
+// all) the assembled stencil [27][9][NN]; then the coarsest inverse (two buffers of D x (D + 1),
+// D = 3 NN_c).
+constexpr int kMg3Node = 324 + 6 + 9 + 243;
 __host__ __device__ inline long long mg3_elems(int n) {
   const int L = mg3_levels(n);
   if (!L) return 0;
   long long e = 0;
   for (int l = 1; l <= L; ++l) {
     const long long m = n >> l, nn = m * m * m;
-    e += 324 * nn + 6 * nn + 9 * nn;
+    e += kMg3Node * nn;
   }
   const long long m = n >> L, D = 3 * m * m * m;
   return e + 2 * D * (D + 1);
@@ -339,10 +502,35 @@ __device__ inline Scratch3<TA> scratch3_layout(unsigned char* base, int NN) {
   return s;
 }
 
-// shared memory: vin [3][NN], vout [3][NN] (TA), reductions, lame, misc
+// coarse vectors r, z, t of every level of grid n
+__host__ __device__ inline int mg3_vec_elems(int n) {
+  int e = 0;
+  for (int l = 1; l <= mg3_levels(n); ++l) e += 9 * (n >> l) * (n >> l) * (n >> l);
+  return e;
+}
+
+// shared memory: reductions, lame, misc, then vin [3][NN], vout [3][NN] (TA) and in mixed mode the fluctuation
+// [3][NN], the residual [3][NN] and the coarse vectors (sized for the grid of the batch that needs most)
+constexpr size_t kSmem3Misc = sizeof(double) * (2 * 512 + 2 * kMaxPhase);  // 128: 16 sums, 81 of the transfer,
+constexpr size_t kSmem3LameT = kSmem3Misc + sizeof(double) * 100;           // Lame table and Fbar in TA
+constexpr size_t kSmem3Fixed = kSmem3Misc + sizeof(double) * 128;
 template <typename TA>
 __host__ __device__ inline size_t smem3_bytes(int NN) {
-  return sizeof(TA) * 6 * (size_t)NN + sizeof(double) * (2 * 512 + 2 * kMaxPhase + 128);
+  size_t most = sizeof(TA) * 6 * (size_t)NN;
+  if (sizeof(TA) == 4)
+    for (int n = 2; n * n * n <= NN; ++n) {
+      const size_t need = sizeof(TA) * (12 * (size_t)n * n * n + mg3_vec_elems(n));
+      if (need > most) most = need;
+    }
+  return kSmem3Fixed + most;
+}
+
+extern __shared__ __align__(16) unsigned char smem3[];
+// The vectors in shared memory, addressed from the shared array itself (through the context's pointers every
+// access would be a generic one).
+template <typename TA>
+__device__ __forceinline__ TA* smem_vin() {
+  return reinterpret_cast<TA*>(smem3 + kSmem3Fixed);
 }
 
 template <typename T>
@@ -366,6 +554,7 @@ struct Mg3Level {
   TA* r;   // [3][NN]
   TA* z;   // [3][NN]
   TA* t;   // [3][NN]
+  TA* st;  // [27 neighbours][9][NN] assembled stencil
 };
 
 template <typename TA>
@@ -375,11 +564,14 @@ struct Mg3 {
   int bc = 0;      // pinned nodes of every level as on the fine grid (pinned3)
   TA omega = TA(0.6);  // smoother damping
   TA* base = nullptr;
+  TA* vec = nullptr;  // coarse vectors in shared memory (null: in the scratch)
   __device__ __forceinline__ Mg3Level<TA> level(int l) const {
     TA* p = base;
+    int nodes = 0;
     for (int q = 1; q < l; ++q) {
       const int m = n >> q;
-      p += 339 * m * m * m;
+      nodes += m * m * m;
+      p += kMg3Node * m * m * m;
     }
     Mg3Level<TA> v;
     v.n = n >> l;
@@ -390,11 +582,17 @@ struct Mg3 {
     v.r = v.mi + 6 * v.NN;
     v.z = v.r + 3 * v.NN;
     v.t = v.z + 3 * v.NN;
+    v.st = p + (kMg3Node - 243) * v.NN;
+    if (vec) {
+      v.r = vec + 9 * nodes;
+      v.z = v.r + 3 * v.NN;
+      v.t = v.z + 3 * v.NN;
+    }
     return v;
   }
   __device__ __forceinline__ TA* inverse() const {
     const Mg3Level<TA> c = level(levels);
-    return c.t + 3 * c.NN;
+    return c.kb + (size_t)kMg3Node * c.NN;
   }
 };
 
@@ -405,78 +603,124 @@ struct Ctx3 {
   Mg3<TA> mg;
   const uint8_t* phase;
   const double* lame;  // shared [kMaxPhase][2]
+  const TA* lame_t;    // the same in the arithmetic type (a conversion from FP64 costs an FP64 instruction),
+  TA* Fb_t;            // and Fbar of the current stage, both shared
   Scratch3<TA> sc;
   TA* vin;   // shared [3][NN]
   TA* vout;  // shared [3][NN]
+  const double* w;  // fluctuation [NN][3] (global)
+  TA* w32;   // mixed: its FP32 copy, shared [3][NN] (FP64 mode reads w itself)
+  int magic;  // ceil(65536 / n), see div_n
   double* red;  // shared 2*512
   int bc;       // 0 periodic, 1 KUBC (pinned3)
   double Fb[9];
 };
 
 // ---------------------------------------------------------------- FP64 residual
+// The FP64 pipe bounds it (64 cycles per warp instruction on an SM sub-partition), so it is written for few FP64
+// instructions: plane by plane (two lanes per element, see Cell3), the neo-Hookean stress P = mu F + c cof F added
+// straight into the sums over the points that share a shape gradient (mu F of a column is the same for both),
+// <P> from those sums, J <= 0 read from the sign bit: about 430 per lane.  Evaluated point by point with the
+// general gradient it took about 2400 per element (16^3: 4.6 million cycles an evaluation).
+__device__ __forceinline__ bool is_positive(double x) {  // x > 0 (false for NaN) by integer comparison
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+
 template <typename TA, int LAW>
-__device__ __noinline__ void residual3(const Ctx3<TA>& c, const double* w, double (&Psum)[9], double& bad) {
-  const int n = c.g.n;
+__device__ __noinline__ void residual3(const Ctx3<TA>& c, double (&Psum)[9], double& bad) {
+  const int n = c.g.n, NE = c.NE, magic = c.magic;
+  const double* w = c.w;
+  const uint8_t* __restrict__ phase = c.phase;
+  double* Rf = c.sc.Rf;
   const double ih = (double)n, cw = 0.125 / (ih * ih);  // wq / h = h^2 / 8
-  for (int e = threadIdx.x; e < c.NE; e += blockDim.x) {
-    int nd[8];
-    c.g.corners(e, nd);
-    double u[8][3];
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-      for (int i = 0; i < 3; ++i) u[a][i] = w[3 * nd[a] + i];
-    const int ph = c.phase[e];
+  int nbad = 0;
+  for (int pass = 0; pass * (int)(blockDim.x / 2) < NE; ++pass) {
+    const Cell3 q = cell3(pass, n, NE, magic, 0);
+    const int ph = phase[q.in ? q.e : 0];
     const double lam = c.lame[2 * ph], mu = c.lame[2 * ph + 1];
-    double y[8][3];
+    const double r = g01(q.upper);
+    double fx[3][2], fy[3][2], fz[3][2][2];  // columns of F at the plane's points
 #pragma unroll
-    for (int a = 0; a < 8; ++a) y[a][0] = y[a][1] = y[a][2] = 0.0;
-#pragma unroll 1
-    for (int q = 0; q < 8; ++q) {
-      const double s = g01(q & 1), t = g01((q >> 1) & 1), r = g01(q >> 2);
-      double G[9], F[9];
-      nat_grad(u, s, t, r, G);
+    for (int i = 0; i < 3; ++i) {
+      double b[4], t[4];
 #pragma unroll
-      for (int k = 0; k < 9; ++k) F[k] = c.Fb[k] + ih * G[k];
-      double P[9];
-      if constexpr (LAW == kLawNH) {
-        // P = mu F + hb F^-T = mu F + (hb / J) cof(F), the reciprocal refined in FP64
-        double cof[9];
-        cof[0] = F[4] * F[8] - F[5] * F[7];
-        cof[1] = F[5] * F[6] - F[3] * F[8];
-        cof[2] = F[3] * F[7] - F[4] * F[6];
-        cof[3] = F[2] * F[7] - F[1] * F[8];
-        cof[4] = F[0] * F[8] - F[2] * F[6];
-        cof[5] = F[1] * F[6] - F[0] * F[7];
-        cof[6] = F[1] * F[5] - F[2] * F[4];
-        cof[7] = F[2] * F[3] - F[0] * F[5];
-        cof[8] = F[0] * F[4] - F[1] * F[3];
-        const double J = F[0] * cof[0] + F[1] * cof[1] + F[2] * cof[2];
-        bad += J > 0.0 ? 0.0 : 1.0;
-        const double c = (0.5 * lam * (J * J - 1.0) - mu) * recip_fp64(J);
+      for (int k = 0; k < 4; ++k) {
+        b[k] = w[3 * q.bot[k] + i];
+        t[k] = w[3 * q.top[k] + i];
+      }
+      plane_grad(b, t, r, fx[i], fy[i], fz[i]);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) P[k] = fma(mu, F[k], c * cof[k]);
-      } else {
-        const double J = F[0] * (F[4] * F[8] - F[5] * F[7]) - F[1] * (F[3] * F[8] - F[5] * F[6]) +
-                         F[2] * (F[3] * F[7] - F[4] * F[6]);
-        bad += J > 0.0 ? 0.0 : 1.0;
-        double S6[6];
-        svk3_S(F, lam, mu, S6);
+      for (int p = 0; p < 2; ++p) {
+        fx[i][p] = fma(ih, fx[i][p], c.Fb[3 * i]);
+        fy[i][p] = fma(ih, fy[i][p], c.Fb[3 * i + 1]);
+        fz[i][p][0] = fma(ih, fz[i][p][0], c.Fb[3 * i + 2]);
+        fz[i][p][1] = fma(ih, fz[i][p][1], c.Fb[3 * i + 2]);
+      }
+    }
+    double sx[3][2], sy[3][2], sz[3][2][2];  // stress columns, summed over the points of one xi, one eta, neither
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-          for (int J2 = 0; J2 < 3; ++J2)
-            P[3 * i + J2] = F[3 * i] * sym6(S6, 0, J2) + F[3 * i + 1] * sym6(S6, 1, J2) + F[3 * i + 2] * sym6(S6, 2, J2);
+      for (int p = 0; p < 2; ++p) {
+        sx[i][p] = LAW == kLawNH ? 2.0 * mu * fx[i][p] : 0.0;
+        sy[i][p] = LAW == kLawNH ? 2.0 * mu * fy[i][p] : 0.0;
+        sz[i][p][0] = LAW == kLawNH ? mu * fz[i][p][0] : 0.0;
+        sz[i][p][1] = LAW == kLawNH ? mu * fz[i][p][1] : 0.0;
       }
 #pragma unroll
-      for (int k = 0; k < 9; ++k) Psum[k] += P[k];
-      nat_scatter(P, cw, s, t, r, y);
+    for (int gy = 0; gy < 2; ++gy)
+#pragma unroll
+      for (int gx = 0; gx < 2; ++gx) {
+        const double F[9] = {fx[0][gy], fy[0][gx], fz[0][gy][gx], fx[1][gy], fy[1][gx], fz[1][gy][gx],
+                             fx[2][gy], fy[2][gx], fz[2][gy][gx]};
+        double cof[9];
+        const double J = cofactors(F, cof);
+        if (q.in && !is_positive(J)) ++nbad;
+        if constexpr (LAW == kLawNH) {
+          // P = mu F + hb F^-T = mu F + (hb / J) cof(F), hb / J = lam J / 2 - (lam / 2 + mu) / J
+          const double cc = fma(0.5 * lam, J, -(0.5 * lam + mu) * recip_fp64(J));
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            sx[i][gy] = fma(cc, cof[3 * i], sx[i][gy]);
+            sy[i][gx] = fma(cc, cof[3 * i + 1], sy[i][gx]);
+            sz[i][gy][gx] = fma(cc, cof[3 * i + 2], sz[i][gy][gx]);
+          }
+        } else {
+          double S6[6];
+          svk3_S(F, lam, mu, S6);
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            auto P = [&](int J2) {
+              return F[3 * i] * sym6(S6, 0, J2) + F[3 * i + 1] * sym6(S6, 1, J2) + F[3 * i + 2] * sym6(S6, 2, J2);
+            };
+            sx[i][gy] += P(0);
+            sy[i][gx] += P(1);
+            sz[i][gy][gx] += P(2);
+          }
+        }
+      }
+    if (q.in) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        Psum[3 * i] += sx[i][0] + sx[i][1];
+        Psum[3 * i + 1] += sy[i][0] + sy[i][1];
+        Psum[3 * i + 2] += (sz[i][0][0] + sz[i][0][1]) + (sz[i][1][0] + sz[i][1][1]);
+      }
     }
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
+    for (int i = 0; i < 3; ++i) {
+      double b[4], t[4];
+      plane_scatter(sx[i], sy[i], sz[i], r, b, t);
 #pragma unroll
-      for (int i = 0; i < 3; ++i) c.sc.Rf[(size_t)(3 * a + i) * c.NE + e] = y[a][i];
+      for (int k = 0; k < 4; ++k) {  // the lower lane stages the bottom corners, the upper the top ones
+        const double send = q.upper ? b[k] : t[k];
+        const double y = (q.upper ? t[k] : b[k]) + __shfl_xor_sync(0xffffffffu, send, 16);
+        if (q.in) Rf[(size_t)(3 * (k + (q.upper ? 4 : 0)) + i) * NE + q.e] = cw * y;
+      }
+    }
   }
+  bad += (double)nbad;
 }
 
 // sum over this thread's elements of psi at the Gauss points (FP64; Eq. NH-free-energy)
@@ -530,11 +774,12 @@ __device__ __noinline__ double energy3(const Ctx3<TA>& c, const double* w) {
 template <typename TA>
 __device__ __forceinline__ void gather_R(const Ctx3<TA>& c, int v, double (&R)[3]) {
   const int n = c.g.n;
-  const int i = v % n, j = (v / n) % n, k = v / (n * n);
+  const int jk = div_n(v, c.magic), i = v - n * jk, k = div_n(jk, c.magic), j = jk - n * k;
+  const int im = i ? i - 1 : n - 1, jm = j ? j - 1 : n - 1, km = k ? k - 1 : n - 1;
   R[0] = R[1] = R[2] = 0.0;
 #pragma unroll
   for (int a = 0; a < 8; ++a) {
-    const int e = c.g.node(i + n - (a & 1), j + n - ((a >> 1) & 1), k + n - ((a >> 2) & 1));
+    const int e = (a & 1 ? im : i) + n * ((a & 2 ? jm : j) + n * (a & 4 ? km : k));
 #pragma unroll
     for (int d = 0; d < 3; ++d) R[d] += c.sc.Rf[(size_t)(3 * a + d) * c.NE + e];
   }
@@ -548,6 +793,8 @@ __device__ __noinline__ void tangent3(const Ctx3<TA>& c, const double* w, double
   const int n = c.g.n, NN = c.g.NN;
   TA* diag = c.vin;  // [6][NN] spans vin and vout
   for (int v = threadIdx.x; v < 6 * NN; v += blockDim.x) diag[v] = TA(0);
+  if (sizeof(TA) == 4)
+    for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) c.w32[(v % 3) * NN + v / 3] = (TA)w[v];
   __syncthreads();
   const TA ih = (TA)n, wq = TA(0.125) / (ih * ih * ih);
   for (int e = threadIdx.x; e < c.NE; e += blockDim.x) {
@@ -693,10 +940,113 @@ __device__ __noinline__ void tangent3(const Ctx3<TA>& c, const double* w, double
 }
 
 // Kept out of line so the element loop gets its own register allocation (no spills).
-// vout = K vin (mode 0) or vout = L_c: the element operator applied to the constant
-// gradient E_c (mode 1, c = 3k + L).  Pinned node 0 row zeroed.
+// vout = K vin.  Pinned rows zero.
+// Two lanes per element (Cell3).  F is evaluated again from the fluctuation (in shared memory in mixed mode)
+// at every application: stored Gauss-point data were 1.5 MB per 16^3 RVE and application, more than the L2 holds
+// for the 152 RVEs in flight (25 % hits), for about 50 operations a point.  Bound by instruction issue (half of
+// the slots) and the corner steps' barriers.
 template <typename TA, int LAW>
-__device__ __noinline__ void apply3(const Ctx3<TA>& c, int mode, int cidx) {
+__device__ __noinline__ void apply3(const Ctx3<TA>& c) {
+  // everything the loop needs in registers: the context itself is in local memory
+  const int n = c.g.n, NN = c.g.NN, NE = c.NE, magic = c.magic, bc = c.bc;
+  const TA* vin = smem_vin<TA>();
+  TA* vout = smem_vin<TA>() + 3 * NN;
+  const TA* w32 = smem_vin<TA>() + 6 * NN;  // mixed mode
+  const double* w = c.w;
+  const uint8_t* __restrict__ phase = c.phase;
+  const TA* lame = reinterpret_cast<const TA*>(smem3 + kSmem3LameT);
+  const TA* Fb = lame + 2 * kMaxPhase;
+  for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) vout[v] = TA(0);
+  __syncthreads();
+  const TA ih = (TA)n, cw = TA(0.125) / (ih * ih);  // wq / h
+  const int first = (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
+  int ph_next = first < NE ? phase[first] : 0;
+  for (int pass = 0; pass * (int)(blockDim.x / 2) < NE; ++pass) {
+    const Cell3 q = cell3(pass, n, NE, magic, bc);
+    const int ph = ph_next;
+    if (q.e + (int)(blockDim.x / 2) < NE) ph_next = phase[q.e + blockDim.x / 2];  // a pass ahead
+    const TA lam = lame[2 * ph], mu = lame[2 * ph + 1];
+    const TA r = (TA)g01(q.upper);
+    TA fx[3][2], fy[3][2], fz[3][2][2];  // columns of F at the plane's points
+    TA dx[3][2], dy[3][2], dz[3][2][2];  // and of the increment's gradient
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      TA b[4], t[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if constexpr (sizeof(TA) == 4) {
+          b[k] = w32[i * NN + q.bot[k]];
+          t[k] = w32[i * NN + q.top[k]];
+        } else {
+          b[k] = (TA)w[3 * q.bot[k] + i];
+          t[k] = (TA)w[3 * q.top[k] + i];
+        }
+      }
+      plane_grad(b, t, r, fx[i], fy[i], fz[i]);
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        fx[i][p] = Fb[3 * i] + ih * fx[i][p];
+        fy[i][p] = Fb[3 * i + 1] + ih * fy[i][p];
+        fz[i][p][0] = Fb[3 * i + 2] + ih * fz[i][p][0];
+        fz[i][p][1] = Fb[3 * i + 2] + ih * fz[i][p][1];
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        b[k] = vin[i * NN + q.bot[k]];
+        t[k] = vin[i * NN + q.top[k]];
+      }
+      plane_grad(b, t, r, dx[i], dy[i], dz[i]);
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        dx[i][p] *= ih;
+        dy[i][p] *= ih;
+        dz[i][p][0] *= ih;
+        dz[i][p][1] *= ih;
+      }
+    }
+    TA sx[3][2], sy[3][2], sz[3][2][2];
+#pragma unroll
+    for (int gy = 0; gy < 2; ++gy)
+#pragma unroll
+      for (int gx = 0; gx < 2; ++gx) {
+        const TA F[9] = {fx[0][gy], fy[0][gx], fz[0][gy][gx], fx[1][gy], fy[1][gx], fz[1][gy][gx],
+                         fx[2][gy], fy[2][gx], fz[2][gy][gx]};
+        const TA d[9] = {dx[0][gy], dy[0][gx], dz[0][gy][gx], dx[1][gy], dy[1][gx], dz[1][gy][gx],
+                         dx[2][gy], dy[2][gx], dz[2][gy][gx]};
+        TA dP[9];
+        if constexpr (LAW == kLawNH) {
+          nh_action(F, d, lam, mu, dP);
+        } else {
+          TA S6[6];
+          svk3_S(F, lam, mu, S6);
+          svk_tangent_action(F, S6, lam, mu, d, dP);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          sx[i][gy] = gx ? sx[i][gy] + dP[3 * i] : dP[3 * i];
+          sy[i][gx] = gy ? sy[i][gx] + dP[3 * i + 1] : dP[3 * i + 1];
+          sz[i][gy][gx] = dP[3 * i + 2];
+        }
+      }
+    TA yb[3][4], yt[3][4];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      plane_scatter(sx[i], sy[i], sz[i], r, yb[i], yt[i]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        yb[i][k] *= cw;
+        yt[i][k] *= cw;
+      }
+    }
+    add_corners(q, yb, yt, vout, NN, n);
+  }
+}
+
+// vout = L_c: the element operator applied to the constant gradient E_c (c = 3k + L), from the Gauss-point data
+// that <A> was summed from: L enters the transferred tangent to first order beside <A>, and both see F rounded
+// the same way.  Nine times per transfer.  Pinned rows zero.
+template <typename TA, int LAW>
+__device__ __noinline__ void unit_gradient3(const Ctx3<TA>& c, int cidx) {
   const int n = c.g.n, NN = c.g.NN;
   for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) c.vout[v] = TA(0);
   __syncthreads();
@@ -704,13 +1054,6 @@ __device__ __noinline__ void apply3(const Ctx3<TA>& c, int mode, int cidx) {
   for (int e = threadIdx.x; e < c.NE; e += blockDim.x) {
     int nd[8];
     c.g.corners(e, nd);
-    TA u[8][3];
-    if (mode == 0) {
-#pragma unroll
-      for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) u[a][i] = c.vin[i * NN + nd[a]];
-    }
     const int ph = c.phase[e];
     const TA mu = (TA)c.lame[2 * ph + 1];
     TA y[8][3];
@@ -720,15 +1063,8 @@ __device__ __noinline__ void apply3(const Ctx3<TA>& c, int mode, int cidx) {
     for (int q = 0; q < 8; ++q) {  // fully unrolled: the shape-function weights fold to constants
       const TA s = (TA)g01(q & 1), t = (TA)g01((q >> 1) & 1), r = (TA)g01(q >> 2);
       TA dF[9];
-      if (mode == 0) {
-        TA G[9];
-        nat_grad(u, s, t, r, G);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) dF[k] = ih * G[k];
-      } else {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) dF[k] = k == cidx ? TA(1) : TA(0);
-      }
+      for (int k = 0; k < 9; ++k) dF[k] = k == cidx ? TA(1) : TA(0);
       TA dP[9];
       if constexpr (LAW == kLawNH) {
         TA qv[12];
@@ -1002,6 +1338,39 @@ __device__ __noinline__ void mg3_build_coarsest(const Mg3<TA>& mg) {
   }
 }
 
+// Assembled 27-point stencil of a smoothing level from its element blocks: neighbour nb = (dx + 1) + 3 (dy + 1)
+// + 9 (dz + 1).  243 values per node in place of the 576 block entries that the eight elements around it hold
+// (level 1 of 16^3: an application took 150 000 cycles gathering those).
+template <typename TA>
+__device__ __noinline__ void mg3_build_stencil(const Mg3<TA>& mg, int l) {
+  const Mg3Level<TA> L = mg.level(l);
+  const int n = L.n, NN = L.NN;
+  for (int task = threadIdx.x; task < 27 * NN; task += blockDim.x) {
+    const int nb = task / NN, v = task % NN;
+    const int i = v % n, j = (v / n) % n, k = v / (n * n);
+    const int d[3] = {nb % 3 - 1, (nb / 3) % 3 - 1, nb / 9 - 1};
+    TA acc[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) acc[q] = TA(0);
+    for (int a = 0; a < 8; ++a) {  // v is corner a of the element, its neighbour corner b
+      int b = 0;
+      bool in = true;
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        const int o = ((a >> x) & 1) + d[x];
+        in = in && (o == 0 || o == 1);
+        b |= (o & 1) << x;
+      }
+      if (!in) continue;
+      const int E = node3(n, (i - (a & 1) + n) % n, (j - ((a >> 1) & 1) + n) % n, (k - (a >> 2) + n) % n);
+#pragma unroll
+      for (int q = 0; q < 9; ++q) acc[q] += mg3_kb<TA>(L, E, a, b, q / 3, q % 3);
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) L.st[(size_t)(nb * 9 + q) * NN + v] = acc[q];
+  }
+}
+
 // After tangent3: all coarse levels of the current tangent.
 template <typename TA, int LAW>
 __device__ void mg3_build(const Ctx3<TA>& c) {
@@ -1011,29 +1380,60 @@ __device__ void mg3_build(const Ctx3<TA>& c) {
     mg3_build_next<TA>(c.mg, l);
   }
   __syncthreads();
-  for (int l = 1; l < c.mg.levels; ++l) mg3_build_diag<TA>(c.mg, l);
+  for (int l = 1; l < c.mg.levels; ++l) {
+    mg3_build_diag<TA>(c.mg, l);
+    mg3_build_stencil<TA>(c.mg, l);
+  }
   mg3_build_coarsest<TA>(c.mg);  // ends with a barrier
   __syncthreads();
 }
 
-// y = K_l z at node v (gathered from the 8 elements around v; zero at the pinned node)
+// Lanes per node on a level: as many (a power of two) as the block has for its nodes, so that the 27 neighbours
+// of a small level's nodes are loaded side by side.
+__device__ __forceinline__ int lanes_per_node(int NN) {
+  int l = 1;
+  while (l < 8 && 2 * l * NN <= (int)blockDim.x) l *= 2;
+  return l;
+}
+
+// Sum of y over the lanes of a node.
 template <typename TA>
-__device__ __forceinline__ void mg3_apply(const Mg3Level<TA>& L, const TA* z, int v, TA (&y)[3]) {
+__device__ __forceinline__ void node_sum(TA (&y)[3], int lanes) {
+  for (int o = lanes >> 1; o > 0; o >>= 1)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) y[d] += __shfl_xor_sync(0xffffffffu, y[d], o);
+}
+
+__device__ __forceinline__ int wrapped(int i, int n) { return i < 0 ? i + n : i >= n ? i - n : i; }
+
+// For every node of a level: body(v, lane, lanes) by the node's lanes, `end(v)` by its first lane after the sum
+// of what body left in y.  Whole warps stay in the loop.
+template <typename TA, typename Body, typename End>
+__device__ __forceinline__ void for_nodes(int NN, Body body, End end) {
+  const int lanes = lanes_per_node(NN), lane = threadIdx.x & (lanes - 1), shift = __ffs(lanes) - 1;
+  for (int x0 = 0; x0 < NN * lanes; x0 += blockDim.x) {
+    const int v = (x0 + threadIdx.x) >> shift;
+    TA y[3] = {TA(0), TA(0), TA(0)};
+    if (v < NN) body(v, lane, lanes, y);
+    node_sum<TA>(y, lanes);
+    if (v < NN && lane == 0) end(v, y);
+  }
+}
+
+// this lane's share of y = K_l z at node v (zero at a pinned node)
+template <typename TA>
+__device__ __forceinline__ void mg3_apply(const Mg3Level<TA>& L, const TA* z, int v, int lane, int lanes, TA (&y)[3]) {
   const int n = L.n, NN = L.NN, i = v % n, j = (v / n) % n, k = v / (n * n);
-  y[0] = y[1] = y[2] = TA(0);
   if (pinned3(v, n, L.bc)) return;
-  for (int a = 0; a < 8; ++a) {
-    const int ei = (i - (a & 1) + n) % n, ej = (j - ((a >> 1) & 1) + n) % n, ek = (k - (a >> 2) + n) % n;
-    const int E = node3(n, ei, ej, ek);
+  const TA* st = L.st + v;
+#pragma unroll 3
+  for (int nb = lane; nb < 27; nb += lanes) {
+    const int nz = nb / 9, ny = nb / 3 - 3 * nz, nx = nb - 3 * (nb / 3);
+    const int u = node3(n, wrapped(i + nx - 1, n), wrapped(j + ny - 1, n), wrapped(k + nz - 1, n));
+    const TA z0 = z[u], z1 = z[NN + u], z2 = z[2 * NN + u];
+    const TA* m = st + (size_t)(nb * 9) * NN;
 #pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      const int nb = node3(n, (ei + (b & 1)) % n, (ej + ((b >> 1) & 1)) % n, (ek + (b >> 2)) % n);
-      const TA z0 = z[nb], z1 = z[NN + nb], z2 = z[2 * NN + nb];
-#pragma unroll
-      for (int ii = 0; ii < 3; ++ii)
-        y[ii] += mg3_kb<TA>(L, E, a, b, ii, 0) * z0 + mg3_kb<TA>(L, E, a, b, ii, 1) * z1 +
-                 mg3_kb<TA>(L, E, a, b, ii, 2) * z2;
-    }
+    for (int ii = 0; ii < 3; ++ii) y[ii] += m[(3 * ii) * NN] * z0 + m[(3 * ii + 1) * NN] * z1 + m[(3 * ii + 2) * NN] * z2;
   }
 }
 
@@ -1046,50 +1446,54 @@ __device__ __forceinline__ void mg3_smooth(const TA* mi, int NN, int v, const TA
   z[2] = om * (m02 * r[0] + m12 * r[1] + m22 * r[2]);
 }
 
-// Full-weighting restriction to coarse node I of grid nc of the fine residual t(v) = ta[v] -
-// tb[v] (tb may be null) on grid 2 nc; zero at the pinned node.  Stores r and, for a smoothing
-// level, the pre-smoothed z.
+// Full-weighting restriction to the nodes of level l of the fine residual t(v) = ta[v] - tb[v] (tb may be null)
+// on the grid twice as fine; zero at a pinned node.  Stores r and, for a smoothing level, the pre-smoothed z.
 template <typename TA>
-__device__ __forceinline__ void mg3_restrict_smooth(const Mg3<TA>& mg, int l, const TA* ta, const TA* tb, int I) {
+__device__ __forceinline__ void mg3_restrict_smooth(const Mg3<TA>& mg, int l, const TA* ta, const TA* tb) {
   const Mg3Level<TA> C = mg.level(l);
   const int nc = C.n, nf = 2 * nc, NNf = nf * nf * nf;
-  const int ci = I % nc, cj = (I / nc) % nc, ck = I / (nc * nc);
-  TA r[3] = {TA(0), TA(0), TA(0)};
-  if (!pinned3(I, nc, mg.bc)) {
-    for (int dz = -1; dz <= 1; ++dz)
-      for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-        for (int dx = -1; dx <= 1; ++dx) {
-          const TA w = TA((dx ? 0.5f : 1.0f) * (dy ? 0.5f : 1.0f) * (dz ? 0.5f : 1.0f));
-          const int f = node3(nf, (2 * ci + dx + nf) % nf, (2 * cj + dy + nf) % nf, (2 * ck + dz + nf) % nf);
+  for_nodes<TA>(
+      C.NN,
+      [&](int I, int lane, int lanes, TA(&r)[3]) {
+        if (pinned3(I, nc, mg.bc)) return;
+        const int ci = I % nc, cj = (I / nc) % nc, ck = I / (nc * nc);
+#pragma unroll 3
+        for (int nb = lane; nb < 27; nb += lanes) {
+          const int nz = nb / 9, ny = nb / 3 - 3 * nz, nx = nb - 3 * (nb / 3);
+          const TA w = (nx == 1 ? TA(1) : TA(0.5)) * (ny == 1 ? TA(1) : TA(0.5)) * (nz == 1 ? TA(1) : TA(0.5));
+          const int f = node3(nf, wrapped(2 * ci + nx - 1, nf), wrapped(2 * cj + ny - 1, nf), wrapped(2 * ck + nz - 1, nf));
 #pragma unroll
           for (int d = 0; d < 3; ++d) r[d] += w * (tb ? ta[d * NNf + f] - tb[d * NNf + f] : ta[d * NNf + f]);
         }
-  }
+      },
+      [&](int I, const TA(&r)[3]) {
 #pragma unroll
-  for (int d = 0; d < 3; ++d) C.r[d * C.NN + I] = r[d];
-  if (l < mg.levels) {
-    TA z[3];
-    mg3_smooth<TA>(C.mi, C.NN, I, r, mg.omega, z);
+        for (int d = 0; d < 3; ++d) C.r[d * C.NN + I] = r[d];
+        if (l < mg.levels) {
+          TA z[3];
+          mg3_smooth<TA>(C.mi, C.NN, I, r, mg.omega, z);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) C.z[d * C.NN + I] = z[d];
-  }
+          for (int d = 0; d < 3; ++d) C.z[d * C.NN + I] = z[d];
+        }
+      });
 }
 
-// Trilinear prolongation of the coarse vector zc (grid nf/2) to fine node v of grid nf.
+// Trilinear prolongation of the coarse vector zc (grid nf/2) to fine node (i, j, k) of grid nf: the mean of the
+// eight coarse nodes around it (the same node twice along an axis where it lies on one).
 template <typename TA>
-__device__ __forceinline__ void mg3_prolong(const TA* zc, int nf, int v, TA (&z)[3]) {
+__device__ __forceinline__ void mg3_prolong(const TA* zc, int nf, int i, int j, int k, TA (&z)[3]) {
   const int nc = nf >> 1, NNc = nc * nc * nc;
-  const int i = v % nf, j = (v / nf) % nf, k = v / (nf * nf);
+  const int x[2] = {i >> 1, wrapped((i + 1) >> 1, nc)}, y[2] = {j >> 1, wrapped((j + 1) >> 1, nc)},
+            w[2] = {k >> 1, wrapped((k + 1) >> 1, nc)};
   z[0] = z[1] = z[2] = TA(0);
-  for (int p = 0; p < 8; ++p) {
-    const int px = p & 1, py = (p >> 1) & 1, pz = p >> 2;
-    if ((px && !(i & 1)) || (py && !(j & 1)) || (pz && !(k & 1))) continue;
-    const TA w = TA(((i & 1) ? 0.5f : 1.0f) * ((j & 1) ? 0.5f : 1.0f) * ((k & 1) ? 0.5f : 1.0f));
-    const int c = node3(nc, ((i >> 1) + px) % nc, ((j >> 1) + py) % nc, ((k >> 1) + pz) % nc);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) z[d] += w * zc[d * NNc + c];
+  for (int p = 0; p < 8; ++p) {
+    const int c = node3(nc, x[p & 1], y[(p >> 1) & 1], w[p >> 2]);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) z[d] += zc[d * NNc + c];
   }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) z[d] *= TA(0.125);
 }
 
 // where the corrected z of level l ends: t of a smoothing level, z of the coarsest
@@ -1107,25 +1511,27 @@ __device__ __noinline__ void mg3_coarse_cycle(const Mg3<TA>& mg) {
   const TA om = mg.omega;
   for (int l = 1; l < mg.levels; ++l) {  // descend
     const Mg3Level<TA> v = mg.level(l);
-    for (int x = tid; x < v.NN; x += blockDim.x) {
-      TA kz[3];
-      mg3_apply<TA>(v, v.z, x, kz);
+    for_nodes<TA>(
+        v.NN, [&](int x, int lane, int lanes, TA(&y)[3]) { mg3_apply<TA>(v, v.z, x, lane, lanes, y); },
+        [&](int x, const TA(&kz)[3]) {
 #pragma unroll
-      for (int d = 0; d < 3; ++d) v.t[d * v.NN + x] = v.r[d * v.NN + x] - kz[d];
-    }
+          for (int d = 0; d < 3; ++d) v.t[d * v.NN + x] = v.r[d * v.NN + x] - kz[d];
+        });
     __syncthreads();
-    const Mg3Level<TA> cn = mg.level(l + 1);
-    for (int x = tid; x < cn.NN; x += blockDim.x) mg3_restrict_smooth<TA>(mg, l + 1, v.t, nullptr, x);
+    mg3_restrict_smooth<TA>(mg, l + 1, v.t, nullptr);
     __syncthreads();
   }
-  {  // coarsest: z = A^-1 r (rows of the pinned node: identity, z = 0 there)
+  {  // coarsest: z = A^-1 r (rows of the pinned node: identity, z = 0 there), several lanes per row
     const Mg3Level<TA> C = mg.level(mg.levels);
-    const int D = 3 * C.NN, ld = D + 1;
+    const int D = 3 * C.NN, ld = D + 1, lanes = D <= 32 ? 16 : 4, lane = tid & (lanes - 1);
     const TA* A = mg.inverse();
-    for (int row = tid; row < D; row += blockDim.x) {
+    for (int x0 = 0; x0 < D * lanes; x0 += blockDim.x) {
+      const int row = (x0 + tid) / lanes;
       TA zz = TA(0);
-      for (int q = 0; q < D; ++q) zz += A[(size_t)row * ld + q] * C.r[q];
-      C.z[row] = pinned3(row % C.NN, C.n, mg.bc) ? TA(0) : zz;
+      if (row < D)
+        for (int q = lane; q < D; q += lanes) zz += A[(size_t)row * ld + q] * C.r[q];
+      for (int o = lanes >> 1; o > 0; o >>= 1) zz += __shfl_xor_sync(0xffffffffu, zz, o);
+      if (row < D && lane == 0) C.z[row] = pinned3(row % C.NN, C.n, mg.bc) ? TA(0) : zz;
     }
     __syncthreads();
   }
@@ -1134,20 +1540,21 @@ __device__ __noinline__ void mg3_coarse_cycle(const Mg3<TA>& mg) {
     const TA* zc = mg3_result<TA>(mg, l + 1);
     for (int x = tid; x < v.NN; x += blockDim.x) {
       TA zp[3];
-      mg3_prolong<TA>(zc, v.n, x, zp);
+      mg3_prolong<TA>(zc, v.n, x % v.n, (x / v.n) % v.n, x / (v.n * v.n), zp);
 #pragma unroll
       for (int d = 0; d < 3; ++d) v.z[d * v.NN + x] += zp[d];
     }
     __syncthreads();
-    for (int x = tid; x < v.NN; x += blockDim.x) {
-      TA kz[3], rr[3], dz[3];
-      mg3_apply<TA>(v, v.z, x, kz);
+    for_nodes<TA>(
+        v.NN, [&](int x, int lane, int lanes, TA(&y)[3]) { mg3_apply<TA>(v, v.z, x, lane, lanes, y); },
+        [&](int x, const TA(&kz)[3]) {
+          TA rr[3], dz[3];
 #pragma unroll
-      for (int d = 0; d < 3; ++d) rr[d] = v.r[d * v.NN + x] - kz[d];
-      mg3_smooth<TA>(v.mi, v.NN, x, rr, om, dz);
+          for (int d = 0; d < 3; ++d) rr[d] = v.r[d * v.NN + x] - kz[d];
+          mg3_smooth<TA>(v.mi, v.NN, x, rr, om, dz);
 #pragma unroll
-      for (int d = 0; d < 3; ++d) v.t[d * v.NN + x] = v.z[d * v.NN + x] + dz[d];
-    }
+          for (int d = 0; d < 3; ++d) v.t[d * v.NN + x] = v.z[d * v.NN + x] + dz[d];
+        });
     __syncthreads();
   }
 }
@@ -1166,88 +1573,103 @@ __device__ __forceinline__ T div3(T a, T b) {
 template <typename TA, int LAW>
 __device__ __noinline__ void mg3_vcycle_fine(const Ctx3<TA>& c, const TA* r) {
   const Mg3<TA>& mg = c.mg;
-  const int NN = c.g.NN;
-  apply3<TA, LAW>(c, 0, 0);  // vout = K vin
-  const Mg3Level<TA> L1 = mg.level(1);
-  for (int I = threadIdx.x; I < L1.NN; I += blockDim.x) mg3_restrict_smooth<TA>(mg, 1, r, c.vout, I);
+  const int NN = c.g.NN, n = c.g.n;
+  TA* vin = smem_vin<TA>();
+  const TA* vout = vin + 3 * NN;
+  apply3<TA, LAW>(c);  // vout = K vin
+  mg3_restrict_smooth<TA>(mg, 1, r, vout);
   __syncthreads();
   mg3_coarse_cycle<TA>(mg);
   const TA* zc = mg3_result<TA>(mg, 1);
   for (int v = threadIdx.x; v < NN; v += blockDim.x) {
+    const int jk = div_n(v, c.magic), k = div_n(jk, c.magic);
     TA zp[3];
-    mg3_prolong<TA>(zc, c.g.n, v, zp);
+    mg3_prolong<TA>(zc, n, v - n * jk, jk - n * k, k, zp);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) c.vin[d * NN + v] += zp[d];
+    for (int d = 0; d < 3; ++d) vin[d * NN + v] += zp[d];
   }
   __syncthreads();
-  apply3<TA, LAW>(c, 0, 0);  // vout = K vin
+  apply3<TA, LAW>(c);  // vout = K vin
+#pragma unroll 2
   for (int v = threadIdx.x; v < NN; v += blockDim.x) {
     TA rr[3], dz[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) rr[d] = r[d * NN + v] - c.vout[d * NN + v];
+    for (int d = 0; d < 3; ++d) rr[d] = r[d * NN + v] - vout[d * NN + v];
     mg3_smooth<TA>(c.sc.mi, NN, v, rr, mg.omega, dz);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) c.vin[d * NN + v] += dz[d];
+    for (int d = 0; d < 3; ++d) vin[d * NN + v] += dz[d];
   }
   __syncthreads();
 }
 
 // Chronopoulos-Gear PCG for K x = b; b given in sc.r on entry (overwritten), x in sc.x.
+// One pass of the loop over the nodes updates p, s, x, r and smooths the new residual into vin (r, vin and vout
+// are in shared memory in mixed mode; p, s, x and the inverted blocks stream from the block's scratch).
 template <typename TA, int LAW>
 __device__ int pcg3(const Ctx3<TA>& c, TA rtol, int max_it, bool truncate, int* status, bool warm = false) {
   const int NN = c.g.NN;
-  TA* x = c.sc.x;
-  TA* r = c.sc.r;
-  TA* p = c.sc.p;
-  TA* s = c.sc.s;
-  const TA* mi = c.sc.mi;
-  auto precond_to_vin = [&]() {  // u = M^-1 r -> vin: block-Jacobi, or the multigrid V-cycle
-    const TA om = c.mg.levels ? c.mg.omega : TA(1);
+  TA* __restrict__ x = c.sc.x;
+  TA* __restrict__ p = c.sc.p;
+  TA* __restrict__ s = c.sc.s;
+  const TA* __restrict__ mi = c.sc.mi;
+  TA* vin = smem_vin<TA>();
+  const TA* vout = vin + 3 * NN;
+  TA* r = sizeof(TA) == 4 ? vin + 9 * NN : c.sc.r;
+  const TA om = c.mg.levels ? c.mg.omega : TA(1);
+  auto smooth_to_vin = [&]() {  // om M^-1 r (inverted nodal blocks)
+#pragma unroll 2
     for (int v = threadIdx.x; v < NN; v += blockDim.x) {
-      const TA r0 = r[v], r1 = r[NN + v], r2 = r[2 * NN + v];
-      const TA m00 = mi[v], m01 = mi[NN + v], m02 = mi[2 * NN + v], m11 = mi[3 * NN + v], m12 = mi[4 * NN + v],
-               m22 = mi[5 * NN + v];
-      c.vin[v] = om * (m00 * r0 + m01 * r1 + m02 * r2);
-      c.vin[NN + v] = om * (m01 * r0 + m11 * r1 + m12 * r2);
-      c.vin[2 * NN + v] = om * (m02 * r0 + m12 * r1 + m22 * r2);
+      const TA rr[3] = {r[v], r[NN + v], r[2 * NN + v]};
+      TA z[3];
+      mg3_smooth<TA>(mi, NN, v, rr, om, z);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) vin[d * NN + v] = z[d];
     }
+  };
+  auto precond_rest = [&]() {  // vin = om M^-1 r -> u = M^-1 r: block-Jacobi, or the multigrid V-cycle
     __syncthreads();
     if (c.mg.levels) mg3_vcycle_fine<TA, LAW>(c, r);
   };
   // inner products: per thread and per warp in TA, over the block in FP64 (block_dot2_fp64); the
-  // stopping test compares the FP64 sums, the step scalars are formed in TA from them
+  // stopping test compares FP64 sums, the step scalars are formed in TA from them
   auto dots = [&](double& gam, double& del) {
     TA g = TA(0), d = TA(0);
+#pragma unroll 4
     for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) {
-      g += r[v] * c.vin[v];
-      d += c.vout[v] * c.vin[v];
+      g += r[v] * vin[v];
+      d += vout[v] * vin[v];
     }
     block_dot2_fp64<TA>(g, d, c.red + 2 * 512 - 64, gam, del);
   };
   *status = kStatusOk;
   double gref = -1.0;  // stopping reference b^T M^-1 b of a warm start
   int it = 0;
+  smooth_to_vin();
   if (!warm) {
+#pragma unroll 4
     for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) x[v] = TA(0);
   } else {
     // x holds the start value x0 (the previous solve's solution): iterate on r = b - K x0 with
     // the stopping reference of b (one more preconditioner application and apply, counted)
-    precond_to_vin();
+    precond_rest();
     {
       TA g = TA(0);
-      for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) g += r[v] * c.vin[v];
+      for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) g += r[v] * vin[v];
       double unused;
       block_dot2_fp64<TA>(g, TA(0), c.red + 2 * 512 - 64, gref, unused);
     }
-    for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) c.vin[v] = x[v];
+#pragma unroll 4
+    for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) vin[v] = x[v];
     __syncthreads();
-    apply3<TA, LAW>(c, 0, 0);
-    for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) r[v] -= c.vout[v];
-    __syncthreads();
+    apply3<TA, LAW>(c);
+    for (int v = threadIdx.x; v < NN; v += blockDim.x)  // by nodes: smoothed by the same thread below
+#pragma unroll
+      for (int d = 0; d < 3; ++d) r[d * NN + v] -= vout[d * NN + v];
     it = 1;
+    smooth_to_vin();
   }
-  precond_to_vin();
-  apply3<TA, LAW>(c, 0, 0);
+  precond_rest();
+  apply3<TA, LAW>(c);
   double gd, dd;
   dots(gd, dd);
   TA gamma = (TA)gd, delta = (TA)dd;
@@ -1268,7 +1690,7 @@ __device__ int pcg3(const Ctx3<TA>& c, TA rtol, int max_it, bool truncate, int* 
   if (!(dd > 0.0)) {
     if (truncate && delta < TA(0)) {
       const TA a0 = div3(gamma, -delta);
-      for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) x[v] = a0 * c.vin[v];
+      for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) x[v] = a0 * vin[v];
       *status = kStatusNegCurv;
     } else {
       *status = kStatusPcgBreakdown;
@@ -1277,22 +1699,30 @@ __device__ int pcg3(const Ctx3<TA>& c, TA rtol, int max_it, bool truncate, int* 
     return 0;
   }
   TA alpha = div3(gamma, delta), beta = TA(0);
-  for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) {
-    p[v] = c.vin[v];
-    s[v] = c.vout[v];
-  }
-  for (;;) {
+  for (bool first = true;; first = false) {
     if (it >= max_it) {
       *status = kStatusPcgCap;
       break;
     }
-    for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) {
-      x[v] += alpha * p[v];
-      r[v] -= alpha * s[v];
+#pragma unroll 2
+    for (int v = threadIdx.x; v < NN; v += blockDim.x) {  // p = u + beta p, s = w + beta s, x += alpha p, r -= alpha s
+      TA rr[3], z[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const int q = d * NN + v;
+        const TA pq = first ? vin[q] : vin[q] + beta * p[q], sq = first ? vout[q] : vout[q] + beta * s[q];
+        p[q] = pq;
+        s[q] = sq;
+        x[q] += alpha * pq;
+        rr[d] = r[q] - alpha * sq;
+        r[q] = rr[d];
+      }
+      mg3_smooth<TA>(mi, NN, v, rr, om, z);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) vin[d * NN + v] = z[d];
     }
-    __syncthreads();
-    precond_to_vin();
-    apply3<TA, LAW>(c, 0, 0);
+    precond_rest();
+    apply3<TA, LAW>(c);
     double gnd, dnd;
     dots(gnd, dnd);
     const TA gn = (TA)gnd, dn = (TA)dnd;
@@ -1310,11 +1740,6 @@ __device__ int pcg3(const Ctx3<TA>& c, TA rtol, int max_it, bool truncate, int* 
     }
     alpha = div3(gn, den);
     gamma = gn;
-    for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) {
-      p[v] = c.vin[v] + beta * p[v];
-      s[v] = c.vout[v] + beta * s[v];
-    }
-    __syncthreads();
   }
   __syncthreads();
   return it;
@@ -1330,24 +1755,41 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
   c.g.NN = NN;
   c.NE = NN;
   c.phase = a.phase + a.rve_phase_off[rv];
-  c.vin = reinterpret_cast<TA*>(smem);
-  c.vout = c.vin + 3 * NN;
-  c.red = reinterpret_cast<double*>(smem + sizeof(TA) * 6 * (size_t)a.nn_max);
+  c.red = reinterpret_cast<double*>(smem);
   double* lame_s = c.red + 2 * 512;
   double* misc = lame_s + 2 * kMaxPhase;
   c.lame = lame_s;
+  TA* lame_t = reinterpret_cast<TA*>(smem + kSmem3LameT);
+  c.lame_t = lame_t;
+  c.Fb_t = lame_t + 2 * kMaxPhase;
+  c.vin = reinterpret_cast<TA*>(smem + kSmem3Fixed);
+  c.vout = c.vin + 3 * NN;
+  c.w32 = nullptr;
+  c.magic = (65536 + n - 1) / n;
   c.sc = scratch3_layout<TA>(gscr, NN);
+  c.mg.vec = nullptr;
+  if (sizeof(TA) == 4) {  // mixed: the FP32 fluctuation, the residual and the coarse vectors in shared memory too
+    c.w32 = c.vout + 3 * NN;
+    c.sc.r = c.w32 + 3 * NN;
+    c.mg.vec = c.sc.r + 3 * NN;
+  }
   c.mg.levels = a.mg ? mg3_levels(n) : 0;
   c.mg.n = n;
   c.mg.bc = a.bc;
   c.mg.omega = (TA)a.mg_omega;
   c.bc = a.bc;
   c.mg.base = c.sc.mg;
-  if (threadIdx.x < 2 * kMaxPhase) lame_s[threadIdx.x] = a.rve_lame[(size_t)rv * 2 * kMaxPhase + threadIdx.x];
+  if (threadIdx.x < 2 * kMaxPhase) {
+    const double v = a.rve_lame[(size_t)rv * 2 * kMaxPhase + threadIdx.x];
+    lame_s[threadIdx.x] = v;
+    lame_t[threadIdx.x] = (TA)v;
+  }
 #pragma unroll
   for (int k = 0; k < 9; ++k) c.Fb[k] = a.F[(size_t)qp * 9 + k];
+  if (threadIdx.x < 9) c.Fb_t[threadIdx.x] = (TA)a.F[(size_t)qp * 9 + threadIdx.x];
   const double* w_in = a.w_in + a.qp_w_off[qp];
   double* w = a.w_out + a.qp_w_off[qp];
+  c.w = w;
   // the current fluctuation is kept in w_out (FP64, global); node 0 pinned to zero
   for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) w[v] = pinned3(v / 3, n, a.bc) ? 0.0 : w_in[v];
   __syncthreads();
@@ -1365,7 +1807,7 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
       double bad = 0.0;
 #pragma unroll
       for (int k = 0; k < 9; ++k) Psum[k] = 0.0;
-      residual3<TA, LAW>(c, w, Psum, bad);
+      residual3<TA, LAW>(c, Psum, bad);
       __syncthreads();
       double rr = 0.0;
       for (int v = threadIdx.x; v < NN; v += blockDim.x) {
@@ -1473,6 +1915,9 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
 #pragma unroll
     for (int k = 0; k < 9; ++k)
       c.Fb[k] = stage == stages ? Ft[k] : (k % 4 == 0 ? 1.0 : 0.0) + (Ft[k] - (k % 4 == 0 ? 1.0 : 0.0)) * stage / stages;
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int k = 0; k < 9; ++k) c.Fb_t[k] = (TA)c.Fb[k];
     __syncthreads();
   }
   const int it = it_total;
@@ -1503,7 +1948,7 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
     for (int part = 0; part < 3; ++part) block_sum_n<double>(As + 15 * part, 15, c.red);
     // right-hand sides L_c (c = 3k + L) stored [c][3][NN]
     for (int cc = 0; cc < 9; ++cc) {
-      apply3<TA, LAW>(c, 1, cc);
+      unit_gradient3<TA, LAW>(c, cc);
       for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) c.sc.L[(size_t)cc * 3 * NN + v] = c.vout[v];
     }
     __syncthreads();
@@ -1583,7 +2028,6 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
 
 template <typename TA, int LAW>
 __global__ void __launch_bounds__(kThreads3D, 1) rve3d_kernel(const Rve2dArgs a) {
-  extern __shared__ __align__(16) unsigned char smem3[];
   __shared__ int s_item;
   unsigned char* gscr = reinterpret_cast<unsigned char*>(a.scratch) + (size_t)blockIdx.x * scratch3_bytes<TA>(a.nn_max);
   for (;;) {
@@ -1592,7 +2036,9 @@ __global__ void __launch_bounds__(kThreads3D, 1) rve3d_kernel(const Rve2dArgs a)
     const int item = s_item;
     __syncthreads();
     if (item >= (a.n_dev ? *a.n_dev : a.n_qp)) break;
-    solve_item_3d<TA, LAW>(a, a.order[item], smem3, gscr);
+    const int qp = a.order[item];
+    if (a.only_n && a.rve_n[a.qp_rve[qp]] != a.only_n) continue;  // another launch's grid
+    solve_item_3d<TA, LAW>(a, qp, smem3, gscr);
   }
 }
 
@@ -1606,22 +2052,31 @@ size_t rve3d_scratch_bytes(int nn_max, bool mixed, int n_blocks) {
   return (mixed ? scratch3_bytes<float>(nn_max) : scratch3_bytes<double>(nn_max)) * (size_t)n_blocks;
 }
 
+// Blocks of RVEs with nn nodes on one SM: two of 256 threads where there are more RVEs than SMs and the shared
+// memory holds both (n <= 12 in mixed precision), so that one works while the other waits at a barrier or runs its
+// FP64 residual; one of 512 otherwise (one RVE alone is 1.3 times faster with it).  304 RVEs of 8^3: 17.2 ms with
+// one, 13.4 with two, 16.5 with four of 128 threads; 200: 15.9, 12.9, 16.5; 304 of 12^3: 55.0, 48.6.
+int rve3d_blocks_per_sm(int nn, bool mixed, int count, int num_sms) {
+  return mixed && count > num_sms && 2 * (rve3d_smem_bytes(nn, true) + 1024) <= 228 * 1024 ? 2 : 1;
+}
+
 template <typename TA, int LAW>
-cudaError_t rve3d_launch_instance(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream) {
+cudaError_t rve3d_launch_instance(const Rve2dArgs& a, int n_blocks, int threads, size_t smem, cudaStream_t stream) {
   const cudaError_t err =
       cudaFuncSetAttribute(rve3d_kernel<TA, LAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  rve3d_kernel<TA, LAW><<<n_blocks, kThreads3D, smem, stream>>>(a);
+  rve3d_kernel<TA, LAW><<<n_blocks, threads, smem, stream>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t rve3d_launch(const Rve2dArgs& a, bool mixed, int n_blocks, cudaStream_t stream) {
+cudaError_t rve3d_launch(const Rve2dArgs& a, bool mixed, int n_blocks, int per_sm, cudaStream_t stream) {
+  const int threads = kThreads3D / per_sm;
   const size_t smem = rve3d_smem_bytes(a.nn_max, mixed);
   if (mixed)
-    return a.law == kLawSVK ? rve3d_launch_instance<float, kLawSVK>(a, n_blocks, smem, stream)
-                            : rve3d_launch_instance<float, kLawNH>(a, n_blocks, smem, stream);
-  return a.law == kLawSVK ? rve3d_launch_instance<double, kLawSVK>(a, n_blocks, smem, stream)
-                          : rve3d_launch_instance<double, kLawNH>(a, n_blocks, smem, stream);
+    return a.law == kLawSVK ? rve3d_launch_instance<float, kLawSVK>(a, n_blocks, threads, smem, stream)
+                            : rve3d_launch_instance<float, kLawNH>(a, n_blocks, threads, smem, stream);
+  return a.law == kLawSVK ? rve3d_launch_instance<double, kLawSVK>(a, n_blocks, threads, smem, stream)
+                          : rve3d_launch_instance<double, kLawNH>(a, n_blocks, threads, smem, stream);
 }
 
 }  // namespace fehmm

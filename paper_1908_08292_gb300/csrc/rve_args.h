@@ -34,7 +34,7 @@ struct Rve2dArgs {
   int mg;                // 1: multigrid-preconditioned PCG where the grid allows it (2D)
   long long scratch_stride;  // per-block scratch, in elements of the kernel's arithmetic type (2D)
   const int32_t* n_dev;  // optional: number of work items in device memory (order = a qp list)
-  int only_n;            // 2D: solve only the items of this grid size (0: every item)
+  int only_n;            // solve only the items of this grid size (0: every item)
   int fixed_n;        // fixed-layout launches only: grid size of every RVE
   int phase_per_qp;   // fixed-layout launches only: 1 = one phase map per qp, 0 = one shared
   int bc;             // 0 periodic (node 0 pinned), 1 KUBC (nodes on the planes x_c = 0 pinned)
@@ -54,7 +54,8 @@ cudaError_t rve2d_launch(const Rve2dArgs& a, bool mixed, int n_blocks, cudaStrea
 cudaError_t rve2d_launch_fixed_fp64(const Rve2dArgs& a, int n_blocks, cudaStream_t stream);
 size_t rve3d_smem_bytes(int nn_max, bool mixed);
 size_t rve3d_scratch_bytes(int nn_max, bool mixed, int n_blocks);
-cudaError_t rve3d_launch(const Rve2dArgs& a, bool mixed, int n_blocks, cudaStream_t stream);
+int rve3d_blocks_per_sm(int nn, bool mixed, int count, int num_sms);
+cudaError_t rve3d_launch(const Rve2dArgs& a, bool mixed, int n_blocks, int per_sm, cudaStream_t stream);
 
 struct MacroArgs {
   int dim;
