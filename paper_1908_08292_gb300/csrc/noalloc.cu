@@ -5,8 +5,8 @@
 // (a host that hands the library only pre-registered buffers), code paths that must not
 // allocate while a memory pool is being torn down or resized, and callers that need a
 // predictable footprint fixed at load time.  For them this entry point uses no dynamic
-// device memory at all: the per-block scratch the FP64 kernel needs (staged element
-// tangents and the assembled stencil) and its work counter live in file-scope
+// device memory at all: the per-block scratch the FP64 kernel is given (staged element
+// tangents; room for the stencil of the grids that do not hold it in registers) and its work counter live in file-scope
 // `static __device__` arrays of a fixed maximum size.  Every GPU on which the library is
 // loaded holds that memory (kNoallocScratchBytes, about 22 MB) until the process exits.
 //
@@ -27,7 +27,7 @@ namespace fehmm {
 namespace {
 
 constexpr int kNoallocMaxNN = 256;      // grid_n <= 16
-constexpr int kNoallocMaxBlocks = 152;  // one block per SM on a GB300, at most
+constexpr int kNoallocMaxBlocks = 152;  // blocks of the largest grid; smaller grids get as many as fit
 constexpr size_t kNoallocScratchDoubles = (size_t)kNoallocMaxBlocks * 72 * kNoallocMaxNN;
 constexpr int kMaxDevices = 64;
 

@@ -1,7 +1,7 @@
 // Host side of the 2D batched periodic-RVE solver: shared-memory and scratch sizes and the
 // dispatch to the kernel instantiations.  Each instantiation is compiled in a translation unit
 // of its own (rve2d_k_*.cu) so that the builds run in parallel; the device code is rve2d.cuh.
-#include "rve2d.cuh"
+#include "rve2d_fp64.cuh"
 
 #include <algorithm>
 
@@ -13,20 +13,19 @@ cudaError_t rve2d_launch_mixed_mg_svk(const Rve2dArgs& a, int n_blocks, size_t s
 cudaError_t rve2d_launch_mixed_mg_svk_small(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream);
 cudaError_t rve2d_launch_mixed_bj_nh(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream);
 cudaError_t rve2d_launch_mixed_bj_svk(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream);
-cudaError_t rve2d_launch_fp64_mg_nh(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream);
-cudaError_t rve2d_launch_fp64_mg_svk(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream);
-cudaError_t rve2d_launch_fp64_bj_nh(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream);
-cudaError_t rve2d_launch_fp64_bj_svk(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream);
-cudaError_t rve2d_launch_fp64_fixed_nh(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream);
+cudaError_t rve2d_launch_fp64_mg_nh(const Rve2dArgs& a, int n_blocks, cudaStream_t stream);
+cudaError_t rve2d_launch_fp64_mg_svk(const Rve2dArgs& a, int n_blocks, cudaStream_t stream);
+cudaError_t rve2d_launch_fp64_bj_nh(const Rve2dArgs& a, int n_blocks, cudaStream_t stream);
+cudaError_t rve2d_launch_fp64_bj_svk(const Rve2dArgs& a, int n_blocks, cudaStream_t stream);
+cudaError_t rve2d_launch_fp64_fixed_nh(const Rve2dArgs& a, int n_blocks, cudaStream_t stream);
 
 size_t rve2d_smem_bytes(int nn_max, bool mixed) {
-  return mixed ? offsets2d<float>(nn_max).total : offsets2d<double>(nn_max).total;
+  return mixed ? offsets2d<float>(nn_max).total : offsets_d2(nn_max, true).total;
 }
 
 long long rve2d_scratch_stride(int nn_max, bool mixed) {
-  // mixed: staged element tangents [36][nn_max] and the coarse element matrices of the multigrid;
-  // FP64: stencil and staged tangents [72][nn_max], then the whole multigrid
-  return mixed ? 36LL * nn_max + mg_slow_max(nn_max) : 72LL * nn_max + mg_fast_max(nn_max) + mg_slow_max(nn_max);
+  // mixed: staged element tangents [36][nn_max] and the coarse element matrices of the multigrid
+  return mixed ? 36LL * nn_max + mg_slow_max(nn_max) : scratch_d2(nn_max, true);
 }
 
 size_t rve2d_scratch_bytes(int nn_max, bool mixed, int n_blocks) {
@@ -36,7 +35,7 @@ size_t rve2d_scratch_bytes(int nn_max, bool mixed, int n_blocks) {
 // Blocks of RVEs with nn nodes that one SM holds: 128 registers per thread, the shared memory of the
 // layout plus 1 KB the driver takes per block.
 int rve2d_blocks_per_sm(int nn, bool mixed) {
-  const int regs = 65536 / (128 * (mixed ? threads2d<float>(nn) : threads2d<double>(nn)));
+  const int regs = 65536 / (128 * (mixed ? threads2d<float>(nn) : threads_d2(nn)));
   const int smem = (int)((228 * 1024) / (rve2d_smem_bytes(nn, mixed) + 1024));
   return std::max(1, std::min(regs, smem));
 }
@@ -56,12 +55,12 @@ cudaError_t rve2d_launch(const Rve2dArgs& a, bool mixed, int n_blocks, cudaStrea
     if (mg) return svk ? rve2d_launch_mixed_mg_svk(a, n_blocks, smem, stream) : rve2d_launch_mixed_mg_nh(a, n_blocks, smem, stream);
     return svk ? rve2d_launch_mixed_bj_svk(a, n_blocks, smem, stream) : rve2d_launch_mixed_bj_nh(a, n_blocks, smem, stream);
   }
-  if (mg) return svk ? rve2d_launch_fp64_mg_svk(a, n_blocks, smem, stream) : rve2d_launch_fp64_mg_nh(a, n_blocks, smem, stream);
-  return svk ? rve2d_launch_fp64_bj_svk(a, n_blocks, smem, stream) : rve2d_launch_fp64_bj_nh(a, n_blocks, smem, stream);
+  if (mg) return svk ? rve2d_launch_fp64_mg_svk(a, n_blocks, stream) : rve2d_launch_fp64_mg_nh(a, n_blocks, stream);
+  return svk ? rve2d_launch_fp64_bj_svk(a, n_blocks, stream) : rve2d_launch_fp64_bj_nh(a, n_blocks, stream);
 }
 
 cudaError_t rve2d_launch_fixed_fp64(const Rve2dArgs& a, int n_blocks, cudaStream_t stream) {
-  return rve2d_launch_fp64_fixed_nh(a, n_blocks, rve2d_smem_bytes(a.nn_max, false), stream);
+  return rve2d_launch_fp64_fixed_nh(a, n_blocks, stream);
 }
 
 }  // namespace fehmm

@@ -22,12 +22,12 @@
 //    about 1100 cycles a phase.  4096 RVEs of 32 x 32: 31.2 -> 24.5 ms; 1000 of 16 x 16 2.54 -> 1.59 ms.
 //  * w (FP64) lives in shared memory; the residual is evaluated per element in FP64 and the
 //    element forces are staged in shared memory, then gathered per node (no atomics).
-//  * Mixed precision (TA = float): element tangents are staged in the block's global scratch
+//  * FP32 tangents and solves (TA = float): element tangents are staged in the block's global scratch
 //    (L2 resident) and the assembled 9-point block stencil of each owned node (9 x 2x2 floats)
 //    is gathered into REGISTERS, where it stays for the whole PCG; the PCG exchanges only the
 //    search direction through shared memory, which also holds the multigrid's coarse levels
-//    (kept over the Newton iterations of a solve).  FP64 mode (TA = double) keeps the staged element
-//    tangents and the stencil in a per-block global scratch area (L2 resident).
+//    (kept over the Newton iterations of a solve).  FP64 mode has a thread layout of its own
+//    (rve2d_fp64.cuh) and shares the grid, law and multigrid definitions of this file.
 //  * Preconditioner: geometric multigrid V(1,1)-cycle with Galerkin coarse levels (grids
 //    n = 2^k m, m <= 4; a separate kernel instantiation), else block-Jacobi (inverted 2x2
 //    nodal diagonal blocks).
@@ -38,8 +38,6 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
-
-#include <type_traits>
 
 #include "fehmm_device.cuh"
 #include "rve_args.h"
@@ -52,8 +50,8 @@ constexpr int kThreads2D = 512;  // largest block: n = 32
 // Threads of a block that solves RVEs of n^2 = nn nodes: one per node pair, whole warps, and as many
 // such blocks on an SM as its registers hold.  (With 512 threads for every grid the idle warps of a small
 // one took part in every barrier and executed the vector operations on zeros.)  At least four warps: the
-// dense coarsest level spreads over them, and in FP64 each of the SM's four sub-partitions has a quarter of
-// its FP64 rate (8 x 8, 64 points, FP64: 3.63 ms with one warp, 2.64 ms with four, 3.41 ms with 16).
+// dense coarsest level spreads over them, and the FP64 residual over the SM's four sub-partitions, each of
+// which has a quarter of its FP64 rate.
 template <typename TA>
 __host__ __device__ constexpr int threads2d(int nn) {
   const int t = (nn / 2 + 31) / 32 * 32;
@@ -121,12 +119,7 @@ __host__ __device__ constexpr long long mg_slow_elems(int n) {
   for (int l = 1; l <= L; ++l) e += 36LL * (n >> l) * (n >> l);
   return e;
 }
-// Largest region sizes over the grids a batch with n^2 <= nn_max may hold.
-__host__ __device__ constexpr long long mg_fast_max(int nn_max) {
-  long long m = 0;
-  for (int n = 2; n * n <= nn_max; n += 2) m = mg_fast_elems(n) > m ? mg_fast_elems(n) : m;
-  return m;
-}
+// Largest region size over the grids a batch with n^2 <= nn_max may hold.
 __host__ __device__ constexpr long long mg_slow_max(int nn_max) {
   long long m = 0;
   for (int n = 2; n * n <= nn_max; n += 2) m = mg_slow_elems(n) > m ? mg_slow_elems(n) : m;
@@ -136,7 +129,7 @@ __host__ __device__ constexpr long long mg_slow_max(int nn_max) {
 template <typename TA>
 struct Smem2D {
   double2* w;        // [NN] fluctuation (FP64)
-  float2* w32;       // [NN] FP32 copy (mixed mode only)
+  float2* w32;       // [NN] FP32 copy
   vec2_t<TA>* p;     // [2][NN] PCG exchange vector (u = M^-1 r), two alternating buffers
   vec2_t<TA>* x;     // [NN] PCG solution (owned nodes written by their thread)
   unsigned char* stage;  // element forces / element tangents / condensation solutions
@@ -154,7 +147,6 @@ struct Offsets2D {
 
 template <typename TA>
 __host__ __device__ constexpr Offsets2D offsets2d(int NN) {
-  constexpr bool REG = std::is_same<TA, float>::value;
   Offsets2D o{};
   size_t off = 0;
   const auto take = [&off](size_t bytes) {
@@ -163,18 +155,17 @@ __host__ __device__ constexpr Offsets2D offsets2d(int NN) {
     return at;
   };
   o.w = take(sizeof(double2) * NN);
-  o.w32 = REG ? take(sizeof(float2) * NN) : 0;
+  o.w32 = take(sizeof(float2) * NN);
   o.p = take(2 * sizeof(vec2_t<TA>) * NN);
   o.x = take(sizeof(vec2_t<TA>) * NN);
   size_t stage_bytes = sizeof(double) * 8 * NN;                               // element forces
-  // condensation solutions X[4][NN] and right-hand sides L[4][NN]; in mixed mode followed by
+  // condensation solutions X[4][NN] and right-hand sides L[4][NN]; followed by
   // the multigrid fast region of the RVE's grid (largest over the grids up to NN)
   if (sizeof(vec2_t<TA>) * 8 * NN > stage_bytes) stage_bytes = sizeof(vec2_t<TA>) * 8 * NN;
-  if (REG)
-    for (int m = 2; m * m <= NN; m += 2) {
-      const size_t need = sizeof(vec2_t<TA>) * 8 * (size_t)m * m + sizeof(TA) * (size_t)mg_fast_elems(m);
-      if (need > stage_bytes) stage_bytes = need;
-    }
+  for (int m = 2; m * m <= NN; m += 2) {
+    const size_t need = sizeof(vec2_t<TA>) * 8 * (size_t)m * m + sizeof(TA) * (size_t)mg_fast_elems(m);
+    if (need > stage_bytes) stage_bytes = need;
+  }
   o.stage = take(stage_bytes);
   o.red_n = 10 * (threads2d<TA>(NN) / 32);  // block_sum of up to 10 values
   o.red = take(sizeof(double) * (2 * o.red_n + 34));
@@ -188,7 +179,7 @@ template <typename TA>
 __device__ __forceinline__ Smem2D<TA> smem2d(const Offsets2D& o, unsigned char* base) {
   Smem2D<TA> s;
   s.w = reinterpret_cast<double2*>(base + o.w);
-  s.w32 = std::is_same<TA, float>::value ? reinterpret_cast<float2*>(base + o.w32) : nullptr;
+  s.w32 = reinterpret_cast<float2*>(base + o.w32);
   s.p = reinterpret_cast<vec2_t<TA>*>(base + o.p);
   s.x = reinterpret_cast<vec2_t<TA>*>(base + o.x);
   s.stage = base + o.stage;
@@ -237,15 +228,10 @@ __device__ __forceinline__ Own2D make_own(int n, int bc) {
   return o;
 }
 
-// Stencil storage.  REG (FP32): registers, block nb of owned node s as two row pairs
-// K2[s][nb][0] = (K_xx, K_xy), K2[s][nb][1] = (K_yx, K_yy), consumed by paired FP32 FMAs
-// (FFMA2).  Otherwise (FP64): global scratch [36][NN] in row-major block order.
-template <typename TA, bool REG>
+// Stencil of the owned node pair, in registers: block nb of owned node s as two row pairs
+// K2[s][nb][0] = (K_xx, K_xy), K2[s][nb][1] = (K_yx, K_yy), consumed by paired FP32 FMAs (FFMA2).
 struct Stencil {
   float2 K2[2][9][2];
-  TA* g;  // global stencil base (FP64 mode)
-  int NN;
-  __device__ __forceinline__ TA get(int nb, int c, int node) const { return g[(size_t)(nb * 4 + c) * NN + node]; }
 };
 
 // ------------------------------------------------------------------ constitutive laws (2D)
@@ -538,89 +524,45 @@ __device__ __forceinline__ void gather_stencil(int node, int n, const TA* stage_
 // y = K p for the owned node pair; p of neighbours from shared memory.  The four
 // neighbour rows (2s-1 .. 2s+2) are streamed one at a time: row r feeds the lower node
 // (row offset r-1) and the upper node (row offset r-2), so only one row is live.
-template <typename TA, bool REG>
-__device__ __forceinline__ void apply_pair(const Stencil<TA, REG>& S, const Own2D& o, const vec2_t<TA>* ps,
-                                           const TA (&pown)[4], TA (&y)[4]) {
-  if constexpr (REG) {
-    // acc[s][i] accumulates (K_i0 p_x, K_i1 p_y) pairs; y_i = acc.x + acc.y at the end
-    float2 acc[2][2] = {{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}};
+__device__ __forceinline__ void apply_pair(const Stencil& S, const Own2D& o, const float2* ps, const float (&pown)[4],
+                                           float (&y)[4]) {
+  // acc[s][i] accumulates (K_i0 p_x, K_i1 p_y) pairs; y_i = acc.x + acc.y at the end
+  float2 acc[2][2] = {{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}};
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      float2 P[3];
+  for (int r = 0; r < 4; ++r) {
+    float2 P[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        if (c == 1 && r == 1) {
-          P[c] = make_float2(pown[0], pown[1]);
-        } else if (c == 1 && r == 2) {
-          P[c] = make_float2(pown[2], pown[3]);
-        } else {
-          P[c] = ps[o.rows[r] + o.cols[c]];
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        if (r <= 2) {
-          const int nb = r * 3 + c;
-          acc[0][0] = __ffma2_rn(S.K2[0][nb][0], P[c], acc[0][0]);
-          acc[0][1] = __ffma2_rn(S.K2[0][nb][1], P[c], acc[0][1]);
-        }
-        if (r >= 1) {
-          const int nb = (r - 1) * 3 + c;
-          acc[1][0] = __ffma2_rn(S.K2[1][nb][0], P[c], acc[1][0]);
-          acc[1][1] = __ffma2_rn(S.K2[1][nb][1], P[c], acc[1][1]);
-        }
+    for (int c = 0; c < 3; ++c) {
+      if (c == 1 && r == 1) {
+        P[c] = make_float2(pown[0], pown[1]);
+      } else if (c == 1 && r == 2) {
+        P[c] = make_float2(pown[2], pown[3]);
+      } else {
+        P[c] = ps[o.rows[r] + o.cols[c]];
       }
     }
-    y[0] = acc[0][0].x + acc[0][0].y;
-    y[1] = acc[0][1].x + acc[0][1].y;
-    y[2] = acc[1][0].x + acc[1][0].y;
-    y[3] = acc[1][1].x + acc[1][1].y;
-  } else {
-    TA y0x = TA(0), y0y = TA(0), y1x = TA(0), y1y = TA(0);
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      vec2_t<TA> P[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        if (c == 1 && r == 1) {
-          P[c] = mk2<TA>(pown[0], pown[1]);
-        } else if (c == 1 && r == 2) {
-          P[c] = mk2<TA>(pown[2], pown[3]);
-        } else {
-          P[c] = ps[o.rows[r] + o.cols[c]];
-        }
+    for (int c = 0; c < 3; ++c) {
+      if (r <= 2) {
+        const int nb = r * 3 + c;
+        acc[0][0] = __ffma2_rn(S.K2[0][nb][0], P[c], acc[0][0]);
+        acc[0][1] = __ffma2_rn(S.K2[0][nb][1], P[c], acc[0][1]);
       }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        if (r <= 2) {
-          const int nb = r * 3 + c;
-          y0x += S.get(nb, 0, o.node[0]) * P[c].x + S.get(nb, 1, o.node[0]) * P[c].y;
-          y0y += S.get(nb, 2, o.node[0]) * P[c].x + S.get(nb, 3, o.node[0]) * P[c].y;
-        }
-        if (r >= 1) {
-          const int nb = (r - 1) * 3 + c;
-          y1x += S.get(nb, 0, o.node[1]) * P[c].x + S.get(nb, 1, o.node[1]) * P[c].y;
-          y1y += S.get(nb, 2, o.node[1]) * P[c].x + S.get(nb, 3, o.node[1]) * P[c].y;
-        }
+      if (r >= 1) {
+        const int nb = (r - 1) * 3 + c;
+        acc[1][0] = __ffma2_rn(S.K2[1][nb][0], P[c], acc[1][0]);
+        acc[1][1] = __ffma2_rn(S.K2[1][nb][1], P[c], acc[1][1]);
       }
     }
-    y[0] = y0x;
-    y[1] = y0y;
-    y[2] = y1x;
-    y[3] = y1y;
   }
+  y[0] = acc[0][0].x + acc[0][0].y;
+  y[1] = acc[0][1].x + acc[0][1].y;
+  y[2] = acc[1][0].x + acc[1][0].y;
+  y[3] = acc[1][1].x + acc[1][1].y;
 }
 
-// Quotient for the CG step scalars: fast reciprocal-based division in FP32 (a few ulp,
-// irrelevant for the step lengths), IEEE division in FP64 mode.
-template <typename T>
-__device__ __forceinline__ T cg_div(T a, T b) {
-  if constexpr (sizeof(T) == 4) {
-    return __fdividef(a, b);
-  } else {
-    return a / b;
-  }
-}
+// Quotient for the CG step scalars: fast reciprocal-based division (a few ulp, irrelevant for the step lengths).
+__device__ __forceinline__ float cg_div(float a, float b) { return __fdividef(a, b); }
 
 template <typename TA>
 __device__ __forceinline__ void invert_block(const TA (&Kself)[4], bool pinned, TA (&Mi)[4]) {
@@ -647,7 +589,7 @@ __device__ __forceinline__ void invert_block(const TA (&Kself)[4], bool pinned, 
 //    preconditioner for CG).  Coarsest level (at most 16 nodes, 32 dofs): exact, through its
 //    dense inverse, computed by Gauss-Jordan elimination in one warp.
 //  * Fine level: the stencil of the PCG.  Coarse levels: stencil, inverted blocks and vectors
-//    in the fast region (shared memory in mixed mode, block scratch in FP64 mode); coarse
+//    in the fast region (shared memory; in FP64 mode block scratch above 24 x 24); coarse
 //    element matrices (needed only while building) in the block's global scratch.
 template <typename TA>
 struct alignas(16) Block2 {
@@ -1020,8 +962,8 @@ __device__ __forceinline__ void mg_coarse_cycle(const MgCtx<TA>& mg) {
 // warm: xs holds a start value x0 at the owned nodes (the previous solve's solution); the
 // iteration runs on r = b - K x0 and stops at the same rtol relative to b^T M^-1 b as a start
 // from zero (one more preconditioner application and apply, counted as one iteration).
-template <typename TA, bool REG, bool kMG>
-__device__ __forceinline__ int pcg_pair(const Stencil<TA, REG>& S, const Own2D& o, const TA (&Minv)[2][4],
+template <typename TA, bool kMG>
+__device__ __forceinline__ int pcg_pair(const Stencil& S, const Own2D& o, const TA (&Minv)[2][4],
                                         const MgCtx<TA>& mg, const TA (&b)[4],
                         vec2_t<TA>* xs, TA rtol, int max_it, vec2_t<TA>* ps, double* red, int* status,
                         bool truncate, bool warm = false) {
@@ -1064,7 +1006,7 @@ __device__ __forceinline__ int pcg_pair(const Stencil<TA, REG>& S, const Own2D& 
     }
     __syncthreads();
     if (o.active) {
-      apply_pair<TA, REG>(S, o, pbuf, u, w);
+      apply_pair(S, o, pbuf, u, w);
       if (o.pin[0]) w[0] = w[1] = TA(0);  // pinned nodes
       if (o.pin[1]) w[2] = w[3] = TA(0);
     } else {
@@ -1155,14 +1097,14 @@ __device__ __forceinline__ int pcg_pair(const Stencil<TA, REG>& S, const Own2D& 
   if (*status == kStatusOk && gamma0 > 0.0 && !(warm && gamma0 <= stop)) {
     if (!(dd > 0.0)) {
       if (truncate && delta < TA(0)) {
-        const TA a0 = cg_div<TA>(gamma, -delta);
+        const TA a0 = cg_div(gamma, -delta);
         x_axpy(a0, u);
         *status = kStatusNegCurv;
       } else {
         *status = kStatusPcgBreakdown;
       }
     } else {
-      TA alpha = cg_div<TA>(gamma, delta);
+      TA alpha = cg_div(gamma, delta);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         p[k] = u[k];
@@ -1188,13 +1130,13 @@ __device__ __forceinline__ int pcg_pair(const Stencil<TA, REG>& S, const Own2D& 
           break;
         }
         if (gnd <= stop) break;
-        const TA beta = cg_div<TA>(gn, gamma);
-        const TA den = dn - beta * cg_div<TA>(gn, alpha);  // p_new^T K p_new
+        const TA beta = cg_div(gn, gamma);
+        const TA den = dn - beta * cg_div(gn, alpha);  // p_new^T K p_new
         if (!(den > TA(0))) {
           *status = (truncate && den < TA(0)) ? kStatusNegCurv : kStatusPcgBreakdown;
           break;
         }
-        alpha = cg_div<TA>(gn, den);
+        alpha = cg_div(gn, den);
         gamma = gn;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -1216,25 +1158,19 @@ __device__ __forceinline__ int pcg_pair(const Stencil<TA, REG>& S, const Own2D& 
 // Minv (inverted nodal blocks, zero on idle threads and the pinned node) stays in
 // registers; with withL the condensation right-hand sides go to shared memory,
 // Lb[c][NN] = -L_c of each owned node.
-template <typename TA, bool REG, bool kMG, int LAW>
+template <typename TA, bool kMG, int LAW>
 __device__ __forceinline__ void build_tangent(const Own2D& o, const Smem2D<TA>& sm, TA* stage_k,
-                                              const TA (&Fb)[4], const uint8_t* phase, Stencil<TA, REG>& S,
+                                              const TA (&Fb)[4], const uint8_t* phase, Stencil& S,
                                               TA (&Minv)[2][4], bool withL, vec2_t<TA>* Lb, const MgCtx<TA>& mg,
                                               bool build_mg = true) {
   TA L[2][2][4];
   const int n = o.n, NN = o.NN;
-  const vec2_t<TA>* wsrc;
-  if constexpr (REG) {
-    wsrc = reinterpret_cast<const vec2_t<TA>*>(sm.w32);
-  } else {
-    wsrc = reinterpret_cast<const vec2_t<TA>*>(sm.w);
-  }
   if (o.active) {
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
       const int e = o.node[s];
       const int ph = phase[e];
-      element_tangent<TA, LAW>(e, n, wsrc, Fb, (TA)sm.lame[2 * ph], (TA)sm.lame[2 * ph + 1], stage_k, e, NN);
+      element_tangent<TA, LAW>(e, n, sm.w32, Fb, (TA)sm.lame[2 * ph], (TA)sm.lame[2 * ph + 1], stage_k, e, NN);
     }
   }
   __syncthreads();
@@ -1255,19 +1191,10 @@ __device__ __forceinline__ void build_tangent(const Own2D& o, const Smem2D<TA>& 
 #pragma unroll
         for (int c = 0; c < 4; ++c) Ln[a][c] = TA(0);
     }
-    if constexpr (REG) {
 #pragma unroll
-      for (int nb = 0; nb < 9; ++nb) {
-        S.K2[s][nb][0] = make_float2(Kn[nb][0], Kn[nb][1]);
-        S.K2[s][nb][1] = make_float2(Kn[nb][2], Kn[nb][3]);
-      }
-    } else {
-      if (o.active) {
-#pragma unroll
-        for (int nb = 0; nb < 9; ++nb)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) S.g[(size_t)(nb * 4 + c) * NN + o.node[s]] = Kn[nb][c];
-      }
+    for (int nb = 0; nb < 9; ++nb) {
+      S.K2[s][nb][0] = make_float2(Kn[nb][0], Kn[nb][1]);
+      S.K2[s][nb][1] = make_float2(Kn[nb][2], Kn[nb][3]);
     }
     TA self[4] = {Kn[4][0], Kn[4][1], Kn[4][2], Kn[4][3]};
     TA mi[4];
@@ -1281,7 +1208,7 @@ __device__ __forceinline__ void build_tangent(const Own2D& o, const Smem2D<TA>& 
         for (int c = 0; c < 4; ++c) L[s][a][c] = Ln[a][c];
     }
   }
-  __syncthreads();  // stage reads done; global stencil writes visible
+  __syncthreads();  // stage reads done
   if (o.active && withL) {
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
@@ -1391,33 +1318,19 @@ __device__ __forceinline__ void element_transfer(int e, int n, const vec2_t<TA>*
   for (int k = 0; k < 10; ++k) Q[k] += (double)q[k];
 }
 
-// kFixed: one grid size for the whole batch, arrays indexed arithmetically (qp -> RVE qp or 0,
-// fluctuation of qp at qp*2*n*n) instead of through the context's index tables.
 // N: the grid size of every item where it is known when compiling (0: read per item).
-template <typename TA, bool kFixed, bool kMG, int LAW, int N>
-__device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const Smem2D<TA>& sm, TA* gscr) {
-  constexpr bool REG = std::is_same<TA, float>::value;
+template <typename TA, bool kMG, int LAW, int N>
+__device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const Smem2D<TA>& sm) {
   const int tid = threadIdx.x;
-  const int rv = kFixed ? (a.phase_per_qp ? qp : 0) : a.qp_rve[qp];
-  const int n = N ? N : kFixed ? a.fixed_n : a.rve_n[rv];
+  const int rv = a.qp_rve[qp];
+  const int n = N ? N : a.rve_n[rv];
   const int NN = n * n;
   const int nn_max = N ? N * N : a.nn_max;
   const Own2D o = make_own(n, a.bc);
-  const uint8_t* phase = a.phase + (kFixed ? (size_t)rv * n * n : (size_t)a.rve_phase_off[rv]);
-  const size_t w_off = kFixed ? (size_t)qp * 2 * n * n : (size_t)a.qp_w_off[qp];
+  const uint8_t* phase = a.phase + (size_t)a.rve_phase_off[rv];
+  const size_t w_off = (size_t)a.qp_w_off[qp];
   const double* w_in = a.w_in + w_off;
   double* w_out = a.w_out + w_off;
-  if constexpr (kFixed) {
-    // the fixed-layout entry takes its phase maps as device data that the host never sees:
-    // a phase id outside the material table is reported (status kStatusBadPhase) before any
-    // table read
-    int badp = 0;
-    for (int e = tid; e < NN; e += blockDim.x) badp |= phase[e] >= kMaxPhase;
-    if (__syncthreads_or(badp)) {
-      if (tid == 0) a.status[qp] = kStatusBadPhase;
-      return;
-    }
-  }
   // Fbar of the current continuation stage, in shared memory (misc[0..3]); read where used
   if (tid < 4) sm.misc[tid] = a.F[(size_t)qp * 4 + tid];
   if (tid < 2 * kMaxPhase) sm.lame[tid] = a.rve_lame[(size_t)rv * 2 * kMaxPhase + tid];
@@ -1425,20 +1338,15 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
     double2 wv = make_double2(w_in[2 * v], w_in[2 * v + 1]);
     if (pinned2(v % n, v / n, a.bc)) wv = make_double2(0.0, 0.0);
     sm.w[v] = wv;
-    if constexpr (REG) sm.w32[v] = make_float2((float)wv.x, (float)wv.y);
+    sm.w32[v] = make_float2((float)wv.x, (float)wv.y);
   }
   __syncthreads();
 
   double* stage_f = reinterpret_cast<double*>(sm.stage);
-  // staged element tangents [36][NN]: the block's global scratch in both modes
-  TA* stage_k = REG ? reinterpret_cast<TA*>(a.scratch) + (size_t)blockIdx.x * a.scratch_stride
-                    : gscr + (size_t)36 * NN;
-  Stencil<TA, REG> S;
-  S.g = gscr;
-  S.NN = NN;
-  // multigrid levels: fast region after the condensation arrays in the stage area (mixed) or
-  // after the staged tangents and stencil in the block scratch (FP64); slow region in the
-  // block scratch
+  // block scratch: staged element tangents [36][NN], then the slow region of the multigrid, whose fast region follows
+  // the condensation arrays in the stage area
+  TA* stage_k = reinterpret_cast<TA*>(a.scratch) + (size_t)blockIdx.x * a.scratch_stride;
+  Stencil S;
   MgCtx<TA> mg;
   mg.n = n;
   if constexpr (N > 0) {
@@ -1449,13 +1357,8 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
   }
   mg.bc = a.bc;
   mg.omega = (TA)a.mg_omega;
-  if constexpr (REG) {
-    mg.fast = reinterpret_cast<TA*>(sm.stage + 8 * (size_t)NN * sizeof(vec2_t<TA>));
-    mg.slow = reinterpret_cast<TA*>(a.scratch) + (size_t)blockIdx.x * a.scratch_stride + (size_t)36 * nn_max;
-  } else {
-    mg.fast = gscr + (size_t)72 * nn_max;
-    mg.slow = mg.fast + mg_fast_max(nn_max);
-  }
+  mg.fast = reinterpret_cast<TA*>(sm.stage + 8 * (size_t)NN * sizeof(vec2_t<TA>));
+  mg.slow = stage_k + (size_t)36 * nn_max;
   double* redD = sm.red + 2 * sm.red_n;  // the PCG's FP64 dot buffer
   vec2_t<TA>* Xs = reinterpret_cast<vec2_t<TA>*>(sm.stage);  // [4][NN]
   vec2_t<TA>* Lb = Xs + 4 * NN;                               // [4][NN]
@@ -1523,7 +1426,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
             wv.x -= step * (double)dx.x;
             wv.y -= step * (double)dx.y;
             sm.w[nd] = wv;
-            if constexpr (REG) sm.w32[nd] = make_float2((float)wv.x, (float)wv.y);
+            sm.w32[nd] = make_float2((float)wv.x, (float)wv.y);
           }
         }
         __syncthreads();
@@ -1567,9 +1470,9 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
       for (int attempt = 0;; ++attempt) {
         {
           const TA Fb[4] = {(TA)sm.misc[0], (TA)sm.misc[1], (TA)sm.misc[2], (TA)sm.misc[3]};
-          build_tangent<TA, REG, kMG, LAW>(o, sm, stage_k, Fb, phase, S, Minv, false, Lb, mg, !reuse);
+          build_tangent<TA, kMG, LAW>(o, sm, stage_k, Fb, phase, S, Minv, false, Lb, mg, !reuse);
         }
-        cg_total += pcg_pair<TA, REG, kMG>(S, o, Minv, mg, b, sm.x, (TA)a.cg_rtol, a.max_cg, sm.p, redD, &pst, true);
+        cg_total += pcg_pair<TA, kMG>(S, o, Minv, mg, b, sm.x, (TA)a.cg_rtol, a.max_cg, sm.p, redD, &pst, true);
         __syncthreads();
         if (reuse && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap || pst == kStatusNegCurv)) {
           reuse = false;  // once more with levels of the current tangent
@@ -1597,7 +1500,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
           wv.x += (double)dx.x;
           wv.y += (double)dx.y;
           sm.w[nd] = wv;
-          if constexpr (REG) sm.w32[nd] = make_float2((float)wv.x, (float)wv.y);
+          sm.w32[nd] = make_float2((float)wv.x, (float)wv.y);
         }
       }
       __syncthreads();
@@ -1610,7 +1513,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
       stage = 0;
       for (int v = tid; v < NN; v += blockDim.x) {
         sm.w[v] = make_double2(0.0, 0.0);
-        if constexpr (REG) sm.w32[v] = make_float2(0.f, 0.f);
+        sm.w32[v] = make_float2(0.f, 0.f);
       }
     } else if (failed || stage >= stages) {
       break;
@@ -1666,7 +1569,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
     // rebuilds the whole tangent with fresh levels and starts the transfer again.
     bool reuse_t = kMG && mg.levels && a.mg_reuse && it > 0;
     for (;;) {
-      build_tangent<TA, REG, kMG, LAW>(o, sm, stage_k, Fb, phase, S, Minv, true, Lb, mg, !reuse_t);
+      build_tangent<TA, kMG, LAW>(o, sm, stage_k, Fb, phase, S, Minv, true, Lb, mg, !reuse_t);
       bool redo = false;
       int t_total = 0, t_max = 0, t_status = kStatusOk;
       for (int c = 0; c < 4; ++c) {
@@ -1685,7 +1588,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
             for (int s = 0; s < 2; ++s)
               X[c * NN + o.node[s]] = o.pin[s] ? mk2<TA>(TA(0), TA(0)) : X0[c * NN + o.node[s]];
           }
-          ci += pcg_pair<TA, REG, kMG>(S, o, Minv, mg, b, X + c * NN, (TA)a.cond_rtol, a.max_cond_cg, sm.p, redD,
+          ci += pcg_pair<TA, kMG>(S, o, Minv, mg, b, X + c * NN, (TA)a.cond_rtol, a.max_cond_cg, sm.p, redD,
                                        &pst, false, warm);
           __syncthreads();
           if (reuse_t && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap)) {
@@ -1713,12 +1616,6 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
       reuse_t = false;
     }
     __syncthreads();
-    const vec2_t<TA>* wsrc;
-    if constexpr (REG) {
-      wsrc = reinterpret_cast<const vec2_t<TA>*>(sm.w32);
-    } else {
-      wsrc = reinterpret_cast<const vec2_t<TA>*>(sm.w);
-    }
 #pragma unroll
     for (int k = 0; k < 10; ++k) Q[k] = 0.0;
     if (o.active) {
@@ -1726,7 +1623,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
       for (int s = 0; s < 2; ++s) {
         const int e = o.node[s];
         const int ph = phase[e];
-        element_transfer<TA, LAW>(e, n, wsrc, X, Fb, (TA)sm.lame[2 * ph], (TA)sm.lame[2 * ph + 1], Q);
+        element_transfer<TA, LAW>(e, n, sm.w32, X, Fb, (TA)sm.lame[2 * ph], (TA)sm.lame[2 * ph + 1], Q);
       }
     }
     block_sum<10, double>(Q, sm.red + (it & 1) * sm.red_n);
@@ -1769,7 +1666,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
   __syncthreads();
 }
 
-template <typename TA, bool kFixed, bool kMG, int LAW, int N>
+template <typename TA, bool kMG, int LAW, int N>
 __global__ void __launch_bounds__(N ? threads2d<TA>(N * N) : kThreads2D, N ? 512 / threads2d<TA>(N * N) : 1)
 rve2d_kernel(const Rve2dArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1781,29 +1678,27 @@ rve2d_kernel(const Rve2dArgs a) {
     sm = smem2d<TA>(offsets2d<TA>(a.nn_max), smem_raw);
   }
   __shared__ int s_item;
-  constexpr bool REG = std::is_same<TA, float>::value;
-  TA* gscr = REG ? nullptr : reinterpret_cast<TA*>(a.scratch) + (size_t)blockIdx.x * a.scratch_stride;
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(a.queue, 1);
     __syncthreads();
     const int item = s_item;
     __syncthreads();
     if (item >= (a.n_dev ? *a.n_dev : a.n_qp)) break;
-    const int qp = kFixed ? item : a.order[item];
-    if (!kFixed && a.only_n && a.rve_n[a.qp_rve[qp]] != a.only_n) continue;  // another launch's grid
-    solve_item_2d<TA, kFixed, kMG, LAW, N>(a, qp, sm, gscr);
+    const int qp = a.order[item];
+    if (a.only_n && a.rve_n[a.qp_rve[qp]] != a.only_n) continue;  // another launch's grid
+    solve_item_2d<TA, kMG, LAW, N>(a, qp, sm);
   }
 }
 
 }  // namespace
 
 // Launch of one instantiation (grid of n_blocks persistent blocks, smem dynamic shared bytes).
-template <typename TA, bool kFixed, bool kMG, int LAW, int N = 0>
+template <typename TA, bool kMG, int LAW, int N = 0>
 inline cudaError_t rve2d_launch_instance(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream) {
-  const cudaError_t err = cudaFuncSetAttribute(rve2d_kernel<TA, kFixed, kMG, LAW, N>,
+  const cudaError_t err = cudaFuncSetAttribute(rve2d_kernel<TA, kMG, LAW, N>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  rve2d_kernel<TA, kFixed, kMG, LAW, N><<<n_blocks, threads2d<TA>(a.nn_max), smem, stream>>>(a);
+  rve2d_kernel<TA, kMG, LAW, N><<<n_blocks, threads2d<TA>(a.nn_max), smem, stream>>>(a);
   return cudaGetLastError();
 }
 

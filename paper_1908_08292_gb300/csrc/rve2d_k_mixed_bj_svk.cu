@@ -3,6 +3,6 @@
 
 namespace fehmm {
 cudaError_t rve2d_launch_mixed_bj_svk(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream) {
-  return rve2d_launch_instance<float, false, false, 1>(a, n_blocks, smem, stream);
+  return rve2d_launch_instance<float, false, 1>(a, n_blocks, smem, stream);
 }
 }  // namespace fehmm

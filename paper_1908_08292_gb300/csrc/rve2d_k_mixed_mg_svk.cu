@@ -3,7 +3,7 @@
 
 namespace fehmm {
 cudaError_t rve2d_launch_mixed_mg_svk(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream) {
-  if (a.nn_max == 24 * 24) return rve2d_launch_instance<float, false, true, 1, 24>(a, n_blocks, smem, stream);
-  return rve2d_launch_instance<float, false, true, 1, 32>(a, n_blocks, smem, stream);
+  if (a.nn_max == 24 * 24) return rve2d_launch_instance<float, true, 1, 24>(a, n_blocks, smem, stream);
+  return rve2d_launch_instance<float, true, 1, 32>(a, n_blocks, smem, stream);
 }
 }  // namespace fehmm
