@@ -50,60 +50,117 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
-// Sum of NV values over the whole block; every thread receives the totals.
-// buf: shared memory with room for NV values per warp; blockDim.x must be a multiple of 32.
-// Contains one __syncthreads(); callers alternate buffers between consecutive calls.
-template <int NV, typename T>
-__device__ __forceinline__ void block_sum(T (&v)[NV], T* buf) {
+// FP64 sums of NV values over a block of up to 16 warps; every thread receives the totals.  An FP64 warp instruction
+// holds its sub-partition for 64 cycles, so each sum is formed once: the values are dealt to the lanes in the first
+// levels of the shuffle tree (16 additions for ten values, where a tree for each takes 50), and the warps add up
+// different values of the block.  buf: kBlockSumDoubles doubles of shared memory; consecutive calls may use the same
+// (each barrier orders one part's reads before the next call's writes).  Two barriers.
+constexpr int kBlockSumDoubles = 170;
+template <int NV>
+__device__ __forceinline__ void block_sum_fp64(double (&v)[NV], double* buf) {
+  constexpr int P = NV <= 1 ? 1 : NV <= 8 ? 8 : 16, kShift = NV <= 1 ? 5 : NV <= 8 ? 2 : 1;
+  static_assert(NV <= 10, "the buffer holds ten values");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  double a[P];
 #pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0) {
+  for (int k = 0; k < P; ++k) a[k] = k < NV ? v[k] : 0.0;
+  int o = 16;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) buf[k * nw + warp] = v[k];
+  for (int cnt = P / 2; cnt >= 1; cnt /= 2) {
+    const bool upper = lane & o;
+#pragma unroll
+    for (int j = 0; j < cnt; ++j) {
+      const double send = upper ? a[j] : a[j + cnt], keep = upper ? a[j + cnt] : a[j];
+      a[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    o >>= 1;
+  }
+#pragma unroll
+  for (int q = 16 / P; q >= 1; q >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], q);
+  const int held = lane >> kShift;  // the value this lane holds
+  if ((lane & ((1 << kShift) - 1)) == 0 && held < NV) buf[16 * held + warp] = a[0];
+  __syncthreads();
+  for (int k = warp; k < NV; k += nw) {
+    double t = lane < nw ? buf[16 * k + lane] : 0.0;
+    for (int q = 8; q >= 1; q >>= 1)
+      if (q < nw) t += __shfl_xor_sync(0xffffffffu, t, q);
+    if (lane == 0) buf[160 + k] = t;
   }
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(lane < nw ? buf[k * nw + lane] : T(0));
+  for (int k = 0; k < NV; ++k) v[k] = buf[160 + k];
 }
 
-// Two inner products summed over a block of up to 16 warps, the block-level sum in FP64: each thread's
-// partial and the warp's shuffle tree stay in T (FP32 in mixed mode), lane 0 of every warp
-// stores its warp sum as a double, and warp 0 adds the 16 warp sums of each product in FP64
-// (lanes 0-15 the first, lanes 16-31 the second, a 4-level shuffle tree in a fixed order, so
-// every launch sums identically) and broadcasts them.  Two barriers.  buf: 34 doubles of shared
-// memory; consecutive calls may reuse it (the second barrier orders every read of a call before
-// the next call's writes).
+__device__ __forceinline__ bool positive_fp64(double x) {  // x > 0 (false for NaN) without an FP64 instruction
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+
+// The two inner products of a PCG step over a block of up to 16 warps, and the tests on them.  Each thread's
+// partial and the warp's shuffle tree are in T (FP32 in mixed mode); warp 0 adds the warp sums in FP64 (lanes 0-15 the
+// first, lanes 16-31 the second product, in a fixed order) and compares them there, and the block receives them
+// rounded to T with the outcome of the tests as flags.  (With the FP64 sums broadcast, every warp converted and
+// compared them itself: five FP64-pipe instructions a warp, at 16 warps about 1300 cycles of an iteration.)
+// stop is compared with the first sum and needed by warp 0 only, as wide, the unrounded first sum, is valid there.
+// buf: kDotDoubles doubles; consecutive calls may use the same.  Two barriers.
+constexpr int kDotDoubles = 36;
+constexpr int kDotNonNeg = 1, kDotPos = 2, kDotFinite = 4, kDotStop = 8, kDotCurvPos = 16;
 template <typename T>
-__device__ __forceinline__ void block_dot2_fp64(T a, T b, double* buf, double& sa, double& sb) {
+__device__ __forceinline__ int block_dot2(T a, T b, double* buf, double stop, T& sa, T& sb, double& wide) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  T* part = reinterpret_cast<T*>(buf);
+  T* out = reinterpret_cast<T*>(buf + 32);
+  int* flags = reinterpret_cast<int*>(buf + 34);
   a = warp_sum(a);
   b = warp_sum(b);
   if (lane == 0) {
-    buf[warp] = (double)a;
-    buf[16 + warp] = (double)b;
+    part[warp] = a;
+    part[16 + warp] = b;
   }
   __syncthreads();
+  wide = 0.0;
   if (warp == 0) {
     const int nw = blockDim.x >> 5;
-    double v = (lane & 15) < nw ? buf[lane] : 0.0;
+    double v = (lane & 15) < nw ? (double)part[lane] : 0.0;
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((lane & 15) == 0) buf[32 + (lane >> 4)] = v;
+    for (int o = 8; o > 0; o >>= 1)
+      if (o < nw) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 15) == 0) out[lane >> 4] = (T)v;
+    wide = __shfl_sync(0xffffffffu, v, 0);
+    const double curv = __shfl_sync(0xffffffffu, v, 16);
+    if (lane == 0) {
+      const long long g = __double_as_longlong(wide);  // ordered as the doubles where both are >= 0
+      const bool zero = (g << 1) == 0, pos = positive_fp64(wide);
+      *flags = (pos || zero ? kDotNonNeg : 0) | (pos ? kDotPos : 0) |
+               ((g & 0x7ff0000000000000ll) != 0x7ff0000000000000ll ? kDotFinite : 0) |
+               ((pos || zero) && g <= __double_as_longlong(stop) ? kDotStop : 0) | (positive_fp64(curv) ? kDotCurvPos : 0);
+    }
   }
   __syncthreads();
-  sa = buf[32];
-  sb = buf[33];
+  sa = out[0];
+  sb = out[1];
+  return *flags;
 }
 
 // 1/J for the FP64 neo-Hookean stress of the residuals: the FP32 approximate reciprocal (rcp.approx, relative error
 // below 2^-22) refined by one third-order step in FP64, x <- x + x (e + e^2) with e = 1 - J x, which cubes the
-// relative error (below FP64 rounding): three FP64 instructions where two Newton-Raphson steps take four.  J below
-// FP32's normal range (a collapsed element) gives a non-finite result, which the Newton loop treats like J <= 0.
+// relative error (below FP64 rounding).  Conversions are FP64-pipe instructions too, so J's FP32 value and the
+// reciprocal's FP64 value are put together from their bits where both are normal FP32 numbers: three FP64
+// instructions in all.  J below FP32's normal range (a collapsed element) gives a non-finite result, which the Newton
+// loop treats like J <= 0.
 __device__ __forceinline__ double recip_fp64(double J) {
   float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)J));
-  const double x = (double)r;
+  double x;
+  const int hi = __double2hiint(J);
+  if ((unsigned)(hi - (897 << 20)) < (252u << 20)) {
+    const float f = __uint_as_float(__funnelshift_l(__double2loint(J), hi, 3) + 0x40000000u);  // exponent bias 1023 -> 127
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
+    const unsigned b = __float_as_uint(r);
+    x = __hiloint2double((int)(b >> 3) + (896 << 20), (int)(b << 29));
+  } else {
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)J));
+    x = (double)r;
+  }
   const double e = fma(-J, x, 1.0);
   return fma(x, fma(e, e, e), x);
 }

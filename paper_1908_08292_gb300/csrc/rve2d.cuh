@@ -58,6 +58,8 @@ __host__ __device__ constexpr int threads2d(int nn) {
   return t < 128 ? 128 : t;
 }
 
+__device__ __forceinline__ int wrap_dec(int i, int n) { return i == 0 ? n - 1 : i - 1; }
+__device__ __forceinline__ int wrap_inc(int i, int n) { return i == n - 1 ? 0 : i + 1; }
 __host__ __device__ constexpr int offx(int a) { return (a == 1 || a == 2) ? 1 : 0; }
 __host__ __device__ constexpr int offy(int a) { return a >= 2 ? 1 : 0; }
 // upper-triangle index of a symmetric 8x8 element matrix
@@ -109,9 +111,9 @@ __host__ __device__ constexpr long long mg_fast_elems(int n) {
     e += 36 * nn + 4 * nn + 3 * 2 * nn;  // stencil, Minv, r/z/t
   }
   const long long nc = (long long)(n >> L) * (n >> L), D = 2 * nc;
-  // fine-level residual, coarsest r/z and its inverse (row stride D + 1; two buffers for the
-  // out-of-place Gauss-Jordan steps)
-  return 2LL * n * n + e + 2 * 2 * nc + 2 * D * (D + 1);
+  // fine-level residual, coarsest r/z, its inverse (row stride D + 4), its matrix (row stride D + 1) and the pivot
+  // rows of the inversion
+  return 2LL * n * n + e + 2 * 2 * nc + D * (D + 4) + D * (D + 1) + 64;
 }
 __host__ __device__ constexpr long long mg_slow_elems(int n) {
   const int L = mg_levels(n);
@@ -126,6 +128,8 @@ __host__ __device__ constexpr long long mg_slow_max(int nn_max) {
   return m;
 }
 
+constexpr int kResidualTable = 2 + 4 * kMaxPhase;  // doubles of the residual's constants (residual_table)
+
 template <typename TA>
 struct Smem2D {
   double2* w;        // [NN] fluctuation (FP64)
@@ -133,16 +137,15 @@ struct Smem2D {
   vec2_t<TA>* p;     // [2][NN] PCG exchange vector (u = M^-1 r), two alternating buffers
   vec2_t<TA>* x;     // [NN] PCG solution (owned nodes written by their thread)
   unsigned char* stage;  // element forces / element tangents / condensation solutions
-  double* red;       // reduction buffers: two of red_n doubles, then the PCG's dot buffer (34)
-  int red_n;
+  double* red;       // buffers of block_sum_fp64 and block_dot2
   double* lame;      // [kMaxPhase][2]
+  double* restab;    // the residual's constants (residual_table)
   double* misc;      // [16]: Fbar (0..3), homogenised P and W (4..8)
 };
 
 // Byte offsets of the arrays in the block's shared memory (constants where the grid is one).
 struct Offsets2D {
-  size_t w, w32, p, x, stage, red, lame, misc, total;
-  int red_n;
+  size_t w, w32, p, x, stage, red, lame, restab, misc, total;
 };
 
 template <typename TA>
@@ -167,9 +170,9 @@ __host__ __device__ constexpr Offsets2D offsets2d(int NN) {
     if (need > stage_bytes) stage_bytes = need;
   }
   o.stage = take(stage_bytes);
-  o.red_n = 10 * (threads2d<TA>(NN) / 32);  // block_sum of up to 10 values
-  o.red = take(sizeof(double) * (2 * o.red_n + 34));
+  o.red = take(sizeof(double) * (kBlockSumDoubles + kDotDoubles));
   o.lame = take(sizeof(double) * 2 * kMaxPhase);
+  o.restab = take(sizeof(double) * kResidualTable);
   o.misc = take(sizeof(double) * 16);
   o.total = off;
   return o;
@@ -184,8 +187,8 @@ __device__ __forceinline__ Smem2D<TA> smem2d(const Offsets2D& o, unsigned char* 
   s.x = reinterpret_cast<vec2_t<TA>*>(base + o.x);
   s.stage = base + o.stage;
   s.red = reinterpret_cast<double*>(base + o.red);
-  s.red_n = o.red_n;
   s.lame = reinterpret_cast<double*>(base + o.lame);
+  s.restab = reinterpret_cast<double*>(base + o.restab);
   s.misc = reinterpret_cast<double*>(base + o.misc);
   return s;
 }
@@ -265,103 +268,172 @@ __device__ __forceinline__ T law2_P(T F00, T F01, T F10, T F11, T lam, T mu, T& 
 }
 
 // ------------------------------------------------------------------ residual (FP64)
-// FP64 first Piola-Kirchhoff stress at one Gauss point (the residual's law; same factored forms
-// as law2_P, with the reciprocal above in place of a division).
-template <int LAW>
-__device__ __forceinline__ double law2_P_fp64(double F00, double F01, double F10, double F11, double hl, double hk,
-                                              double lam, double mu, double& P00, double& P01, double& P10,
-                                              double& P11) {
-  if constexpr (LAW == kLawNH) {
-    // c = lam J / 2 - (lam / 2 + mu) / J with hl = lam / 2, hk = lam / 2 + mu
-    const double J = fma(F00, F11, -F01 * F10);
-    const double c = fma(hl, J, -hk * recip_fp64(J));
-    P00 = fma(mu, F00, c * F11);
-    P01 = fma(mu, F01, -c * F10);
-    P10 = fma(mu, F10, -c * F01);
-    P11 = fma(mu, F11, c * F00);
-    return J;
-  } else {
-    return law2_P<LAW, double>(F00, F01, F10, F11, lam, mu, P00, P01, P10, P11);
-  }
-}
-
-// Element e's nodal forces into stage[k][e] (k = 2*local_node + comp) and this thread's
-// contributions to sum wt P and to the J <= 0 flag.
-//
 // With natural coordinates (s, t) in [0,1]^2 the displacement gradient is bilinear: the first
-// column of F depends on t only, the second on s only.  The nodal forces are (wq / h) P G_a with
-// wq = h^2 / 4 and G_a the natural-coordinate shape gradients, i.e. sums of P's first column
+// column of F depends on t only, the second on s only.  The nodal forces are k P G_a with
+// k = wq / h = h / 4 and G_a the natural-coordinate shape gradients, i.e. sums of P's first column
 // weighted by (1 - t) or t and of its second column weighted by (1 - s) or s.  The stress is
 // therefore summed over the Gauss points of equal t (first column) or equal s (second column)
 // first, and the two Gauss abscissae g0 and g1 = 1 - g0 give both weights.
+//
+// FP64 instructions bound it (64 cycles a warp and sub-partition each, conversions, comparisons and the steps of a
+// division included): the constants come from a table, J > 0 is tested on its bits, the block's sums are formed once:
+// about 140 an element with its share of the gather and the norm, of 190 before (4096 RVEs of 32 x 32, mixed: 490 of
+// 1840 thousand cycles an RVE).  The FP64 arithmetic itself is kept: the FP32 solves that follow turn differences in
+// the last bit of a small residual into differences of 1e-9 in the tangent.
+
+// The residual's constants in shared memory (k g0, k g1, then per phase lam / 2, lam / 2 + mu, mu, lam).
+__device__ __forceinline__ void residual_table(int n, const double* lame, double* tab) {
+  const int tid = threadIdx.x;
+  if (tid < kMaxPhase) {
+    const double lam = lame[2 * tid], mu = lame[2 * tid + 1], hl = 0.5 * lam;
+    tab[2 + 4 * tid] = hl;
+    tab[3 + 4 * tid] = hl + mu;
+    tab[4 + 4 * tid] = mu;
+    tab[5 + 4 * tid] = lam;
+  }
+  if (tid < 2) tab[tid] = 0.25 / (double)n * gauss01(tid);
+}
+
+// FP64 first Piola-Kirchhoff stress at one Gauss point (same factored forms as law2_P) from the table's constants m
+// of the phase; false where not J > 0.
 template <int LAW>
-__device__ __forceinline__ void element_residual(int e, int n, const double2* w, const double* Fb,
-                                                 double lam, double mu, double* stage_f, double (&Psum)[4],
-                                                 double& bad) {
-  const int i = e % n, j = e / n, ip = (i + 1) % n, jp = (j + 1) % n;
-  const double2 w0 = w[e], w1 = w[ip + n * j], w2 = w[ip + n * jp], w3 = w[i + n * jp];
-  const double ih = unfolded((double)n);
-  const double2 d10 = make_double2(w1.x - w0.x, w1.y - w0.y);
-  const double2 d30 = make_double2(w3.x - w0.x, w3.y - w0.y);
-  const double2 e1 = make_double2((w2.x - w3.x) - d10.x, (w2.y - w3.y) - d10.y);
-  const double2 e2 = make_double2((w2.x - w1.x) - d30.x, (w2.y - w1.y) - d30.y);
-  const double hl = 0.5 * lam, hk = hl + mu;
-  // F's first column at t = g0, g1; second column at s = g0, g1
-  double Fc0[2][2], Fc1[2][2];
+__device__ __forceinline__ bool stress2(double F00, double F01, double F10, double F11, const double (&m)[4], double& P00,
+                                        double& P01, double& P10, double& P11) {
+  if constexpr (LAW == kLawNH) {
+    // c = lam J / 2 - (lam / 2 + mu) / J
+    const double J = fma(F00, F11, -F01 * F10);
+    const double c = fma(m[0], J, -m[1] * recip_fp64(J));
+    P00 = fma(m[2], F00, c * F11);
+    P01 = fma(m[2], F01, -c * F10);
+    P10 = fma(m[2], F10, -c * F01);
+    P11 = fma(m[2], F11, c * F00);
+    return positive_fp64(J);
+  } else {
+    return positive_fp64(law2_P<LAW, double>(F00, F01, F10, F11, m[3], m[2], P00, P01, P10, P11));
+  }
+}
+
+// The displacement differences of element e: F's first column is Fb + (d0 + t e1) / h, its second Fb + (d1 + s e2) / h.
+struct ElementF {
+  double d0x, d0y, d1x, d1y, e1x, e1y, e2x, e2y, ih;
+  const double* Fb;
+  __device__ __forceinline__ ElementF(int e, int n, const double2* w, const double* Fbar) : Fb(Fbar) {
+    const int i = e % n, j = e / n, ip = wrap_inc(i, n), jp = wrap_inc(j, n);
+    const double2 w0 = w[e], w1 = w[ip + n * j], w2 = w[ip + n * jp], w3 = w[i + n * jp];
+    ih = unfolded((double)n);
+    d0x = w1.x - w0.x;
+    d0y = w1.y - w0.y;
+    d1x = w3.x - w0.x;
+    d1y = w3.y - w0.y;
+    e1x = (w2.x - w3.x) - d0x;
+    e1y = (w2.y - w3.y) - d0y;
+    e2x = (w2.x - w1.x) - d1x;
+    e2y = (w2.y - w1.y) - d1y;
+  }
+  __device__ __forceinline__ double F00(double t) const { return fma(ih, fma(t, e1x, d0x), Fb[0]); }
+  __device__ __forceinline__ double F10(double t) const { return fma(ih, fma(t, e1y, d0y), Fb[2]); }
+  __device__ __forceinline__ double F01(double s) const { return fma(ih, fma(s, e2x, d1x), Fb[1]); }
+  __device__ __forceinline__ double F11(double s) const { return fma(ih, fma(s, e2y, d1y), Fb[3]); }
+};
+
+// One component of element e's nodal forces from the stress columns' sums (first column per t, second per s);
+// weight 1 - t is g1 at t = g0 and g0 at t = g1.
+__device__ __forceinline__ void element_forces(double a0, double a1, double b0, double b1, double kg0, double kg1, double* f,
+                                               int NN) {
+  const double Sa0 = fma(kg1, a0, kg0 * a1), Sa1 = fma(kg0, a0, kg1 * a1);
+  const double Sb0 = fma(kg1, b0, kg0 * b1), Sb1 = fma(kg0, b0, kg1 * b1);
+  f[0 * NN] = -Sa0 - Sb0;
+  f[2 * NN] = Sa0 - Sb1;
+  f[4 * NN] = Sa1 + Sb1;
+  f[6 * NN] = -Sa1 + Sb0;
+}
+
+// Element e's nodal forces into stage[k][e] (k = 2*local_node + comp), this thread's sums of P and its number of
+// points with J <= 0.
+template <int LAW>
+__device__ __forceinline__ void element_residual(int e, int n, const double2* w, const double* Fb, const double* tab,
+                                                 int phase, double* stage_f, double (&Psum)[4], int& nbad) {
+  const ElementF f(e, n, w, Fb);
+  const double* mt = tab + 2 + 4 * phase;
+  const double m[4] = {mt[0], mt[1], mt[2], mt[3]};
+  double F0[2][2], F1[2][2], q0x[2], q0y[2], q1x[2], q1y[2];
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
     const double t = gauss01(g);
-    Fc0[g][0] = fma(ih, fma(t, e1.x, d10.x), Fb[0]);
-    Fc0[g][1] = fma(ih, fma(t, e1.y, d10.y), Fb[2]);
-    Fc1[g][0] = fma(ih, fma(t, e2.x, d30.x), Fb[1]);
-    Fc1[g][1] = fma(ih, fma(t, e2.y, d30.y), Fb[3]);
+    F0[g][0] = f.F00(t);
+    F0[g][1] = f.F10(t);
+    F1[g][0] = f.F01(t);
+    F1[g][1] = f.F11(t);
   }
-  double q0x[2], q0y[2], q1x[2], q1y[2];  // P's first column summed over s (per t), second over t (per s)
-  int nbad = 0;
 #pragma unroll
-  for (int gy = 0; gy < 2; ++gy) {
+  for (int gy = 0; gy < 2; ++gy)
 #pragma unroll
     for (int gx = 0; gx < 2; ++gx) {
       double P00, P01, P10, P11;
-      const double J = law2_P_fp64<LAW>(Fc0[gy][0], Fc1[gx][0], Fc0[gy][1], Fc1[gx][1], hl, hk, lam, mu, P00, P01,
-                                        P10, P11);
-      nbad += (J > 0.0) ? 0 : 1;
-      if (gx == 0) {
-        q0x[gy] = P00;
-        q0y[gy] = P10;
-      } else {
-        q0x[gy] += P00;
-        q0y[gy] += P10;
-      }
-      if (gy == 0) {
-        q1x[gx] = P01;
-        q1y[gx] = P11;
-      } else {
-        q1x[gx] += P01;
-        q1y[gx] += P11;
-      }
+      nbad += !stress2<LAW>(F0[gy][0], F1[gx][0], F0[gy][1], F1[gx][1], m, P00, P01, P10, P11);
+      q0x[gy] = gx ? q0x[gy] + P00 : P00;
+      q0y[gy] = gx ? q0y[gy] + P10 : P10;
+      q1x[gx] = gy ? q1x[gx] + P01 : P01;
+      q1y[gx] = gy ? q1y[gx] + P11 : P11;
     }
-  }
-  if (nbad) bad += (double)nbad;
   Psum[0] += q0x[0] + q0x[1];
   Psum[1] += q1x[0] + q1x[1];
   Psum[2] += q0y[0] + q0y[1];
   Psum[3] += q1y[0] + q1y[1];
-  const double k = 0.25 / ih, kg0 = k * gauss01(0), kg1 = k * gauss01(1);
-  // weight 1 - t is g1 at t = g0 and g0 at t = g1
-  const double Sa0x = fma(kg1, q0x[0], kg0 * q0x[1]), Sa1x = fma(kg0, q0x[0], kg1 * q0x[1]);
-  const double Sa0y = fma(kg1, q0y[0], kg0 * q0y[1]), Sa1y = fma(kg0, q0y[0], kg1 * q0y[1]);
-  const double Sb0x = fma(kg1, q1x[0], kg0 * q1x[1]), Sb1x = fma(kg0, q1x[0], kg1 * q1x[1]);
-  const double Sb0y = fma(kg1, q1y[0], kg0 * q1y[1]), Sb1y = fma(kg0, q1y[0], kg1 * q1y[1]);
   const int NN = n * n;
-  stage_f[0 * NN + e] = -Sa0x - Sb0x;
-  stage_f[1 * NN + e] = -Sa0y - Sb0y;
-  stage_f[2 * NN + e] = Sa0x - Sb1x;
-  stage_f[3 * NN + e] = Sa0y - Sb1y;
-  stage_f[4 * NN + e] = Sa1x + Sb1x;
-  stage_f[5 * NN + e] = Sa1y + Sb1y;
-  stage_f[6 * NN + e] = -Sa1x + Sb0x;
-  stage_f[7 * NN + e] = -Sa1y + Sb0y;
+  const double kg0 = tab[0], kg1 = tab[1];
+  element_forces(q0x[0], q0x[1], q1x[0], q1x[1], kg0, kg1, stage_f + e, NN);
+  element_forces(q0y[0], q0y[1], q1y[0], q1y[1], kg0, kg1, stage_f + NN + e, NN);
+}
+
+// The same by two lanes, each with the points of one t; whole warps call it (in: the element exists).
+template <int LAW>
+__device__ __forceinline__ void element_residual_half(bool in, int e, int half, int n, const double2* w, const double* Fb,
+                                                      const double* tab, int phase, double* stage_f, double (&Psum)[4],
+                                                      int& nbad) {
+  const ElementF f(e, n, w, Fb);
+  const double* mt = tab + 2 + 4 * phase;
+  const double m[4] = {mt[0], mt[1], mt[2], mt[3]}, t = gauss01(half);
+  const double F00 = f.F00(t), F10 = f.F10(t);
+  double q0x = 0.0, q0y = 0.0, q1x[2], q1y[2];
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    double P00, P10;
+    const bool good = stress2<LAW>(F00, f.F01(gauss01(g)), F10, f.F11(gauss01(g)), m, P00, q1x[g], P10, q1y[g]);
+    nbad += in && !good;
+    q0x = g ? q0x + P00 : P00;
+    q0y = g ? q0y + P10 : P10;
+  }
+  if (in) {
+    Psum[0] += q0x;
+    Psum[1] += q1x[0] + q1x[1];
+    Psum[2] += q0y;
+    Psum[3] += q1y[0] + q1y[1];
+  }
+  // lane 0 of the pair forms the x forces, lane 1 the y forces
+  const auto other = [](double v) { return __shfl_xor_sync(0xffffffffu, v, 1); };
+  const double o0 = other(half ? q0x : q0y), o1 = other(half ? q1x[0] : q1y[0]), o2 = other(half ? q1x[1] : q1y[1]);
+  const double a0 = half ? o0 : q0x, a1 = half ? q0y : o0;  // first column at t = g0, g1
+  const double b0 = (half ? q1y[0] : q1x[0]) + o1, b1 = (half ? q1y[1] : q1x[1]) + o2;
+  const int NN = n * n;
+  if (in) element_forces(a0, a1, b0, b1, tab[0], tab[1], stage_f + half * NN + e, NN);
+}
+
+// All elements of a block's RVE.  Two lanes an element where that still is one pass of the block: a lane then
+// executes about 70 FP64 instructions in place of 128.  Where threads are fewer, an element per thread.
+template <int LAW>
+__device__ __forceinline__ void block_residual(int n, const double2* w, const double* Fb, const double* tab,
+                                               const uint8_t* phase, double* stage_f, double (&Psum)[4], int& nbad) {
+  const int NN = n * n, tid = threadIdx.x;
+  if (2 * NN <= (int)blockDim.x) {
+    if ((tid & ~31) < 2 * NN) {
+      const bool in = tid < 2 * NN;
+      const int e = in ? tid >> 1 : 0;
+      element_residual_half<LAW>(in, e, tid & 1, n, w, Fb, tab, phase[e], stage_f, Psum, nbad);
+    }
+  } else {
+    for (int e = tid; e < NN; e += blockDim.x) element_residual<LAW>(e, n, w, Fb, tab, phase[e], stage_f, Psum, nbad);
+  }
 }
 
 // Psi summed over the element's Gauss points: neo-Hookean lam/4 (J^2-1) - (lam/2+mu) ln J +
@@ -646,9 +718,13 @@ struct MgCtx {
     }
     return v;
   }
-  __device__ __forceinline__ TA* coarsest_inverse() const {
+  __device__ __forceinline__ TA* coarsest_inverse() const {  // [D][D + 4]
     const MgLevel<TA> v = level(levels);
     return reinterpret_cast<TA*>(v.z + v.NN);
+  }
+  __device__ __forceinline__ TA* coarsest_matrix() const {  // [D][D + 1], then two pivot rows
+    const int D = 2 * (n >> levels) * (n >> levels);
+    return coarsest_inverse() + D * (D + 4);
   }
 };
 
@@ -706,8 +782,6 @@ __device__ __forceinline__ void mg_coarse_element(const TA* kf, int nf, int E, T
 }
 
 // Periodic neighbours without integer division.
-__device__ __forceinline__ int wrap_dec(int i, int n) { return i == 0 ? n - 1 : i - 1; }
-__device__ __forceinline__ int wrap_inc(int i, int n) { return i == n - 1 ? 0 : i + 1; }
 
 // y = K_l z at node v = (i, j) of a coarse level (zero at the pinned node).
 template <typename TA>
@@ -804,33 +878,41 @@ __device__ __forceinline__ void mg_stencil_block(const TA* ke, int n, int i, int
     }
 }
 
+// 1 / x for finite positive normal x (exponent split off, FP32 reciprocal of the mantissa refined twice); else 1 / x
+__device__ __forceinline__ double recip_d(double x) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (e == 0 || e > 2040 || hi < 0) return 1.0 / x;
+  const double m = __hiloint2double((hi & 0xfffff) | (1023 << 20), __double2loint(x));
+  float f;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"((float)m));
+  double q = (double)f;
+  const double err = fma(-m, q, 1.0);
+  q = fma(q, fma(err, err, err), q);
+  return __hiloint2double(__double2hiint(q) + ((1023 - e) << 20), __double2loint(q));
+}
+
+// One entry of a Gauss-Jordan step: a - aik akj ip, in the pivot's column (own) -aik ip.  In FP64 with the pivot
+// row's kj = akj ip formed once, one FP64 instruction an entry.
+__device__ __forceinline__ float dense_update(float a, float aik, float akj, float ip, float, bool own) {
+  return own ? -aik * ip : a - aik * akj * ip;
+}
+__device__ __forceinline__ double dense_update(double a, double aik, double, double ip, double kj, bool own) {
+  return fma(-aik, own ? ip : kj, own ? 0.0 : a);
+}
+__device__ __forceinline__ float dense_recip(float x) { return 1.f / x; }
+__device__ __forceinline__ double dense_recip(double x) { return recip_d(x); }
+
+// Dense pinned matrix of the coarsest level (one row per thread) and its inverse by Gauss-Jordan elimination: the
+// matrix in registers, a column per lane and the rows dealt to the warps, so that a step has one barrier and moves
+// only the pivot row through shared memory.  (With the matrix in shared memory a step took 2300 cycles at four warps,
+// 900 at 16, which was 12 % of an 8 x 8 solve.)  D <= 32, at least four warps.
 template <typename TA>
-__device__ __forceinline__ void mg_build_part2(const MgCtx<TA>& mg) {
+__device__ __forceinline__ void mg_invert_coarsest(const MgCtx<TA>& mg) {
   const int tid = threadIdx.x;
-  __syncthreads();  // part 1's element matrices complete
-  for (int l = 1; l < mg.levels; ++l) {  // stencils and inverted blocks of the smoothing levels
-    const MgLevel<TA> v = mg.level(l);
-    for (int node = tid; node < v.NN; node += blockDim.x) {
-      const int i = node % v.n, j = node / v.n;
-#pragma unroll 1
-      for (int nb = 0; nb < 9; ++nb) {
-        TA blk[4];
-        mg_stencil_block<TA>(v.ke, v.n, i, j, nb, blk);
-        v.st[nb * v.NN + node] = {blk[0], blk[1], blk[2], blk[3]};
-        if (nb == 4) {
-          TA m[4];
-          invert_block<TA>(blk, pinned2(i, j, v.bc), m);
-          v.mi[node] = {m[0], m[1], m[2], m[3]};
-        }
-      }
-    }
-  }
-  // coarsest: dense pinned matrix (one row per thread), then its inverse by Gauss-Jordan
-  // elimination, one pivot per step over the whole block, alternating between two buffers
   const MgLevel<TA> c = mg.level(mg.levels);
   const int D = 2 * c.NN, ld = D + 1;
-  TA* A = mg.coarsest_inverse();
-  TA* B = A + (size_t)D * ld;
+  TA* A = mg.coarsest_matrix();
+  TA* piv = A + (size_t)D * ld;  // [2][32]
   if (tid < D) {
     const int node = tid >> 1, ii = tid & 1, ni = node % c.n, nj = node / c.n;
     for (int q = 0; q < D; ++q) A[(size_t)tid * ld + q] = TA(0);
@@ -854,24 +936,60 @@ __device__ __forceinline__ void mg_build_part2(const MgCtx<TA>& mg) {
     }
   }
   __syncthreads();
-  // one column per lane (D <= 32), the rows dealt to the warps
   const int j = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  for (int k = 0; k < D; ++k) {  // SPD: no pivoting; D is even, so the result ends in A
-    const TA* Ao = (k & 1) ? B : A;
-    TA* An = (k & 1) ? A : B;
-    const TA ip = TA(1) / Ao[(size_t)k * ld + k];
-    if (j < D) {
-      const TA akj = Ao[(size_t)k * ld + j];
-      for (int i = warp; i < D; i += nw) {
-        const TA aik = Ao[(size_t)i * ld + k];
-        TA v;
-        if (i == k) v = (j == k) ? ip : akj * ip;
-        else v = (j == k) ? -aik * ip : Ao[(size_t)i * ld + j] - aik * akj * ip;
-        An[(size_t)i * ld + j] = v;
-      }
+  TA a[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int i = warp + nw * q;
+    a[q] = i < D && j < D ? A[(size_t)i * ld + j] : TA(0);
+  }
+  if (warp == 0) piv[j] = a[0];
+  __syncthreads();
+  for (int k = 0; k < D; ++k) {  // SPD: no pivoting
+    const TA* pk = piv + 32 * (k & 1);
+    const TA ip = dense_recip(pk[k]), akj = pk[j], kj = akj * ip;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = warp + nw * q;  // uniform in the warp
+      if (i >= D) break;
+      const TA aik = __shfl_sync(0xffffffffu, a[q], k);
+      if (i == k) a[q] = j == k ? ip : kj;
+      else a[q] = dense_update(a[q], aik, akj, ip, kj, j == k);
+      if (i == k + 1) piv[32 * ((k + 1) & 1) + j] = a[q];
     }
     __syncthreads();
   }
+  TA* I = mg.coarsest_inverse();
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int i = warp + nw * q;
+    if (i < D && j < D) I[(size_t)i * (D + 4) + j] = a[q];
+  }
+  __syncthreads();
+}
+
+template <typename TA>
+__device__ __forceinline__ void mg_build_part2(const MgCtx<TA>& mg) {
+  const int tid = threadIdx.x;
+  __syncthreads();  // part 1's element matrices complete
+  for (int l = 1; l < mg.levels; ++l) {  // stencils and inverted blocks of the smoothing levels
+    const MgLevel<TA> v = mg.level(l);
+    for (int node = tid; node < v.NN; node += blockDim.x) {
+      const int i = node % v.n, j = node / v.n;
+#pragma unroll 1
+      for (int nb = 0; nb < 9; ++nb) {
+        TA blk[4];
+        mg_stencil_block<TA>(v.ke, v.n, i, j, nb, blk);
+        v.st[nb * v.NN + node] = {blk[0], blk[1], blk[2], blk[3]};
+        if (nb == 4) {
+          TA m[4];
+          invert_block<TA>(blk, pinned2(i, j, v.bc), m);
+          v.mi[node] = {m[0], m[1], m[2], m[3]};
+        }
+      }
+    }
+  }
+  mg_invert_coarsest<TA>(mg);
 }
 
 // Restricted residual of coarse node t of level l (from the residual t_f of the finer grid nf),
@@ -891,6 +1009,29 @@ template <typename TA>
 __device__ __forceinline__ const vec2_t<TA>* mg_result(const MgCtx<TA>& mg, int l) {
   const MgLevel<TA> v = mg.level(l);
   return l == mg.levels ? v.z : v.t;
+}
+
+// Row tid / 4 of A r, by four lanes (at least 4 D threads; A with row stride D + 4, which spreads a warp's eight rows
+// over the banks).  The sums are those of 16 lanes per row and a shuffle tree over them, with two of its four levels
+// inside the lane: 32 x 32, the coarsest level with 16 lanes per row and their four levels of shuffles 1350 cycles
+// of a V-cycle, at 128 threads (8 x 8) 2000.
+template <typename TA>
+__device__ __forceinline__ TA coarsest_row(const TA* A, const TA* r, int D) {
+  const int row = threadIdx.x >> 2, l4 = threadIdx.x & 3;
+  if ((threadIdx.x & ~31) >> 2 >= D) return TA(0);  // a whole warp without rows
+  TA z[4] = {TA(0), TA(0), TA(0), TA(0)};
+  if (row < D) {
+    const TA* Ar = A + (size_t)row * (D + 4);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {  // D <= 32
+      const int q = l4 + 4 * i;
+      if (q < D) z[i & 3] += Ar[q] * r[q];
+    }
+  }
+  TA s = (z[0] + z[2]) + (z[1] + z[3]);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  return s;
 }
 
 // Coarse part of the V-cycle.  On entry level(1) holds the restricted residual (and, for a
@@ -913,21 +1054,12 @@ __device__ __forceinline__ void mg_coarse_cycle(const MgCtx<TA>& mg) {
     if (tid < mg.level(l + 1).NN) mg_restrict_smooth<TA>(mg, l + 1, v.t, v.n, tid);
     __syncthreads();
   }
-  {  // coarsest: z = A^-1 r, 16 lanes per row (rows 0, 1 of the inverse: the pinned identity)
+  {  // coarsest: z = A^-1 r, four lanes per row
     const MgLevel<TA> c = mg.level(mg.levels);
-    const int D = 2 * c.NN, ld = D + 1, l16 = tid & 15;
-    const TA* A = mg.coarsest_inverse();
-    const TA* r = reinterpret_cast<const TA*>(c.r);
-    for (int row0 = 0; row0 < D; row0 += blockDim.x >> 4) {  // whole warps stay in the loop
-      const int row = row0 + (tid >> 4);
-      TA zz = TA(0);
-      if (row < D)
-        for (int q = l16; q < D; q += 16) zz += A[(size_t)row * ld + q] * r[q];
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) zz += __shfl_xor_sync(0xffffffffu, zz, o);
-      if (row < D && l16 == 0)
-        reinterpret_cast<TA*>(c.z)[row] = pinned2((row >> 1) % c.n, (row >> 1) / c.n, c.bc) ? TA(0) : zz;
-    }
+    const TA z = coarsest_row<TA>(mg.coarsest_inverse(), reinterpret_cast<const TA*>(c.r), 2 * c.NN);
+    const int row = tid >> 2;
+    if (row < 2 * c.NN && (tid & 3) == 0)
+      reinterpret_cast<TA*>(c.z)[row] = pinned2((row >> 1) % c.n, (row >> 1) / c.n, c.bc) ? TA(0) : z;
     __syncthreads();
   }
 #pragma unroll
@@ -1056,12 +1188,13 @@ __device__ __forceinline__ int pcg_pair(const Stencil& S, const Own2D& o, const 
     jacobi(t, om);     // post-smoothing
   };
   *status = kStatusOk;
-  double gref = -1.0;  // stopping reference b^T M^-1 b of a warm start
-  int it = 0;
+  double stop = 0.0, wide = 0.0;  // valid in warp 0
+  int it = 0, fref = kDotNonNeg;
   if (warm) {
-    precond();  // u = M^-1 b
-    double unused;
-    block_dot2_fp64<TA>(r[0] * u[0] + r[1] * u[1] + r[2] * u[2] + r[3] * u[3], TA(0), red, gref, unused);
+    precond();  // u = M^-1 b: the stopping reference b^T M^-1 b
+    TA unused0, unused1;
+    fref = block_dot2<TA>(r[0] * u[0] + r[1] * u[1] + r[2] * u[2] + r[3] * u[3], TA(0), red, 0.0, unused0, unused1, wide);
+    if (threadIdx.x < 32) stop = (double)rtol * (double)rtol * wide;
     if (o.active) {  // u = x0, w = K x0, r = b - K x0
       const vec2_t<TA> x0 = xs[o.node[0]], x1 = xs[o.node[1]];
       u[0] = x0.x;
@@ -1082,20 +1215,18 @@ __device__ __forceinline__ int pcg_pair(const Stencil& S, const Own2D& o, const 
   }
   precond();
   exchange_apply();
-  // inner products: per thread and per warp in TA, over the block in FP64 (block_dot2_fp64); the
-  // stopping test compares FP64 sums, the step scalars are formed in TA from them
-  double gd, dd;
-  block_dot2_fp64<TA>(r[0] * u[0] + r[1] * u[1] + r[2] * u[2] + r[3] * u[3],
-                      w[0] * u[0] + w[1] * u[1] + w[2] * u[2] + w[3] * u[3], red, gd, dd);
-  TA gamma = (TA)gd, delta = (TA)dd;
-  const double gamma0 = gd;
-  const double stop = (double)rtol * (double)rtol * (warm ? gref : gamma0);
+  // inner products: per thread and per warp in TA, over the block in FP64; the stopping test compares FP64 sums, the
+  // step scalars are formed in TA from them (block_dot2)
+  TA gamma, delta;
+  const int f0 = block_dot2<TA>(r[0] * u[0] + r[1] * u[1] + r[2] * u[2] + r[3] * u[3],
+                                w[0] * u[0] + w[1] * u[1] + w[2] * u[2] + w[3] * u[3], red, stop, gamma, delta, wide);
+  if (!warm && threadIdx.x < 32) stop = (double)rtol * (double)rtol * wide;
   // a non-finite or negative preconditioned residual norm r^T M^-1 r (a multigrid coarse inverse of
   // an indefinite tangent, or a V-cycle that is not positive definite) is a breakdown, not a
   // converged zero correction
-  if (!isfinite(gamma0) || gamma0 < 0.0 || (warm && !(gref >= 0.0))) *status = kStatusPcgBreakdown;
-  if (*status == kStatusOk && gamma0 > 0.0 && !(warm && gamma0 <= stop)) {
-    if (!(dd > 0.0)) {
+  if (!(f0 & kDotFinite) || !(f0 & kDotNonNeg) || !(fref & kDotNonNeg)) *status = kStatusPcgBreakdown;
+  if (*status == kStatusOk && (f0 & kDotPos) && !(warm && (f0 & kDotStop))) {
+    if (!(f0 & kDotCurvPos)) {
       if (truncate && delta < TA(0)) {
         const TA a0 = cg_div(gamma, -delta);
         x_axpy(a0, u);
@@ -1120,16 +1251,15 @@ __device__ __forceinline__ int pcg_pair(const Stencil& S, const Own2D& o, const 
         for (int k = 0; k < 4; ++k) r[k] -= alpha * s[k];
         precond();
         exchange_apply();
-        double gnd, dnd;
-        block_dot2_fp64<TA>(r[0] * u[0] + r[1] * u[1] + r[2] * u[2] + r[3] * u[3],
-                            w[0] * u[0] + w[1] * u[1] + w[2] * u[2] + w[3] * u[3], red, gnd, dnd);
-        const TA gn = (TA)gnd, dn = (TA)dnd;
+        TA gn, dn;
+        const int f = block_dot2<TA>(r[0] * u[0] + r[1] * u[1] + r[2] * u[2] + r[3] * u[3],
+                                     w[0] * u[0] + w[1] * u[1] + w[2] * u[2] + w[3] * u[3], red, stop, gn, dn, wide);
         ++it;
-        if (!(gnd >= 0.0)) {  // preconditioner not positive definite (or non-finite)
+        if (!(f & kDotNonNeg)) {  // preconditioner not positive definite (or non-finite)
           *status = kStatusPcgBreakdown;
           break;
         }
-        if (gnd <= stop) break;
+        if (f & kDotStop) break;
         const TA beta = cg_div(gn, gamma);
         const TA den = dn - beta * cg_div(gn, alpha);  // p_new^T K p_new
         if (!(den > TA(0))) {
@@ -1165,13 +1295,9 @@ __device__ __forceinline__ void build_tangent(const Own2D& o, const Smem2D<TA>& 
                                               bool build_mg = true) {
   TA L[2][2][4];
   const int n = o.n, NN = o.NN;
-  if (o.active) {
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const int e = o.node[s];
-      const int ph = phase[e];
-      element_tangent<TA, LAW>(e, n, sm.w32, Fb, (TA)sm.lame[2 * ph], (TA)sm.lame[2 * ph + 1], stage_k, e, NN);
-    }
+  for (int e = threadIdx.x; e < NN; e += blockDim.x) {
+    const int ph = phase[e];
+    element_tangent<TA, LAW>(e, n, sm.w32, Fb, (TA)sm.lame[2 * ph], (TA)sm.lame[2 * ph + 1], stage_k, e, NN);
   }
   __syncthreads();
   if (kMG && mg.levels && build_mg) mg_build_part1<TA>(mg, stage_k);  // reads the staged element tangents
@@ -1333,7 +1459,9 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
   double* w_out = a.w_out + w_off;
   // Fbar of the current continuation stage, in shared memory (misc[0..3]); read where used
   if (tid < 4) sm.misc[tid] = a.F[(size_t)qp * 4 + tid];
-  if (tid < 2 * kMaxPhase) sm.lame[tid] = a.rve_lame[(size_t)rv * 2 * kMaxPhase + tid];
+  const double* lame_g = a.rve_lame + (size_t)rv * 2 * kMaxPhase;
+  if (tid < 2 * kMaxPhase) sm.lame[tid] = lame_g[tid];
+  residual_table(n, lame_g, sm.restab);
   for (int v = tid; v < NN; v += blockDim.x) {
     double2 wv = make_double2(w_in[2 * v], w_in[2 * v + 1]);
     if (pinned2(v % n, v / n, a.bc)) wv = make_double2(0.0, 0.0);
@@ -1359,7 +1487,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
   mg.omega = (TA)a.mg_omega;
   mg.fast = reinterpret_cast<TA*>(sm.stage + 8 * (size_t)NN * sizeof(vec2_t<TA>));
   mg.slow = stage_k + (size_t)36 * nn_max;
-  double* redD = sm.red + 2 * sm.red_n;  // the PCG's FP64 dot buffer
+  double* redD = sm.red + kBlockSumDoubles;  // the PCG's dot buffer
   vec2_t<TA>* Xs = reinterpret_cast<vec2_t<TA>*>(sm.stage);  // [4][NN]
   vec2_t<TA>* Lb = Xs + 4 * NN;                               // [4][NN]
   TA Minv[2][4];
@@ -1386,16 +1514,9 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
     for (;;) {
       // ---- FP64 residual
       Psum[0] = Psum[1] = Psum[2] = Psum[3] = 0.0;
-      double bad = 0.0;
-      if (o.active) {
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          const int e = o.node[s];
-          const int ph = phase[e];
-          element_residual<LAW>(e, n, sm.w, sm.misc, sm.lame[2 * ph], sm.lame[2 * ph + 1], stage_f, Psum, bad);
-        }
-      }
-      __syncthreads();
+      int nbad = 0;
+      block_residual<LAW>(n, sm.w, sm.misc, sm.restab, phase, stage_f, Psum, nbad);
+      const bool bad = __syncthreads_or(nbad);
       double R[4] = {0, 0, 0, 0};
       if (o.active) {
 #pragma unroll
@@ -1409,11 +1530,11 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
         if (o.pin[0]) R[0] = R[1] = 0.0;
         if (o.pin[1]) R[2] = R[3] = 0.0;
       }
-      double v2[2] = {R[0] * R[0] + R[1] * R[1] + R[2] * R[2] + R[3] * R[3], bad};
-      block_sum<2, double>(v2, sm.red + (it & 1) * sm.red_n);
+      double v2[1] = {R[0] * R[0] + R[1] * R[1] + R[2] * R[2] + R[3] * R[3]};
+      block_sum_fp64<1>(v2, sm.red);
       const double rn = sqrt(v2[0]);
       if (it == 0) r0 = rn;
-      if ((v2[1] > 0.0 || !isfinite(rn)) && it > 0 && nhalf < kMaxStepHalvings) {
+      if ((bad || !isfinite(rn)) && it > 0 && nhalf < kMaxStepHalvings) {
         // backtrack: w = w_prev + step x  ->  w_prev + (step/2) x
         ++nhalf;
         step *= 0.5;
@@ -1432,7 +1553,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
         __syncthreads();
         continue;
       }
-      if (v2[1] > 0.0) {
+      if (bad) {
         status = kStatusJNonPos;
         break;
       }
@@ -1545,8 +1666,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
       Pv[4] += element_energy<LAW>(e, n, sm.w, sm.misc, sm.lame[2 * ph], sm.lame[2 * ph + 1]);
     }
   }
-  // the last residual norm used buffer (it & 1) and may still be read: use the other one
-  block_sum<5, double>(Pv, sm.red + ((it + 1) & 1) * sm.red_n);
+  block_sum_fp64<5>(Pv, sm.red);
   if (tid == 0) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) sm.misc[4 + k] = Pv[k];
@@ -1618,15 +1738,11 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < 10; ++k) Q[k] = 0.0;
-    if (o.active) {
-#pragma unroll
-      for (int s = 0; s < 2; ++s) {
-        const int e = o.node[s];
-        const int ph = phase[e];
-        element_transfer<TA, LAW>(e, n, sm.w32, X, Fb, (TA)sm.lame[2 * ph], (TA)sm.lame[2 * ph + 1], Q);
-      }
+    for (int e = tid; e < NN; e += blockDim.x) {
+      const int ph = phase[e];
+      element_transfer<TA, LAW>(e, n, sm.w32, X, Fb, (TA)sm.lame[2 * ph], (TA)sm.lame[2 * ph + 1], Q);
     }
-    block_sum<10, double>(Q, sm.red + (it & 1) * sm.red_n);
+    block_sum_fp64<10>(Q, sm.red);
   }
 
   // ---- outputs

@@ -10,8 +10,7 @@
 //    scratch (32 x 32 has four dofs per thread);
 //  * the step scalars are formed by one thread (division and comparison are FP64 instructions too) with a refined
 //    reciprocal (a division is about nine), and both inner products go through one shuffle tree;
-//  * the stress is added straight into the sums over a Gauss line, J > 0 is an integer test, and the part of the
-//    neo-Hookean tangent that is the same matrix for every element is added once, scaled by mu.
+//  * the part of the neo-Hookean tangent that is the same matrix for every element is added once, scaled by mu.
 // Measured on a GB300, one pass from a committed state, against the node-pair layout of rve2d.cuh with TA = double:
 // at 512 threads (first figure) and at one thread per node pair (second).  64 RVEs of 8 x 8: 3.18, 2.45 -> 0.71 ms;
 // 100 of 32 x 32: 18.3, 18.3 -> 12.4 ms; 150 of 16 x 16 through the no-allocation entry: 16.3, 8.6 -> 5.2 ms.
@@ -47,8 +46,8 @@ __host__ __device__ constexpr OffsetsD2 offsets_d2(int NN, bool mg) {
   o.p = take(sizeof(double) * 4 * NN);       // two alternating exchange buffers
   o.x = take(sizeof(double) * 2 * NN);
   o.stage = take(sizeof(double) * 16 * NN);  // element forces [8][NN]; condensation X [4][2 NN], L [4][2 NN]
-  o.red = take(sizeof(double) * (2 * 16 * 10 + 40));
-  o.lame = take(sizeof(double) * 2 * kMaxPhase);
+  o.red = take(sizeof(double) * (kBlockSumDoubles + 40));
+  o.lame = take(sizeof(double) * (2 * kMaxPhase + kResidualTable));
   o.misc = take(sizeof(double) * 16);
   int n = 2;
   while (n * n < NN) ++n;
@@ -66,24 +65,6 @@ __host__ __device__ constexpr long long scratch_d2(int NN, bool mg) {
   return 72LL * NN + (mg ? mg_fast_elems(n) + mg_slow_elems(n) : 0);
 }
 
-__device__ __forceinline__ bool positive_d(double x) {  // x > 0 (false for NaN) by integer comparison
-  const long long b = __double_as_longlong(x);
-  return b > 0 && b <= 0x7ff0000000000000ll;
-}
-
-// 1 / x for finite positive normal x (exponent split off, FP32 reciprocal of the mantissa refined twice); else 1 / x
-__device__ __forceinline__ double recip_d(double x) {
-  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
-  if (e == 0 || e > 2040 || hi < 0) return 1.0 / x;
-  const double m = __hiloint2double((hi & 0xfffff) | (1023 << 20), __double2loint(x));
-  float f;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"((float)m));
-  double q = (double)f;
-  const double err = fma(-m, q, 1.0);
-  q = fma(q, fma(err, err, err), q);
-  return __hiloint2double(__double2hiint(q) + ((1023 - e) << 20), __double2loint(q));
-}
-
 __device__ __forceinline__ double other(double v) { return __shfl_xor_sync(0xffffffffu, v, 1); }  // the pair's lane
 
 template <int DPT, int LAW>
@@ -91,7 +72,7 @@ struct D2 {
   int n, NN, ND, T, bc;
   const uint8_t* phase;
   // shared memory
-  double *w, *p, *x, *stage, *red, *lame, *misc;
+  double *w, *p, *x, *stage, *red, *lame, *restab, *misc;
   // block scratch
   double *ke;     // staged element tangents [36][NN]
   double *st;     // stencil [18][2 NN] (DPT = 4)
@@ -142,76 +123,6 @@ __device__ __forceinline__ Elem2 elem2(int k, int n, int NN) {
   q.nd[2] = ip + n * jp;
   q.nd[3] = i + n * jp;
   return q;
-}
-
-// Element forces into stage[k][e] (k = 2 local node + comp), sums of P and the count of J <= 0 (see
-// element_residual for the Gauss-line sums; P = mu F + c cof F is added straight into them).
-template <int DPT, int LAW>
-__device__ __forceinline__ void residual_d2(const D2<DPT, LAW>& s, double (&Psum)[4], int& nbad) {
-  const int half = threadIdx.x & 1;
-  const double ih = (double)s.n, t = gauss01(half);
-  const double2* w = reinterpret_cast<const double2*>(s.w);
-  const double Fb[4] = {s.misc[0], s.misc[1], s.misc[2], s.misc[3]};
-  for (int k0 = 0; k0 < s.NN; k0 += s.T / 2) {
-    const Elem2 q = elem2(k0 + (threadIdx.x >> 1), s.n, s.NN);
-    const int ph = s.phase[q.e];
-    const double lam = s.lame[2 * ph], mu = s.lame[2 * ph + 1];
-    const double2 w0 = w[q.nd[0]], w1 = w[q.nd[1]], w2 = w[q.nd[2]], w3 = w[q.nd[3]];
-    const double2 d10 = make_double2(w1.x - w0.x, w1.y - w0.y), d30 = make_double2(w3.x - w0.x, w3.y - w0.y);
-    const double2 e1 = make_double2((w2.x - w3.x) - d10.x, (w2.y - w3.y) - d10.y);
-    const double2 e2 = make_double2((w2.x - w1.x) - d30.x, (w2.y - w1.y) - d30.y);
-    const double F00 = fma(ih, fma(t, e1.x, d10.x), Fb[0]), F10 = fma(ih, fma(t, e1.y, d10.y), Fb[2]);
-    double q0x, q0y, q1x[2], q1y[2];  // P's first column on this line, its second column per s (this line's share)
-    if constexpr (LAW == kLawNH) {
-      q0x = 2.0 * mu * F00;
-      q0y = 2.0 * mu * F10;
-    } else {
-      q0x = q0y = 0.0;
-    }
-    const double hl = 0.5 * lam, hk = hl + mu;
-#pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      const double sg = gauss01(g);
-      const double F01 = fma(ih, fma(sg, e2.x, d30.x), Fb[1]), F11 = fma(ih, fma(sg, e2.y, d30.y), Fb[3]);
-      const double J = fma(F00, F11, -F01 * F10);
-      if (q.in && !positive_d(J)) ++nbad;
-      if constexpr (LAW == kLawNH) {
-        const double c = fma(hl, J, -hk * recip_fp64(J));
-        q0x = fma(c, F11, q0x);
-        q0y = fma(-c, F01, q0y);
-        q1x[g] = fma(mu, F01, -c * F10);
-        q1y[g] = fma(mu, F11, c * F00);
-      } else {
-        double P00, P01, P10, P11;
-        law2_P<LAW, double>(F00, F01, F10, F11, lam, mu, P00, P01, P10, P11);
-        q0x += P00;
-        q0y += P10;
-        q1x[g] = P01;
-        q1y[g] = P11;
-      }
-    }
-    if (q.in) {
-      Psum[0] += q0x;
-      Psum[1] += q1x[0] + q1x[1];
-      Psum[2] += q0y;
-      Psum[3] += q1y[0] + q1y[1];
-    }
-    // lane 0 of the pair forms the x forces, lane 1 the y forces
-    const double o0 = other(half ? q0x : q0y), o1 = other(half ? q1x[0] : q1y[0]), o2 = other(half ? q1x[1] : q1y[1]);
-    const double mine = half ? q0y : q0x;
-    const double a0 = half ? o0 : mine, a1 = half ? mine : o0;  // first column at t = g0, g1
-    const double b0 = (half ? q1y[0] : q1x[0]) + o1, b1 = (half ? q1y[1] : q1x[1]) + o2;
-    const double k = 0.25 / ih, kg0 = k * gauss01(0), kg1 = k * gauss01(1);
-    const double Sa0 = fma(kg1, a0, kg0 * a1), Sa1 = fma(kg0, a0, kg1 * a1);
-    const double Sb0 = fma(kg1, b0, kg0 * b1), Sb1 = fma(kg0, b0, kg1 * b1);
-    if (q.in) {
-      double* f = s.stage + half * s.NN + q.e;
-      f[0 * s.NN] = -Sa0 - Sb0;
-      f[2 * s.NN] = Sa0 - Sb1;
-      f[4 * s.NN] = Sa1 + Sb1;
-      f[6 * s.NN] = -Sa1 + Sb0;
-    }
-  }
 }
 
 // Element tangents (36 upper-triangle entries) into ke[tri][e]; each lane adds its line's two points, then the
@@ -443,21 +354,11 @@ __device__ void coarse_cycle_d2(const MgCtx<double>& mg) {
     restrict_smooth_d2(mg, l + 1, t, v.n);
     __syncthreads();
   }
-  {  // coarsest: z = A^-1 r, four lanes per row (row stride D + 1)
+  {  // coarsest: z = A^-1 r, four lanes per row
     const MgLevel<double> c = mg.level(mg.levels);
-    const int D = 2 * c.NN, ld = D + 1, l4 = tid & 3;
-    const double* A = mg.coarsest_inverse();
-    const double* r = reinterpret_cast<const double*>(c.r);
-    for (int row0 = 0; row0 < D; row0 += T >> 2) {
-      const int row = row0 + (tid >> 2);
-      if (row0 + ((tid & ~31) >> 2) >= D) continue;  // a whole warp past the end
-      double z = 0.0;
-      if (row < D)
-        for (int q = l4; q < D; q += 4) z = fma(A[(size_t)row * ld + q], r[q], z);
-      z += __shfl_xor_sync(0xffffffffu, z, 1);
-      z += __shfl_xor_sync(0xffffffffu, z, 2);
-      if (row < D && l4 == 0) reinterpret_cast<double*>(c.z)[row] = pinned2((row >> 1) % c.n, (row >> 1) / c.n, c.bc) ? 0.0 : z;
-    }
+    const double z = coarsest_row<double>(mg.coarsest_inverse(), reinterpret_cast<const double*>(c.r), 2 * c.NN);
+    const int row = tid >> 2;
+    if (row < 2 * c.NN && (tid & 3) == 0) reinterpret_cast<double*>(c.z)[row] = pinned2((row >> 1) % c.n, (row >> 1) / c.n, c.bc) ? 0.0 : z;
     __syncthreads();
   }
   for (int l = mg.levels - 1; l >= 1; --l) {
@@ -560,46 +461,7 @@ __device__ void mg_build_d2(const MgCtx<double>& mg, const double* ke) {
       }
     }
   }
-  // coarsest: dense pinned matrix, then its inverse by Gauss-Jordan (as in mg_build_part2)
-  const MgLevel<double> c = mg.level(mg.levels);
-  const int D = 2 * c.NN, ld = D + 1;
-  double* A = mg.coarsest_inverse();
-  double* B = A + (size_t)D * ld;
-  if (tid < D) {
-    const int node = tid >> 1, ii = tid & 1, ni = node % c.n, nj = node / c.n;
-    for (int q = 0; q < D; ++q) A[(size_t)tid * ld + q] = 0.0;
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const int ei = (ni - offx(l) + c.n) % c.n, ej = (nj - offy(l) + c.n) % c.n, slot = ei + c.n * ej;
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const int nm = (ei + offx(m)) % c.n + c.n * ((ej + offy(m)) % c.n);
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk)
-          A[(size_t)tid * ld + 2 * nm + kk] += c.ke[(size_t)tri8(2 * l + ii, 2 * m + kk) * c.NN + slot];
-      }
-    }
-    if (pinned2(ni, nj, c.bc)) {
-      for (int q = 0; q < D; ++q) A[(size_t)tid * ld + q] = q == tid ? 1.0 : 0.0;
-    } else {
-      for (int q = 0; q < D; q += 2)
-        if (pinned2((q >> 1) % c.n, (q >> 1) / c.n, c.bc)) A[(size_t)tid * ld + q] = A[(size_t)tid * ld + q + 1] = 0.0;
-    }
-  }
-  __syncthreads();
-  const int j = tid & 31, warp = tid >> 5, nw = T >> 5;
-  for (int k = 0; k < D; ++k) {  // SPD: no pivoting; D is even, so the result ends in A
-    const double* Ao = (k & 1) ? B : A;
-    double* An = (k & 1) ? A : B;
-    if (warp < D && j < D) {
-      const double ip = recip_d(Ao[(size_t)k * ld + k]), kj = Ao[(size_t)k * ld + j] * ip;
-      for (int i = warp; i < D; i += nw) {
-        const double aik = Ao[(size_t)i * ld + k];
-        An[(size_t)i * ld + j] = i == k ? (j == k ? ip : kj) : j == k ? -aik * ip : fma(-aik, kj, Ao[(size_t)i * ld + j]);
-      }
-    }
-    __syncthreads();
-  }
+  mg_invert_coarsest<double>(mg);
 }
 
 // ------------------------------------------------------------------ PCG
@@ -673,7 +535,7 @@ __device__ int pcg_d2(const D2<DPT, LAW>& s, const Row<DPT>& R, const double (&M
 #pragma unroll
     for (int q = 0; q < DPT; ++q) u[q] = fma(om, jacobi(q, r[q] - w[q]), u[q]);
   };
-  double* red = s.red + 2 * 16 * 10;
+  double* red = s.red + kBlockSumDoubles;
   double* out = red + 32;  // alpha, beta; [2] the decision
   auto dots = [&](bool both, double& g, double& d) {  // valid in warp 0
     double a = 0.0, e = 0.0;
@@ -875,6 +737,7 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
   s.stage = reinterpret_cast<double*>(smem + off.stage);
   s.red = reinterpret_cast<double*>(smem + off.red);
   s.lame = reinterpret_cast<double*>(smem + off.lame);
+  s.restab = s.lame + 2 * kMaxPhase;
   s.misc = reinterpret_cast<double*>(smem + off.misc);
   s.ke = scr;
   s.st = scr + 36 * (size_t)NN;
@@ -910,7 +773,9 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
   const double* w_in = a.w_in + w_off;
   double* w_out = a.w_out + w_off;
   if (tid < 4) s.misc[tid] = a.F[(size_t)qp * 4 + tid];
-  if (tid < 2 * kMaxPhase) s.lame[tid] = a.rve_lame[(size_t)rv * 2 * kMaxPhase + tid];
+  const double* lame_g = a.rve_lame + (size_t)rv * 2 * kMaxPhase;
+  if (tid < 2 * kMaxPhase) s.lame[tid] = lame_g[tid];
+  residual_table(n, lame_g, s.restab);
 #pragma unroll
   for (int q = 0; q < DPT; ++q)
     if (s.act[q]) s.w[s.dof[q]] = s.pin[q] ? 0.0 : w_in[s.dof[q]];
@@ -925,11 +790,8 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
   double* Lb = s.stage + 4 * ND;   // [4][ND]
   Row<DPT> R;
   double Mi[DPT][2];
-  int status = kStatusNewtonCap, it = 0, cg_total = 0, red_k = 0;
+  int status = kStatusNewtonCap, it = 0, cg_total = 0;
   double Psum[4];
-  auto red = [&]() {  // the two buffers of the sums over the block, in turn
-    return s.red + (red_k++ & 1) * 160;
-  };
   // Newton with step halving, rebuild-and-retry and load continuation exactly as solve_item_2d (the reasons stand
   // there)
   for (;;) {
@@ -940,8 +802,8 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
     for (;;) {
       Psum[0] = Psum[1] = Psum[2] = Psum[3] = 0.0;
       int nbad = 0;
-      residual_d2(s, Psum, nbad);
-      __syncthreads();
+      block_residual<LAW>(n, reinterpret_cast<const double2*>(s.w), s.misc, s.restab, s.phase, s.stage, Psum, nbad);
+      const bool bad = __syncthreads_or(nbad);
       double Rv[DPT], v2[1] = {0.0};
 #pragma unroll
       for (int q = 0; q < DPT; ++q) {
@@ -951,8 +813,7 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
         if (!s.act[q] || s.pin[q]) Rv[q] = 0.0;
         v2[0] = fma(Rv[q], Rv[q], v2[0]);
       }
-      block_sum<1, double>(v2, red());
-      const bool bad = __syncthreads_or(nbad);
+      block_sum_fp64<1>(v2, s.red);
       const double rn = sqrt(v2[0]);
       if (it == 0) r0 = rn;
       if ((bad || !isfinite(rn)) && it > 0 && nhalf < kMaxStepHalvings) {
@@ -1046,7 +907,7 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
       const int ph = s.phase[e];
       Pv[4] += element_energy<LAW>(e, n, reinterpret_cast<const double2*>(s.w), s.misc, s.lame[2 * ph], s.lame[2 * ph + 1]);
     }
-  block_sum<5, double>(Pv, red());
+  block_sum_fp64<5>(Pv, s.red);
 
   int cond_total = 0, cond_max = 0;
   double Q[10];
@@ -1100,7 +961,7 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
 #pragma unroll
     for (int k = 0; k < 10; ++k) Q[k] = 0.0;
     transfer_d2(s, Xs, Q);
-    block_sum<10, double>(Q, red());
+    block_sum_fp64<10>(Q, s.red);
   }
 
 #pragma unroll

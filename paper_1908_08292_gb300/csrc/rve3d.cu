@@ -533,19 +533,6 @@ __device__ __forceinline__ TA* smem_vin() {
   return reinterpret_cast<TA*>(smem3 + kSmem3Fixed);
 }
 
-template <typename T>
-__device__ __forceinline__ void block_sum_n(T* v, int nv, T* buf) {
-  // nv <= 16 values; buf >= 32*16
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int k = 0; k < nv; ++k) {
-    T x = warp_sum(v[k]);
-    if (lane == 0) buf[k * 32 + warp] = x;
-  }
-  __syncthreads();
-  for (int k = 0; k < nv; ++k) v[k] = warp_sum(lane < nw ? buf[k * 32 + lane] : T(0));
-  __syncthreads();
-}
-
 template <typename TA>
 struct Mg3Level {
   int n, NN, bc;
@@ -622,19 +609,13 @@ struct Ctx3 {
 // straight into the sums over the points that share a shape gradient (mu F of a column is the same for both),
 // <P> from those sums, J <= 0 read from the sign bit: about 430 per lane.  Evaluated point by point with the
 // general gradient it took about 2400 per element (16^3: 4.6 million cycles an evaluation).
-__device__ __forceinline__ bool is_positive(double x) {  // x > 0 (false for NaN) by integer comparison
-  const long long b = __double_as_longlong(x);
-  return b > 0 && b <= 0x7ff0000000000000ll;
-}
-
 template <typename TA, int LAW>
-__device__ __noinline__ void residual3(const Ctx3<TA>& c, double (&Psum)[9], double& bad) {
+__device__ __noinline__ void residual3(const Ctx3<TA>& c, double (&Psum)[9], int& nbad) {
   const int n = c.g.n, NE = c.NE, magic = c.magic;
   const double* w = c.w;
   const uint8_t* __restrict__ phase = c.phase;
   double* Rf = c.sc.Rf;
   const double ih = (double)n, cw = 0.125 / (ih * ih);  // wq / h = h^2 / 8
-  int nbad = 0;
   for (int pass = 0; pass * (int)(blockDim.x / 2) < NE; ++pass) {
     const Cell3 q = cell3(pass, n, NE, magic, 0);
     const int ph = phase[q.in ? q.e : 0];
@@ -676,7 +657,7 @@ __device__ __noinline__ void residual3(const Ctx3<TA>& c, double (&Psum)[9], dou
                              fx[2][gy], fy[2][gx], fz[2][gy][gx]};
         double cof[9];
         const double J = cofactors(F, cof);
-        if (q.in && !is_positive(J)) ++nbad;
+        if (q.in && !positive_fp64(J)) ++nbad;
         if constexpr (LAW == kLawNH) {
           // P = mu F + hb F^-T = mu F + (hb / J) cof(F), hb / J = lam J / 2 - (lam / 2 + mu) / J
           const double cc = fma(0.5 * lam, J, -(0.5 * lam + mu) * recip_fp64(J));
@@ -720,7 +701,6 @@ __device__ __noinline__ void residual3(const Ctx3<TA>& c, double (&Psum)[9], dou
       }
     }
   }
-  bad += (double)nbad;
 }
 
 // sum over this thread's elements of psi at the Gauss points (FP64; Eq. NH-free-energy)
@@ -1630,20 +1610,20 @@ __device__ int pcg3(const Ctx3<TA>& c, TA rtol, int max_it, bool truncate, int* 
     __syncthreads();
     if (c.mg.levels) mg3_vcycle_fine<TA, LAW>(c, r);
   };
-  // inner products: per thread and per warp in TA, over the block in FP64 (block_dot2_fp64); the
+  // inner products: per thread and per warp in TA, over the block in FP64 (block_dot2); the
   // stopping test compares FP64 sums, the step scalars are formed in TA from them
-  auto dots = [&](double& gam, double& del) {
+  double stop = 0.0, wide = 0.0;  // valid in warp 0
+  auto dots = [&](TA& gam, TA& del) {
     TA g = TA(0), d = TA(0);
 #pragma unroll 4
     for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) {
       g += r[v] * vin[v];
       d += vout[v] * vin[v];
     }
-    block_dot2_fp64<TA>(g, d, c.red + 2 * 512 - 64, gam, del);
+    return block_dot2<TA>(g, d, c.red + 2 * 512 - 64, stop, gam, del, wide);
   };
   *status = kStatusOk;
-  double gref = -1.0;  // stopping reference b^T M^-1 b of a warm start
-  int it = 0;
+  int it = 0, fref = kDotNonNeg;
   smooth_to_vin();
   if (!warm) {
 #pragma unroll 4
@@ -1655,8 +1635,9 @@ __device__ int pcg3(const Ctx3<TA>& c, TA rtol, int max_it, bool truncate, int* 
     {
       TA g = TA(0);
       for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) g += r[v] * vin[v];
-      double unused;
-      block_dot2_fp64<TA>(g, TA(0), c.red + 2 * 512 - 64, gref, unused);
+      TA unused0, unused1;  // the stopping reference b^T M^-1 b
+      fref = block_dot2<TA>(g, TA(0), c.red + 2 * 512 - 64, 0.0, unused0, unused1, wide);
+      if (threadIdx.x < 32) stop = (double)rtol * (double)rtol * wide;
     }
 #pragma unroll 4
     for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) vin[v] = x[v];
@@ -1670,24 +1651,22 @@ __device__ int pcg3(const Ctx3<TA>& c, TA rtol, int max_it, bool truncate, int* 
   }
   precond_rest();
   apply3<TA, LAW>(c);
-  double gd, dd;
-  dots(gd, dd);
-  TA gamma = (TA)gd, delta = (TA)dd;
-  const double gamma0 = gd;
-  const double stop = (double)rtol * (double)rtol * (warm ? gref : gamma0);
+  TA gamma, delta;
+  const int f0 = dots(gamma, delta);
+  if (!warm && threadIdx.x < 32) stop = (double)rtol * (double)rtol * wide;
   // a non-finite or negative preconditioned residual norm r^T M^-1 r (the preconditioner is not
   // positive definite) is a breakdown
-  if (!isfinite(gamma0) || gamma0 < 0.0 || (warm && !(gref >= 0.0))) {
+  if (!(f0 & kDotFinite) || !(f0 & kDotNonNeg) || !(fref & kDotNonNeg)) {
     *status = kStatusPcgBreakdown;
     __syncthreads();
     return it;
   }
-  if (warm && gamma0 <= stop) {  // the start value already meets the tolerance
+  if (warm && (f0 & kDotStop)) {  // the start value already meets the tolerance
     __syncthreads();
     return it;
   }
-  if (!(gamma0 > 0.0)) return 0;
-  if (!(dd > 0.0)) {
+  if (!(f0 & kDotPos)) return 0;
+  if (!(f0 & kDotCurvPos)) {
     if (truncate && delta < TA(0)) {
       const TA a0 = div3(gamma, -delta);
       for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) x[v] = a0 * vin[v];
@@ -1723,15 +1702,14 @@ __device__ int pcg3(const Ctx3<TA>& c, TA rtol, int max_it, bool truncate, int* 
     }
     precond_rest();
     apply3<TA, LAW>(c);
-    double gnd, dnd;
-    dots(gnd, dnd);
-    const TA gn = (TA)gnd, dn = (TA)dnd;
+    TA gn, dn;
+    const int f = dots(gn, dn);
     ++it;
-    if (!(gnd >= 0.0)) {  // preconditioner not positive definite (or non-finite)
+    if (!(f & kDotNonNeg)) {  // preconditioner not positive definite (or non-finite)
       *status = kStatusPcgBreakdown;
       break;
     }
-    if (gnd <= stop) break;
+    if (f & kDotStop) break;
     beta = div3(gn, gamma);
     const TA den = dn - beta * div3(gn, alpha);
     if (!(den > TA(0))) {
@@ -1804,11 +1782,11 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
     double r0 = 0.0, step = 1.0;
     status = kStatusNewtonCap;
     for (;;) {
-      double bad = 0.0;
+      int nbad = 0;
 #pragma unroll
       for (int k = 0; k < 9; ++k) Psum[k] = 0.0;
-      residual3<TA, LAW>(c, Psum, bad);
-      __syncthreads();
+      residual3<TA, LAW>(c, Psum, nbad);
+      const bool bad = __syncthreads_or(nbad);
       double rr = 0.0;
       for (int v = threadIdx.x; v < NN; v += blockDim.x) {
         double R[3];
@@ -1820,11 +1798,11 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
           c.sc.r[d * NN + v] = (TA)(-R[d]);  // right-hand side of the Newton correction
         }
       }
-      double v2[2] = {rr, bad};
-      block_sum_n<double>(v2, 2, c.red);
+      double v2[1] = {rr};
+      block_sum_fp64<1>(v2, c.red);
       const double rn = sqrt(v2[0]);
       if (it == 0) r0 = rn;
-      if ((v2[1] > 0.0 || !isfinite(rn)) && it > 0 && nhalf < kMaxStepHalvings) {
+      if ((bad || !isfinite(rn)) && it > 0 && nhalf < kMaxStepHalvings) {
         // backtrack: w = w_prev + step x  ->  w_prev + (step/2) x
         ++nhalf;
         step *= 0.5;
@@ -1836,7 +1814,7 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
         __syncthreads();
         continue;
       }
-      if (v2[1] > 0.0) {
+      if (bad) {
         status = kStatusJNonPos;
         break;
       }
@@ -1928,7 +1906,7 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
   for (int k = 0; k < 9; ++k) Pv[k] = Psum[k];
   const bool want_W = usable && (a.flags & kFlagEnergy) && a.W != nullptr;
   Pv[9] = want_W ? energy3<TA, LAW>(c, w) : 0.0;
-  block_sum_n<double>(Pv, 10, c.red);
+  block_sum_fp64<10>(Pv, c.red);
   if (threadIdx.x == 0)
     for (int k = 0; k < 10; ++k) misc[k] = Pv[k];
 
@@ -1944,8 +1922,16 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
     // hits its cap with them is run again with levels rebuilt at the converged state
     bool reuse_t = c.mg.levels && a.mg_reuse && it > 0;
     if (c.mg.levels && !reuse_t) mg3_build<TA, LAW>(c);
-    // <A>: 45 FP64 sums in three reductions of 15
-    for (int part = 0; part < 3; ++part) block_sum_n<double>(As + 15 * part, 15, c.red);
+    // <A>: 45 FP64 sums in five reductions of 9
+#pragma unroll
+    for (int part = 0; part < 5; ++part) {
+      double sum[9];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) sum[k] = As[9 * part + k];
+      block_sum_fp64<9>(sum, c.red);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) As[9 * part + k] = sum[k];
+    }
     // right-hand sides L_c (c = 3k + L) stored [c][3][NN]
     for (int cc = 0; cc < 9; ++cc) {
       unit_gradient3<TA, LAW>(c, cc);
@@ -1994,7 +1980,7 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
 #pragma unroll
         for (int cc = 0; cc < 9; ++cc) col[cc] += (double)c.sc.L[(size_t)cc * 3 * NN + v] * xv;
       }
-      block_sum_n<double>(col, 9, c.red);
+      block_sum_fp64<9>(col, c.red);
       if (threadIdx.x == 0)
         for (int cc = 0; cc < 9; ++cc) LX[9 * cc + cp] = col[cc];
     }

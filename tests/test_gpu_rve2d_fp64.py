@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import synth
-from gpu_harness import rel_err
+from gpu_harness import gpu_batch, rel_err
 from oracle.rve import PeriodicRVE
 
 pytestmark = pytest.mark.gpu
@@ -49,3 +49,16 @@ def test_layout_edges(law, precond):
                 assert rel_err(P[q].cpu().numpy(), ref["P"], 1e-3) < TOL, n
                 assert rel_err(A[q].cpu().numpy(), ref["A"], 1e-3) < TOL, n
                 assert abs(float(W[q]) - ref["W"]) <= TOL * max(abs(ref["W"]), 1e-3), n
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [6, 10])
+def test_collapsed_point_is_reported(precision, n):
+    """det F = 1e-50, below the range of the residual's FP32 reciprocal: the point fails, as with det F <= 0, and does
+    not disturb its neighbour in the batch.  n = 6: two lanes per element, n = 10 one."""
+    phase = synth.phase_from_inclusions(n, 2, [[0.5, 0.5]], [0.25])
+    Fs = np.stack([1e-25 * np.eye(2), np.array([[1.02, 0.01], [0.0, 0.99]])])
+    out = gpu_batch(2, precision, [n], [phase], [[1.0, 10.0]], [[0.3, 0.3]], [0, 0], Fs)
+    ref = PeriodicRVE(n, 2, phase, [1.0, 10.0], [0.3, 0.3]).solve(Fs[1], rtol=1e-14, atol=1e-16)
+    assert out["status"][0] != 0 and out["status"][1] == 0
+    assert rel_err(out["P"][1], ref["P"], 1e-3) < 1e-5  # default tolerances in both modes
