@@ -128,6 +128,27 @@ __host__ __device__ constexpr long long mg_slow_max(int nn_max) {
   return m;
 }
 
+// What a Newton iteration does after its residual: a final status, one more step (-1), or half the last step (-2).
+// Thread 0 decides for the block: the root and the comparisons are some twenty FP64 instructions a warp.  r0, the
+// first residual norm, is kept by thread 0; slot is shared.
+constexpr int kNewtonGoOn = -1, kNewtonHalve = -2;
+__device__ __forceinline__ int newton_code(bool bad, double r2, int it, int nhalf, double& r0, double rtol, double atol, int cap,
+                                           int* slot) {
+  if (threadIdx.x == 0) {
+    int code;
+    const double rn = sqrt(r2);
+    if (it == 0) r0 = rn;
+    if ((bad || !isfinite(rn)) && it > 0 && nhalf < kMaxStepHalvings) code = kNewtonHalve;
+    else if (bad) code = kStatusJNonPos;
+    else if (!isfinite(rn)) code = kStatusNonFinite;
+    else if (rn <= fmax(rtol * r0, atol)) code = kStatusOk;
+    else code = it >= cap ? kStatusNewtonCap : kNewtonGoOn;
+    *slot = code;
+  }
+  __syncthreads();
+  return *slot;
+}
+
 constexpr int kResidualTable = 2 + 4 * kMaxPhase;  // doubles of the residual's constants (residual_table)
 
 template <typename TA>
@@ -902,6 +923,43 @@ __device__ __forceinline__ double dense_update(double a, double aik, double, dou
 __device__ __forceinline__ float dense_recip(float x) { return 1.f / x; }
 __device__ __forceinline__ double dense_recip(double x) { return recip_d(x); }
 
+// Inverse of the D x D matrix A (row stride D + 1) into I (row stride D + 4), ROWS rows per warp in registers, a column
+// per lane.  Straight-line code over the rows: they are independent within a step.
+template <int ROWS, typename TA>
+__device__ __forceinline__ void dense_invert(const TA* A, int D, TA* piv, TA* I) {
+  const int j = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  TA a[ROWS];
+#pragma unroll
+  for (int q = 0; q < ROWS; ++q) {
+    const int i = warp + nw * q;
+    a[q] = i < D && j < D ? A[(size_t)i * (D + 1) + j] : TA(0);
+  }
+  if (warp == 0) piv[j] = a[0];
+  __syncthreads();
+#pragma unroll 1
+  for (int k = 0; k < D; ++k) {  // SPD: no pivoting
+    const TA* pk = piv + 32 * (k & 1);
+    const TA ip = dense_recip(pk[k]), akj = pk[j], kj = akj * ip;
+    const bool own = j == k;
+    TA* next = piv + 32 * ((k + 1) & 1) + j;
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+      const int i = warp + nw * q;
+      const TA aik = __shfl_sync(0xffffffffu, a[q], k);
+      const TA v = dense_update(a[q], aik, akj, ip, kj, own);
+      a[q] = i == k ? (own ? ip : kj) : v;
+      if (i == k + 1) *next = a[q];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < ROWS; ++q) {
+    const int i = warp + nw * q;
+    if (i < D && j < D) I[(size_t)i * (D + 4) + j] = a[q];
+  }
+  __syncthreads();
+}
+
 // Dense pinned matrix of the coarsest level (one row per thread) and its inverse by Gauss-Jordan elimination: the
 // matrix in registers, a column per lane and the rows dealt to the warps, so that a step has one barrier and moves
 // only the pivot row through shared memory.  (With the matrix in shared memory a step took 2300 cycles at four warps,
@@ -936,36 +994,8 @@ __device__ __forceinline__ void mg_invert_coarsest(const MgCtx<TA>& mg) {
     }
   }
   __syncthreads();
-  const int j = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  TA a[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int i = warp + nw * q;
-    a[q] = i < D && j < D ? A[(size_t)i * ld + j] : TA(0);
-  }
-  if (warp == 0) piv[j] = a[0];
-  __syncthreads();
-  for (int k = 0; k < D; ++k) {  // SPD: no pivoting
-    const TA* pk = piv + 32 * (k & 1);
-    const TA ip = dense_recip(pk[k]), akj = pk[j], kj = akj * ip;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int i = warp + nw * q;  // uniform in the warp
-      if (i >= D) break;
-      const TA aik = __shfl_sync(0xffffffffu, a[q], k);
-      if (i == k) a[q] = j == k ? ip : kj;
-      else a[q] = dense_update(a[q], aik, akj, ip, kj, j == k);
-      if (i == k + 1) piv[32 * ((k + 1) & 1) + j] = a[q];
-    }
-    __syncthreads();
-  }
-  TA* I = mg.coarsest_inverse();
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int i = warp + nw * q;
-    if (i < D && j < D) I[(size_t)i * (D + 4) + j] = a[q];
-  }
-  __syncthreads();
+  if ((int)(blockDim.x >> 5) * 4 >= D) dense_invert<4, TA>(A, D, piv, mg.coarsest_inverse());
+  else dense_invert<8, TA>(A, D, piv, mg.coarsest_inverse());
 }
 
 template <typename TA>
@@ -1497,7 +1527,7 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
   // equal increments of Fbar - I.
   // The stage counters live in shared memory (block-uniform) to keep them out of the registers
   // of the PCG loop.
-  __shared__ int s_ctl[3];  // stages, stage, Newton iterations of the earlier stages
+  __shared__ int s_ctl[4];  // stages, stage, Newton iterations of the earlier stages, newton_code
   if (tid == 0) {
     s_ctl[0] = 1;
     s_ctl[1] = 1;
@@ -1532,9 +1562,9 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
       }
       double v2[1] = {R[0] * R[0] + R[1] * R[1] + R[2] * R[2] + R[3] * R[3]};
       block_sum_fp64<1>(v2, sm.red);
-      const double rn = sqrt(v2[0]);
-      if (it == 0) r0 = rn;
-      if ((bad || !isfinite(rn)) && it > 0 && nhalf < kMaxStepHalvings) {
+      const int code = newton_code(bad, v2[0], it, nhalf, r0, a.newton_rtol, a.newton_atol,
+                                   s_ctl[0] > 1 ? max(a.max_newton, kRetryNewtonCap) : a.max_newton, s_ctl + 3);
+      if (code == kNewtonHalve) {
         // backtrack: w = w_prev + step x  ->  w_prev + (step/2) x
         ++nhalf;
         step *= 0.5;
@@ -1553,20 +1583,8 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
         __syncthreads();
         continue;
       }
-      if (bad) {
-        status = kStatusJNonPos;
-        break;
-      }
-      if (!isfinite(rn)) {
-        status = kStatusNonFinite;
-        break;
-      }
-      if (rn <= fmax(a.newton_rtol * r0, a.newton_atol)) {
-        status = kStatusOk;
-        break;
-      }
-      if (it >= (s_ctl[0] > 1 ? max(a.max_newton, kRetryNewtonCap) : a.max_newton)) {
-        status = kStatusNewtonCap;
+      if (code >= 0) {
+        status = code;
         break;
       }
       // ---- tangent and PCG correction.  The multigrid's coarse levels are built at the first

@@ -779,7 +779,7 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
 #pragma unroll
   for (int q = 0; q < DPT; ++q)
     if (s.act[q]) s.w[s.dof[q]] = s.pin[q] ? 0.0 : w_in[s.dof[q]];
-  __shared__ int s_ctl[3];  // stages, stage, Newton iterations of the earlier stages
+  __shared__ int s_ctl[4];  // stages, stage, Newton iterations of the earlier stages, newton_code
   if (tid == 0) {
     s_ctl[0] = 1;
     s_ctl[1] = 1;
@@ -814,9 +814,9 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
         v2[0] = fma(Rv[q], Rv[q], v2[0]);
       }
       block_sum_fp64<1>(v2, s.red);
-      const double rn = sqrt(v2[0]);
-      if (it == 0) r0 = rn;
-      if ((bad || !isfinite(rn)) && it > 0 && nhalf < kMaxStepHalvings) {
+      const int code = newton_code(bad, v2[0], it, nhalf, r0, a.newton_rtol, a.newton_atol,
+                                   s_ctl[0] > 1 ? max(a.max_newton, kRetryNewtonCap) : a.max_newton, s_ctl + 3);
+      if (code == kNewtonHalve) {
         ++nhalf;
         step *= 0.5;
 #pragma unroll
@@ -825,20 +825,8 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
         __syncthreads();
         continue;
       }
-      if (bad) {
-        status = kStatusJNonPos;
-        break;
-      }
-      if (!isfinite(rn)) {
-        status = kStatusNonFinite;
-        break;
-      }
-      if (rn <= fmax(a.newton_rtol * r0, a.newton_atol)) {
-        status = kStatusOk;
-        break;
-      }
-      if (it >= (s_ctl[0] > 1 ? max(a.max_newton, kRetryNewtonCap) : a.max_newton)) {
-        status = kStatusNewtonCap;
+      if (code >= 0) {
+        status = code;
         break;
       }
       bool reuse = kMG && s.mg.levels && a.mg_reuse && it > 0;
