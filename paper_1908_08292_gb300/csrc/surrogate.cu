@@ -268,55 +268,35 @@ struct CombineParams {
   double poly[kPolyTerms];
 };
 
-// Stress, tangent and energy at 32 points per block (one per lane).  Bound by the FP64 pipe (a quarter of
-// 2 lanes a cycle per SM sub-partition), so the FP64 work of a point is spread over the block's 8 warps:
+// Stress, tangent and energy at 32 points per tile (one per lane).  Bound by the FP64 pipe (a warp instruction holds
+// an SM sub-partition for 64 cycles), so the FP64 work of a point is spread over the block's 8 warps:
 // warps 0-6 take three Hessian pairs each of the polynomial part, warp 7 the base law; then the 6 x 6
 // material tangent, and one row (i, J) of A per warp.  F, the network's Hessian and A pass through shared
-// memory, so every global access is a contiguous run.  The whole surrogate evaluation of 32768 points (degree 6), with
-// the fused network: 6.04 -> 0.76 ms, of which the network 0.19.
+// memory, so every global access is a contiguous run.  Two blocks per SM, so that one fills the pipe while the other
+// is between barriers, each building the table once for all its tiles.  32768 points, degree 6: this kernel
+// 0.55 -> 0.39 ms against one block per SM and tile, with gradient and value summed per degree; the whole evaluation
+// with the fused network 6.04 -> 0.60 ms, of which the network 0.20.
 constexpr int kCombineThreads = 256, kCombinePts = 32;
 struct CombineSmem {
-  double T[kBetas * kPairs];  // then the block's rows of A, [32][81]
-  double m[kBetas][kCombinePts];  // the monomials; the first six are x
+  double T[kBetas * kPairs];
+  double m[kBetas][kCombinePts];  // the monomials; the first six are x.  After the Hessian: cc[36] from row 6 on, then
+                                  // the tile's rows of A, [32][81]
   double F[9][kCombinePts], Ci[6][kCombinePts], S[6][kCombinePts], J2[kCombinePts];
-  double gp[7][6][kCombinePts], yp[7][kCombinePts];  // per warp: its pairs' share of gradient and value
-  double cc[36][kCombinePts];
+  double hg[kPairs][kCombinePts], hy[kPairs][kCombinePts];  // Hessian pairs weighted for gradient and value
   float H[kCombinePts * 36];
 };
-static_assert(kBetas * kPairs >= kCombinePts * 81, "A tile fits the table's place");
+static_assert(kBetas * kCombinePts >= (6 + 36) * kCombinePts + kCombinePts * 81, "cc and the A tile fit the monomials' place");
 
-__global__ void __launch_bounds__(kCombineThreads, 1)
+__global__ void __launch_bounds__(kCombineThreads, 2)
 combine_kernel(const __grid_constant__ CombineParams c, const double* F, int n, int emax, const float* y, const float* g,
                const float* H, double* P, double* A, double* Wout) {
   extern __shared__ __align__(16) unsigned char combine_smem[];
   CombineSmem& sm = *reinterpret_cast<CombineSmem*>(combine_smem);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int q0 = blockIdx.x * kCombinePts, np = min(kCombinePts, n - q0), q = q0 + lane;
   const double sq2 = 1.4142135623730950488;
   for (int e = t; e < betas_upto(emax) * kPairs; e += kCombineThreads) sm.T[e] = c.poly[kHess.idx[e]] * (double)kHess.mult[e];
-  for (int e = t; e < kCombinePts * 9; e += kCombineThreads)  // lanes past the end: F = I
-    sm.F[e % 9][e / 9] = e < np * 9 ? F[(size_t)q0 * 9 + e] : (e % 9) % 4 == 0 ? 1.0 : 0.0;
-  if (A)
-    for (int e = t; e < np * 36; e += kCombineThreads) sm.H[e] = H[(size_t)q0 * 36 + e];
-  __syncthreads();
-  double f[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) f[k] = sm.F[k][lane];
-  auto Cij = [&](int I, int J) { return f[I] * f[J] + f[3 + I] * f[3 + J] + f[6 + I] * f[6 + J]; };
-  if (warp < 6) {  // feature p = warp
-    const int I = kMandelI[warp], J = kMandelJ[warp];
-    double cij = 0.0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) cij += sm.F[3 * i + I][lane] * sm.F[3 * i + J][lane];
-    sm.m[warp][lane] = (I == J ? 1.0 : sq2) * 0.5 * (cij - (I == J ? 1.0 : 0.0)) / c.sx;
-  }
-  __syncthreads();
-  for (int e = 2; e <= emax; ++e) {  // every monomial once per point (formed by each warp they cost a third more)
-    for (int k = betas_upto(e - 1) + warp; k < betas_upto(e); k += kCombineThreads / 32)
-      sm.m[k][lane] = sm.m[kHess.up[k]][lane] * sm.m[kHess.var[k]][lane];
-    __syncthreads();
-  }
-  double W = 0.0, Hp[3] = {0.0, 0.0, 0.0};
+  double(*cc)[kCombinePts] = sm.m + 6;
+  double* tileA = &sm.m[42][0];
   int pp[3], pq[3];  // this warp's pairs (warps 0-6)
   {
     int k = 0;
@@ -327,128 +307,165 @@ combine_kernel(const __grid_constant__ CombineParams c, const double* F, int n, 
           pq[k % 3] = r;
         }
   }
-  if (warp < 7) {
-    const double* Tw = sm.T + 3 * warp;
-    double gs[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, ys = 0.0;
-    for (int e = 1; e <= emax; ++e) {  // the form of degree e + 2: monomials of degree e
-      double h0 = 0.0, h1 = 0.0, h2 = 0.0;
+  for (int q0 = blockIdx.x * kCombinePts; q0 < n; q0 += gridDim.x * kCombinePts) {
+    const int np = min(kCombinePts, n - q0), q = q0 + lane;
+    for (int e = t; e < kCombinePts * 9; e += kCombineThreads)  // lanes past the end: F = I
+      sm.F[e % 9][e / 9] = e < np * 9 ? F[(size_t)q0 * 9 + e] : (e % 9) % 4 == 0 ? 1.0 : 0.0;
+    if (A)
+      for (int e = t; e < np * 36; e += kCombineThreads) sm.H[e] = H[(size_t)q0 * 36 + e];
+    __syncthreads();
+    double f[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) f[k] = sm.F[k][lane];
+    auto Cij = [&](int I, int J) { return f[I] * f[J] + f[3 + I] * f[3 + J] + f[6 + I] * f[6 + J]; };
+    if (warp < 6) {  // feature p = warp
+      const int I = kMandelI[warp], J = kMandelJ[warp];
+      double cij = 0.0;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) cij += sm.F[3 * i + I][lane] * sm.F[3 * i + J][lane];
+      sm.m[warp][lane] = (I == J ? 1.0 : sq2) * 0.5 * (cij - (I == J ? 1.0 : 0.0)) / c.sx;
+    }
+    __syncthreads();
+    for (int e = 2; e <= emax; ++e) {  // every monomial once per point (formed by each warp they cost a third more)
+      for (int k = betas_upto(e - 1) + warp; k < betas_upto(e); k += kCombineThreads / 32)
+        sm.m[k][lane] = sm.m[kHess.up[k]][lane] * sm.m[kHess.var[k]][lane];
+      __syncthreads();
+    }
+    double W = 0.0, Hp[3] = {0.0, 0.0, 0.0};
+    if (warp < 7) {
+      const double* Tw = sm.T + 3 * warp;
+      double hg[3] = {0.0, 0.0, 0.0}, hy[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int e = 1; e <= 4; ++e) {  // the form of degree e + 2: monomials of degree e
+        if (e > emax) break;
+        double h[3] = {0.0, 0.0, 0.0};
 #pragma unroll 4
-      for (int k = betas_upto(e - 1); k < betas_upto(e); ++k) {
-        const double m = sm.m[k][lane];
-        const double* T = Tw + k * kPairs;
-        h0 = fma(T[0], m, h0);
-        h1 = fma(T[1], m, h1);
-        h2 = fma(T[2], m, h2);
+        for (int k = betas_upto(e - 1); k < betas_upto(e); ++k) {
+          const double m = sm.m[k][lane];
+          const double* T = Tw + k * kPairs;
+#pragma unroll
+          for (int r = 0; r < 3; ++r) h[r] = fma(T[r], m, h[r]);
+        }
+        const double rg = 1.0 / (e + 1), ry = 1.0 / ((e + 1) * (e + 2));
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          Hp[r] += h[r];
+          hg[r] = fma(rg, h[r], hg[r]);
+          hy[r] = fma(ry, h[r], hy[r]);
+        }
       }
-      const double hs[3] = {h0, h1, h2}, rg = 1.0 / (e + 1), ry = rg / (e + 2);
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        sm.hg[3 * warp + r][lane] = hg[r];
+        sm.hy[3 * warp + r][lane] = hy[r];
+      }
+    } else {  // base law: S = lam/2 (J^2-1) C^-1 + mu (I - C^-1), plus the anisotropic small-strain part
+      double C[9];
+#pragma unroll
+      for (int I = 0; I < 3; ++I)
+#pragma unroll
+        for (int J = 0; J < 3; ++J) C[3 * I + J] = Cij(I, J);
+      const double c00 = C[4] * C[8] - C[5] * C[7], c01 = C[5] * C[6] - C[3] * C[8], c02 = C[3] * C[7] - C[4] * C[6];
+      const double c11 = C[0] * C[8] - C[2] * C[6], c12 = C[2] * C[3] - C[0] * C[5], c22 = C[0] * C[4] - C[1] * C[3];
+      const double J2 = C[0] * c00 + C[1] * c01 + C[2] * c02, rJ = 1.0 / J2;
+      const double Ci[6] = {c00 * rJ, c11 * rJ, c22 * rJ, c12 * rJ, c02 * rJ, c01 * rJ};  // Mandel order, plain entries
+      double sa[6], ea;
+      aniso_base(c.ba, C, sa, ea);
+#pragma unroll
+      for (int p = 0; p < 6; ++p) {
+        sm.Ci[p][lane] = Ci[p];
+        sm.S[p][lane] = 0.5 * c.lam0 * (J2 - 1.0) * Ci[p] + c.mu0 * ((p < 3 ? 1.0 : 0.0) - Ci[p]) + sa[p] / (p < 3 ? 1.0 : sq2);
+      }
+      sm.J2[lane] = J2;
+      if (Wout) W = 0.25 * c.lam0 * (J2 - 1.0) - (0.5 * c.lam0 + c.mu0) * 0.5 * log(J2) + 0.5 * c.mu0 * (C[0] + C[4] + C[8] - 3.0) + ea;
+    }
+    __syncthreads();
+    if (warp == 7) {  // S with the learned correction (its Taylor terms at x = 0 removed), P and W
+      double xs[6], ys = lane < np ? (double)y[q] - c.ba.y0 : 0.0, gp[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int p = 0; p < 6; ++p) xs[p] = sm.m[p][lane];
+      int k = 0;
+#pragma unroll
+      for (int p = 0; p < 6; ++p) {
+        double yd = 0.0, yo = 0.0;  // row p of the value's quadratic form, diagonal and above it
+#pragma unroll
+        for (int r = p; r < 6; ++r, ++k) {
+          const double hg = sm.hg[k][lane], hy = sm.hy[k][lane];
+          gp[p] = fma(hg, xs[r], gp[p]);
+          if (r == p) {
+            yd = hy * xs[p];
+          } else {
+            gp[r] = fma(hg, xs[p], gp[r]);
+            yo = fma(hy, xs[r], yo);
+          }
+        }
+        ys = fma(fma(2.0, yo, yd), xs[p], ys);
+      }
+      double S[6];
+#pragma unroll
+      for (int p = 0; p < 6; ++p) {
+        double hx = 0.0;
+#pragma unroll
+        for (int r = 0; r < 6; ++r) hx += c.ba.H0[6 * p + r] * xs[r];
+        const double gs = (lane < np ? (double)g[(size_t)q * 6 + p] : 0.0) - c.ba.g0[p] - hx + gp[p];
+        ys -= (c.ba.g0[p] + 0.5 * hx) * xs[p];
+        S[p] = sm.S[p][lane] + c.sg / c.sx * gs / (p < 3 ? 1.0 : sq2);
+        sm.S[p][lane] = S[p];
+      }
+      if (lane < np) {
+        if (Wout) Wout[q] = W + c.sg * ys;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int J = 0; J < 3; ++J)
+            P[(size_t)q * 9 + 3 * i + J] = f[3 * i] * S[mandel_index(0, J)] + f[3 * i + 1] * S[mandel_index(1, J)] +
+                                          f[3 * i + 2] * S[mandel_index(2, J)];
+      }
+    } else if (A) {  // CC of this warp's pairs: base law, network (not symmetric in bf16: both orders), polynomial, Ca
+      const double J2 = sm.J2[lane], beta = c.lam0 * (J2 - 1.0) - 2.0 * c.mu0, gam = c.lam0 * J2;
+      const double sc = c.sg / (c.sx * c.sx);
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const double xp = sm.m[pp[k]][lane], xq = sm.m[pq[k]][lane], hr = hs[k] * rg;
-        Hp[k] += hs[k];
-        const bool diag = pp[k] == pq[k];
+        const int p = pp[k], r = pq[k];
+        const int I = kMandelI[p], J = kMandelJ[p], K = kMandelI[r], L = kMandelJ[r];
+        auto ci = [&](int a, int b) { return sm.Ci[mandel_index(a, b)][lane]; };
+        const double base = beta * (-0.5) * (ci(I, K) * ci(J, L) + ci(J, K) * ci(I, L)) + gam * ci(I, J) * ci(K, L);
+        const double rw = (p < 3 ? 1.0 : 1.0 / sq2) * (r < 3 ? 1.0 : 1.0 / sq2);
+        auto entry = [&](int a, int b) {
+          const double hn = (double)sm.H[min(lane, np - 1) * 36 + a * 6 + b] - c.ba.H0[6 * a + b] + Hp[k];
+          return base + (sc * hn + c.ba.Ca[6 * a + b]) * rw;
+        };
+        cc[6 * p + r][lane] = entry(p, r);
+        if (p != r) cc[6 * r + p][lane] = entry(r, p);
+      }
+    }
+    __syncthreads();
+    if (!A) continue;
+    // A_iJkL = d_ik S_JL + F_iI F_kK CC_IJKL, rows (i, J) dealt to the warps
+    for (int row = warp; row < 9; row += kCombineThreads / 32) {
+      const int i = row / 3, J = row % 3;
+      double G[6];
 #pragma unroll
-        for (int r = 0; r < 6; ++r) {
-          if (r == pp[k]) gs[r] = fma(hr, xq, gs[r]);
-          if (r == pq[k] && !diag) gs[r] = fma(hr, xp, gs[r]);
+      for (int r = 0; r < 6; ++r) {
+        G[r] = 0.0;
+#pragma unroll
+        for (int I = 0; I < 3; ++I) G[r] = fma(sm.F[3 * i + I][lane], cc[6 * mandel_index(I, J) + r][lane], G[r]);
+      }
+      double* out = tileA + lane * 81 + row * 9;
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int L = 0; L < 3; ++L) {
+          double v = i == k ? sm.S[mandel_index(J, L)][lane] : 0.0;
+#pragma unroll
+          for (int K = 0; K < 3; ++K) v = fma(f[3 * k + K], G[mandel_index(K, L)], v);
+          out[3 * k + L] = v;
         }
-        ys = fma(hs[k] * ry * (diag ? 1.0 : 2.0), xp * xq, ys);
-      }
     }
-#pragma unroll
-    for (int r = 0; r < 6; ++r) sm.gp[warp][r][lane] = gs[r];
-    sm.yp[warp][lane] = ys;
-  } else {  // base law: S = lam/2 (J^2-1) C^-1 + mu (I - C^-1), plus the anisotropic small-strain part
-    double C[9];
-#pragma unroll
-    for (int I = 0; I < 3; ++I)
-#pragma unroll
-      for (int J = 0; J < 3; ++J) C[3 * I + J] = Cij(I, J);
-    const double c00 = C[4] * C[8] - C[5] * C[7], c01 = C[5] * C[6] - C[3] * C[8], c02 = C[3] * C[7] - C[4] * C[6];
-    const double c11 = C[0] * C[8] - C[2] * C[6], c12 = C[2] * C[3] - C[0] * C[5], c22 = C[0] * C[4] - C[1] * C[3];
-    const double J2 = C[0] * c00 + C[1] * c01 + C[2] * c02, rJ = 1.0 / J2;
-    const double Ci[6] = {c00 * rJ, c11 * rJ, c22 * rJ, c12 * rJ, c02 * rJ, c01 * rJ};  // Mandel order, plain entries
-    double sa[6], ea;
-    aniso_base(c.ba, C, sa, ea);
-#pragma unroll
-    for (int p = 0; p < 6; ++p) {
-      sm.Ci[p][lane] = Ci[p];
-      sm.S[p][lane] = 0.5 * c.lam0 * (J2 - 1.0) * Ci[p] + c.mu0 * ((p < 3 ? 1.0 : 0.0) - Ci[p]) + sa[p] / (p < 3 ? 1.0 : sq2);
-    }
-    sm.J2[lane] = J2;
-    if (Wout) W = 0.25 * c.lam0 * (J2 - 1.0) - (0.5 * c.lam0 + c.mu0) * 0.5 * log(J2) + 0.5 * c.mu0 * (C[0] + C[4] + C[8] - 3.0) + ea;
+    __syncthreads();
+    for (int e = t; e < np * 81; e += kCombineThreads) A[(size_t)q0 * 81 + e] = tileA[e];
+    __syncthreads();
   }
-  __syncthreads();
-  if (warp == 7) {  // S with the learned correction (its Taylor terms at x = 0 removed), P and W
-    double xs[6], ys = lane < np ? (double)y[q] - c.ba.y0 : 0.0;
-#pragma unroll
-    for (int w = 0; w < 7; ++w) ys += sm.yp[w][lane];
-#pragma unroll
-    for (int p = 0; p < 6; ++p) xs[p] = sm.m[p][lane];
-    double S[6];
-#pragma unroll
-    for (int p = 0; p < 6; ++p) {
-      double hx = 0.0, gp = 0.0;
-#pragma unroll
-      for (int r = 0; r < 6; ++r) hx += c.ba.H0[6 * p + r] * xs[r];
-#pragma unroll
-      for (int w = 0; w < 7; ++w) gp += sm.gp[w][p][lane];
-      const double gs = (lane < np ? (double)g[(size_t)q * 6 + p] : 0.0) - c.ba.g0[p] - hx + gp;
-      ys -= (c.ba.g0[p] + 0.5 * hx) * xs[p];
-      S[p] = sm.S[p][lane] + c.sg / c.sx * gs / (p < 3 ? 1.0 : sq2);
-      sm.S[p][lane] = S[p];
-    }
-    if (lane < np) {
-      if (Wout) Wout[q] = W + c.sg * ys;
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int J = 0; J < 3; ++J)
-          P[(size_t)q * 9 + 3 * i + J] = f[3 * i] * S[mandel_index(0, J)] + f[3 * i + 1] * S[mandel_index(1, J)] +
-                                        f[3 * i + 2] * S[mandel_index(2, J)];
-    }
-  } else if (A) {  // CC of this warp's pairs: base law, network (not symmetric in bf16: both orders), polynomial, Ca
-    const double J2 = sm.J2[lane], beta = c.lam0 * (J2 - 1.0) - 2.0 * c.mu0, gam = c.lam0 * J2;
-    const double sc = c.sg / (c.sx * c.sx);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const int p = pp[k], r = pq[k];
-      const int I = kMandelI[p], J = kMandelJ[p], K = kMandelI[r], L = kMandelJ[r];
-      auto ci = [&](int a, int b) { return sm.Ci[mandel_index(a, b)][lane]; };
-      const double base = beta * (-0.5) * (ci(I, K) * ci(J, L) + ci(J, K) * ci(I, L)) + gam * ci(I, J) * ci(K, L);
-      const double rw = (p < 3 ? 1.0 : 1.0 / sq2) * (r < 3 ? 1.0 : 1.0 / sq2);
-      auto entry = [&](int a, int b) {
-        const double hn = (double)sm.H[min(lane, np - 1) * 36 + a * 6 + b] - c.ba.H0[6 * a + b] + Hp[k];
-        return base + (sc * hn + c.ba.Ca[6 * a + b]) * rw;
-      };
-      sm.cc[6 * p + r][lane] = entry(p, r);
-      if (p != r) sm.cc[6 * r + p][lane] = entry(r, p);
-    }
-  }
-  if (!A) return;
-  __syncthreads();
-  // A_iJkL = d_ik S_JL + F_iI F_kK CC_IJKL, rows (i, J) dealt to the warps
-  for (int row = warp; row < 9; row += kCombineThreads / 32) {
-    const int i = row / 3, J = row % 3;
-    double G[6];
-#pragma unroll
-    for (int r = 0; r < 6; ++r) {
-      G[r] = 0.0;
-#pragma unroll
-      for (int I = 0; I < 3; ++I) G[r] = fma(sm.F[3 * i + I][lane], sm.cc[6 * mandel_index(I, J) + r][lane], G[r]);
-    }
-    double* out = sm.T + lane * 81 + row * 9;
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-      for (int L = 0; L < 3; ++L) {
-        double v = i == k ? sm.S[mandel_index(J, L)][lane] : 0.0;
-#pragma unroll
-        for (int K = 0; K < 3; ++K) v = fma(f[3 * k + K], G[mandel_index(K, L)], v);
-        out[3 * k + L] = v;
-      }
-  }
-  __syncthreads();
-  for (int e = t; e < np * 81; e += kCombineThreads) A[(size_t)q0 * 81 + e] = sm.T[e];
 }
 
 // Training targets from full RVE solves at F (= U): features x = Mandel(E)/sx, value target
@@ -710,8 +727,11 @@ extern "C" int fehmm_surrogate_eval(fehmm_mlp* mlp, const fehmm_surrogate_params
   if (cudaFuncSetAttribute(combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CombineSmem)) !=
       cudaSuccess)
     return FEHMM_ERR_CUDA;
-  combine_kernel<<<(n + kCombinePts - 1) / kCombinePts, kCombineThreads, sizeof(CombineSmem), s>>>(c, F, n, emax, y, g, H,
-                                                                                                  P, A, W);
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return FEHMM_ERR_CUDA;
+  const int tiles = (n - 1) / kCombinePts + 1;
+  combine_kernel<<<tiles < 2 * sms ? tiles : 2 * sms, kCombineThreads, sizeof(CombineSmem), s>>>(c, F, n, emax, y, g, H, P, A, W);
   return cudaGetLastError() == cudaSuccess ? FEHMM_OK : FEHMM_ERR_CUDA;
 }
 
