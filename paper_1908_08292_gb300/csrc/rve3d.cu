@@ -9,8 +9,8 @@
 // omega/|K_delta| T^T K T, Eq. k-mac-element-6; the two are checked equal in the oracle tests).
 //
 // GB300 layout:
-//  * One block per RVE, 512 threads and one block per SM, or two of 256 (see rve3d_blocks_per_sm); the points of
-//    each grid size are a launch of their own.  The apply's vectors, in mixed mode also the FP32 fluctuation, the
+//  * One block per RVE, up to 512 threads and one block per SM, or several of up to 256 (rve3d_threads,
+//    rve3d_blocks_per_sm); the points of each grid size are a launch of their own.  The apply's vectors, in mixed mode also the FP32 fluctuation, the
 //    residual and the coarse vectors, live in shared memory; the other PCG vectors stream from per-block scratch.
 //  * Residual and tangent apply: two lanes per element, one for each plane of four Gauss points (Cell3).  The FP64
 //    residual stages element forces in global scratch and gathers them per node; the apply, matrix-free in TA
@@ -29,6 +29,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "fehmm_device.cuh"
@@ -2038,12 +2039,24 @@ size_t rve3d_scratch_bytes(int nn_max, bool mixed, int n_blocks) {
   return (mixed ? scratch3_bytes<float>(nn_max) : scratch3_bytes<double>(nn_max)) * (size_t)n_blocks;
 }
 
-// Blocks of RVEs with nn nodes on one SM: two of 256 threads where there are more RVEs than SMs and the shared
-// memory holds both (n <= 12 in mixed precision), so that one works while the other waits at a barrier or runs its
-// FP64 residual; one of 512 otherwise (one RVE alone is 1.3 times faster with it).  304 RVEs of 8^3: 17.2 ms with
-// one, 13.4 with two, 16.5 with four of 128 threads; 200: 15.9, 12.9, 16.5; 304 of 12^3: 55.0, 48.6.
+// Threads of a block for RVEs of nn elements, at most cap: two lanes an element in as many passes as cap needs, and no
+// more warps than fill these passes evenly.  (At 512 threads 7^3 fills its second pass to a third, and every barrier of
+// 4^3 waits for twelve idle warps.)  Against 512 (256 where there are more RVEs than SMs), mixed precision: 4 RVEs of 4^3
+// 2.68 -> 1.76 ms, of 5^3 3.68 -> 2.77, of 7^3 8.42 -> 7.14, of 6^3 and 8^3 the same; 1000 of 4^3 10.1 -> 6.2.
+static int rve3d_threads(int nn, int cap) {
+  const int passes = (2 * nn + cap - 1) / cap, even = (2 * nn + passes - 1) / passes;
+  return std::max(128, (even + 31) / 32 * 32);
+}
+
+// Blocks of RVEs with nn nodes on one SM: where there are more RVEs than SMs, blocks of up to 256 threads, as many as
+// registers and shared memory hold (two for n <= 12 in mixed precision), so that one works while the other waits at a
+// barrier or runs its FP64 residual; one of up to 512 otherwise (one RVE alone is 1.3 times faster with it).
+// 304 RVEs of 8^3: 17.2 ms with one, 13.4 with two, 16.5 with four of 128 threads; 200: 15.9, 12.9, 16.5; 304 of
+// 12^3: 55.0, 48.6.
 int rve3d_blocks_per_sm(int nn, bool mixed, int count, int num_sms) {
-  return mixed && count > num_sms && 2 * (rve3d_smem_bytes(nn, true) + 1024) <= 228 * 1024 ? 2 : 1;
+  if (!mixed || count <= num_sms) return 1;
+  const int smem = (int)((228 * 1024) / (rve3d_smem_bytes(nn, true) + 1024));
+  return std::max(1, std::min(65536 / (128 * rve3d_threads(nn, kThreads3D / 2)), smem));
 }
 
 template <typename TA, int LAW>
@@ -2056,7 +2069,7 @@ cudaError_t rve3d_launch_instance(const Rve2dArgs& a, int n_blocks, int threads,
 }
 
 cudaError_t rve3d_launch(const Rve2dArgs& a, bool mixed, int n_blocks, int per_sm, cudaStream_t stream) {
-  const int threads = kThreads3D / per_sm;
+  const int threads = rve3d_threads(a.nn_max, per_sm > 1 ? kThreads3D / 2 : kThreads3D);
   const size_t smem = rve3d_smem_bytes(a.nn_max, mixed);
   if (mixed)
     return a.law == kLawSVK ? rve3d_launch_instance<float, kLawSVK>(a, n_blocks, threads, smem, stream)

@@ -85,3 +85,22 @@ def test_more_points_than_sms(law):
         assert rel_err(big["P"][q], small["P"][k], 1e-3) < 1e-9  # both within the Newton tolerance
         assert rel_err(big["A"][q], small["A"][k], 1e-3) < 1e-6  # FP32 tangent
         assert abs(big["W"][q] - small["W"][k]) < 1e-12
+
+
+@pytest.mark.parametrize("size", [3, 4, 5, 6, 7])
+def test_block_shapes_of_small_grids(size):
+    """A grid's block has the threads its element passes fill evenly: 128 to 448, other shapes with more points than
+    SMs (up to four blocks of 128 per SM at 4^3).  A few points of such a batch again in a call of their own."""
+    phases, E, nu = rves()
+    k = SIZES.index(size)
+    n_qp = 330
+    Fs = synth.random_F(834, n_qp, 3, 0.06)
+    big = gpu_batch(3, "mixed", [size], [phases[k]], E[k:k + 1], nu[k:k + 1], np.zeros(n_qp, dtype=np.int32), Fs)
+    some = np.array([0, 1, 153, 328, 329])
+    small = gpu_batch(3, "mixed", [size], [phases[k]], E[k:k + 1], nu[k:k + 1], np.zeros(5, dtype=np.int32), Fs[some])
+    assert np.all(big["status"] == 0) and np.all(small["status"] == 0)
+    for m, q in enumerate(some):
+        assert rel_err(big["P"][q], small["P"][m], 1e-3) < 1e-9  # both within the Newton tolerance
+        assert rel_err(big["A"][q], small["A"][m], 1e-3) < 1e-6  # FP32 tangent
+    ref = PeriodicRVE(size, 3, phases[k], E[k], nu[k]).solve(Fs[329], rtol=1e-14, atol=1e-16)
+    assert rel_err(big["P"][329], ref["P"], 1e-3) < TOL["mixed"] and rel_err(big["A"][329], ref["A"], 1e-3) < TOL["mixed"]
