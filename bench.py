@@ -43,9 +43,9 @@ MACRO_C3, N_STEPS_C3 = 8, 10
 # Algorithmic operation counts per unit of the 2D mixed kernel, counted from the kernel source
 # (an FMA counting 2).
 # residual: differences of the corner fluctuations (12), F's two columns at the two Gauss
-# abscissae (32), per Gauss point J, the refined reciprocal (4 FMA), c and P (26 x 4), the stress
+# abscissae (32), per Gauss point J, the refined reciprocal (3 FMA), c and P (24 x 4), the stress
 # sums per Gauss line and their shape weights (43), nodal forces (8), gather and norm (10)
-FP64_FLOP_PER_ELEMENT_RESIDUAL = 211.0
+FP64_FLOP_PER_ELEMENT_RESIDUAL = 201.0
 FP32_FLOP_PER_ELEMENT_TANGENT = 1350.0   # 8x8 element tangent at 4 Gauss points + stencil gather
 FP32_FLOP_PER_NODE_PCG_ITER = 100.0      # 9-block 2x2 stencil apply + vector updates + 2 dots
 FP32_FLOP_PER_ELEMENT_TRANSFER = 1500.0  # energy form of the tangent transfer (4 unit gradients)
@@ -56,16 +56,19 @@ FP32_FLOP_PER_ELEMENT_TRANSFER = 1500.0  # energy form of the tangent transfer (
 # node), coarse stencils and the coarsest Gauss-Jordan inverse (2 x 32^3 / 1024)
 FP32_FLOP_PER_NODE_MG_ITER = 238.0
 FP32_FLOP_PER_NODE_MG_BUILD = 570.0
-FP64_FLOP_PER_ELEMENT_RESIDUAL_3D = 2620.0   # Hex8: 8 Gauss points x (grad, cof(F), J, 1/J refined, P, nodal forces)
+# Hex8, by planes of four Gauss points (two lanes per element): per lane F (186), the law's constant part (24), per
+# point cof(F), J, 1/J and the stress sums (60 x 4), <P> (24), nodal forces (192); and the gather and norm (27 a node)
+FP64_FLOP_PER_ELEMENT_RESIDUAL_3D = 1360.0
 FP32_FLOP_PER_ELEMENT_TANGENT_3D = 4200.0    # Gauss-point data + 3x3 diagonal blocks
-FP32_FLOP_PER_ELEMENT_APPLY_3D = 4000.0      # matrix-free apply: grad, dP = A:dF, nodal scatter
+# matrix-free apply, per lane: F (186), grad of the increment (162), dP per point (166 x 4), nodal sums (228)
+FP32_FLOP_PER_ELEMENT_APPLY_3D = 2480.0
 FP32_FLOP_PER_NODE_PCG_ITER_3D = 30.0        # preconditioner + vector updates + dots
-# 3D multigrid, per fine element: V-cycle per PCG iteration = two more fine applies (2 x 4000),
-# level-1 gathers (2 x 1152 flop per coarse node / 8), deeper levels, smoothing, restriction and
+# 3D multigrid, per fine element: V-cycle per PCG iteration = two more fine applies (2 x 2480),
+# level-1 stencils (2 x 486 flop per coarse node / 8), deeper levels, smoothing, restriction and
 # prolongation; per tangent build the level-1 element blocks integrated over the 64 fine Gauss
 # points of each coarse element (3312 flop per Gauss point, 212k per coarse element, 26.5k per
 # fine element), deeper levels (2.3k) and the coarsest inverse (<= 0.6k)
-FP32_FLOP_PER_ELEMENT_MG_ITER_3D = 8400.0
+FP32_FLOP_PER_ELEMENT_MG_ITER_3D = 5200.0
 FP32_FLOP_PER_ELEMENT_MG_BUILD_3D = 29000.0
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12   # SMs x FP32 lanes x FMA x max clock
 FP64_PEAK_TFLOPS = 1.25                              # GB300 nominal FP64
@@ -74,9 +77,9 @@ FP64_PEAK_TFLOPS = 1.25                              # GB300 nominal FP64
 # DRAM bytes per RVE solve of the dominant kernel from an ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum of one launch / RVEs in that launch), with the profile summary it comes
 # from; scaled to a launch of the bench by the RVEs it solves.  Only for a capture of the kernel
-# build the bench runs: the captures in profiles/ (155 KB per 2D RVE, 23.9 MB per 3D RVE) predate
-# the kernels' keeping of the coarse levels for the tangent transfer, so no entry is given.
-TRAFFIC_PER_LAUNCH = {}
+# build the bench runs; the 3D capture (23.9 MB per RVE) predates the kernel that reads the
+# fluctuation in place of stored Gauss-point data, so it has no entry.
+TRAFFIC_PER_LAUNCH = {("c2", "mg"): (125.4e3, "profiles/rve2d_kernel_mg_c2_macro16.md")}
 
 
 def workload_config(step_index):
@@ -84,8 +87,8 @@ def workload_config(step_index):
     if _SIZE["workload"] == "c3":
         return {"workload": f"3D FE-HMM macro {MACRO}^3 Hex8 ({MACRO ** 3 * 8} qps), one periodic Hex8 RVE per qp "
                             f"of 8^3/12^3/16^3 elements (uniform draw), 1-4 spheres (volume fraction 0.1-0.3, "
-                            f"stiffness ratio 10), neo-Hookean, mixed FP32/FP64, uneven batch in one persistent "
-                            f"launch, macro iteration 1 of load step {step_index}/{N_STEPS_C3} (uniaxial to 20%)",
+                            f"stiffness ratio 10), neo-Hookean, mixed FP32/FP64, uneven batch in one call"
+                            f", macro iteration 1 of load step {step_index}/{N_STEPS_C3} (uniaxial to 20%)",
                 "n_qp": MACRO ** 3 * 8, "rve_grid": "8/12/16 mixed", "load_step": step_index,
                 "l2": "flushed (256 MB write) between timed steps"}
     W = _SIZE["world"]
@@ -550,8 +553,8 @@ def path_config(steps_timed):
     if wl == "c3":
         return {"workload": f"3D FE-HMM macro {MACRO}^3 Hex8 ({MACRO ** 3 * 8} qps), one periodic Hex8 RVE per qp "
                             f"of 8^3/12^3/16^3 elements (uniform draw), 1-4 spheres (volume fraction 0.1-0.3, "
-                            f"stiffness ratio 10), neo-Hookean, mixed FP32/FP64, uneven batch in one persistent "
-                            f"launch; a step = one whole load step (all macro iterations, nested scheme) of the "
+                            f"stiffness ratio 10), neo-Hookean, mixed FP32/FP64, uneven batch in one call"
+                            f"; a step = one whole load step (all macro iterations, nested scheme) of the "
                             f"10-step uniaxial path to 20%, cycling load steps {ks}",
                 "n_qp": MACRO ** 3 * 8, "rve_grid": "8/12/16 mixed", "load_steps_timed": list(steps_timed),
                 "l2": "flushed (256 MB write) between timed steps"}
