@@ -351,7 +351,8 @@ typedef struct {
  * Surrogate constitutive evaluation at n macro points: F device [n][9] in; P [n][9],
  * A [n][81] (may be NULL), W [n] (may be NULL), inside [n] (1 inside the trust region,
  * else 0) out; work: device floats, fehmm_surrogate_work_floats(n) of them; n <= the MLP's
- * max_batch.  P and A are written for every point; the caller replaces the points outside
+ * max_batch.  sp is read during the call (a captured call keeps its values).  P and A are written
+ * for every point; the caller replaces the points outside
  * the trust region by full RVE solves (fehmm_select + fehmm_rve_solve_list).
  */
 int fehmm_surrogate_eval(fehmm_mlp* mlp, const fehmm_surrogate_params* sp, const double* F, int n,
