@@ -13,7 +13,8 @@
 //  * the part of the neo-Hookean tangent that is the same matrix for every element is added once, scaled by mu.
 // Measured on a GB300, one pass from a committed state, against the node-pair layout of rve2d.cuh with TA = double:
 // at 512 threads (first figure) and at one thread per node pair (second).  64 RVEs of 8 x 8: 3.18, 2.45 -> 0.71 ms;
-// 100 of 32 x 32: 18.3, 18.3 -> 12.4 ms; 150 of 16 x 16 through the no-allocation entry: 16.3, 8.6 -> 5.2 ms.
+// 100 of 32 x 32: 18.3, 18.3 -> 12.4 ms; 150 of 16 x 16 through the no-allocation entry, block-Jacobi: 16.3, 8.6 -> 5.2 ms
+// (3.3 with multigrid).
 #pragma once
 #include "rve2d.cuh"
 
@@ -57,8 +58,9 @@ __host__ __device__ constexpr OffsetsD2 offsets_d2(int NN, bool mg) {
   o.total = off;
   return o;
 }
-// Block scratch (doubles): staged element tangents [36][NN], the stencil [18][2 NN] (large grids), then the
-// multigrid: fast region (where not in shared memory) and slow region.
+// Block scratch (doubles): staged element tangents [36][NN], the stencil [18][2 NN] (grids that do not hold it in
+// registers), then the multigrid: fast region (where not in shared memory) and slow region.  The slow region takes the
+// stencil's place where that is in registers: it has a third of its size.
 __host__ __device__ constexpr long long scratch_d2(int NN, bool mg) {
   int n = 2;
   while (n * n < NN) ++n;
@@ -746,7 +748,7 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
   s.mg.bc = a.bc;
   s.mg.omega = (double)a.mg_omega;
   s.mg.fast = off.fast_in_smem ? reinterpret_cast<double*>(smem + off.fast) : scr + 72 * (size_t)NN;
-  s.mg.slow = scr + 72 * (size_t)NN + (kMG ? mg_fast_elems(n) : 0);
+  s.mg.slow = scr + (kRowInRegs<DPT> ? 36 * (size_t)NN : 72 * (size_t)NN + (kMG ? mg_fast_elems(n) : 0));
 #pragma unroll
   for (int q = 0; q < DPT; ++q) {
     const int d = tid + q * s.T;
@@ -843,12 +845,15 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
           reuse = false;
         } else if (kMG && s.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) && s.mg.omega > 0.2 * omega0) {
           s.mg.omega *= 0.5;
+        } else if (kFixed && kMG && s.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap)) {
+          s.mg.levels = 0;  // block-Jacobi, the entry's preconditioner for grids without a hierarchy
         } else {
           break;
         }
         pst = kStatusOk;
       }
       s.mg.omega = omega0;
+      if (kFixed && kMG) s.mg.levels = mg_levels(n);
       if (pst == kStatusPcgBreakdown) {
         status = kStatusPcgBreakdown;
         break;
@@ -927,11 +932,14 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
             redo = true;
             break;
           }
-          if (!(kMG && s.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) && s.mg.omega > 0.2 * omega0)) break;
-          s.mg.omega *= 0.5;
+          if (!(kMG && s.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap))) break;
+          if (s.mg.omega > 0.2 * omega0) s.mg.omega *= 0.5;
+          else if (kFixed) s.mg.levels = 0;
+          else break;
           pst = kStatusOk;
         }
         s.mg.omega = omega0;
+        if (kFixed && kMG) s.mg.levels = mg_levels(n);
         t_total += ci;
         t_max = ci > t_max ? ci : t_max;
         if (redo) break;

@@ -3,6 +3,8 @@
 and without idle lanes; multigrid levels in shared memory up to 24 x 24, in block scratch at 32 x 32.  Both laws and
 both preconditioners, against the FP64 oracle at the tolerance of FP64 mode, then once more with kept transfer
 solutions."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -62,3 +64,40 @@ def test_collapsed_point_is_reported(precision, n):
     ref = PeriodicRVE(n, 2, phase, [1.0, 10.0], [0.3, 0.3]).solve(Fs[1], rtol=1e-14, atol=1e-16)
     assert out["status"][0] != 0 and out["status"][1] == 0
     assert rel_err(out["P"][1], ref["P"], 1e-3) < 1e-5  # default tolerances in both modes
+
+
+@pytest.mark.parametrize("precond", [1, 0])
+@pytest.mark.parametrize("n", [4, 6, 10, 12, 14, 16])
+def test_noalloc_preconditioners(n, precond):
+    """The no-allocation entry on grids with a multigrid hierarchy (6, 12, 16) and without, by either option."""
+    import torch
+
+    import paper_1908_08292_gb300 as fe
+    dev = torch.device("cuda:0")
+    n_qp = 3
+    E, nu = np.array([1.0, 25.0]), np.array([0.3, 0.3])
+    u = synth.uniform(841, np.arange(n_qp), 3)
+    phases = [synth.phase_from_inclusions(n, 2, [u[q, :2]], [0.2 + 0.1 * u[q, 2]]) for q in range(n_qp)]
+    table = np.zeros((n_qp, 4, 2))
+    table[:, :2, 0] = E * nu / ((1 + nu) * (1 - 2 * nu))
+    table[:, :2, 1] = E / (2 * (1 + nu))
+    opt = fe.Options()
+    assert fe.lib().fehmm_default_options(ctypes.byref(opt), 2, fe.PREC_FP64) == 0
+    for k, v in dict(STRICT, precond=precond).items():
+        setattr(opt, k, v)
+    Fs = synth.random_F(842, n_qp, 2, 0.1)
+    t = dict(phase=torch.tensor(np.stack(phases), dtype=torch.uint8, device=dev), lame=torch.tensor(table, device=dev),
+             w=torch.zeros(n_qp, 2 * n * n, dtype=torch.float64, device=dev), F=torch.tensor(Fs.reshape(n_qp, 4), device=dev),
+             P=torch.zeros(n_qp, 4, dtype=torch.float64, device=dev), A=torch.zeros(n_qp, 16, dtype=torch.float64, device=dev),
+             st=torch.full((n_qp,), -1, dtype=torch.int32, device=dev), it=torch.zeros(n_qp, 4, dtype=torch.int32, device=dev))
+    p = {k: ctypes.c_void_p(v.data_ptr()) for k, v in t.items()}
+    rc = fe.lib().fehmm_rve2d_solve_fp64_noalloc(n_qp, n, 1, p["phase"], p["lame"], p["w"], p["F"], p["P"], p["A"], p["st"],
+                                                 p["it"], ctypes.byref(opt),
+                                                 ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == 0
+    torch.cuda.synchronize()
+    for q in range(n_qp):
+        ref = PeriodicRVE(n, 2, phases[q], E, nu).solve(Fs[q], rtol=1e-14, atol=1e-16)
+        assert int(t["st"][q]) == 0
+        assert rel_err(t["P"][q].cpu().numpy(), ref["P"], 1e-3) < TOL
+        assert rel_err(t["A"][q].cpu().numpy(), ref["A"], 1e-3) < TOL
