@@ -283,10 +283,17 @@ int fehmm_macro_update(fehmm_ctx* ctx, double* u, const double* du, void* stream
  *   K_vals device [nnz] (CSR order of fehmm_macro_csr), f device [n_rows], du device
  *   [n_rows] (output), info device double[3] (output): |f_free|_2 (the macro convergence
  *   measure, taken before the solve), CG iterations, status (0 converged, 1 cap,
- *   2 non-positive curvature, 3 a thread block gave up waiting for another: du is not valid).
+ *   2 non-positive curvature, 3 a thread block gave up waiting for another: du and the iteration
+ *   count are not valid, and the norm is NaN).
  */
 int fehmm_macro_solve(fehmm_ctx* ctx, const double* K_vals, const double* f, double* du, double* info,
                       double rtol, int max_it, void* stream);
+
+/* Cycles of the SM clock that a thread block of the macro solve waits for another one before it
+ * gives up (info status 3).  Default 2^32, about two seconds; 0 gives up on the first word that is
+ * not there yet.  Meshes solved by one block, and those too large for the solve that keeps its rows
+ * in registers, wait for none. */
+int fehmm_macro_set_wait_limit(fehmm_ctx* ctx, long long cycles);
 
 /* CSR pattern of the assembled macro tangent of Eq. Assem_k_T_IK_mac (one d x d block per pair of
  * nodes sharing an element; device pointers owned by the context). */

@@ -74,6 +74,7 @@ _SIGS = {
     "fehmm_macro_update": (_I, [_P, _P, _P, _P]),
     "fehmm_macro_dirichlet_load": (_I, [_P, _P, ctypes.c_double, _P, _P]),
     "fehmm_macro_solve": (_I, [_P, _P, _P, _P, _P, ctypes.c_double, _I, _P]),
+    "fehmm_macro_set_wait_limit": (_I, [_P, ctypes.c_longlong]),
     "fehmm_macro_csr": (_I, [_P, ctypes.POINTER(_P), ctypes.POINTER(_P), ctypes.POINTER(_I), ctypes.POINTER(_I)]),
     "fehmm_launch_count": (ctypes.c_longlong, [_P]),
     "fehmm_autotune": (_I, [_P, _P, _I, ctypes.c_char_p, ctypes.POINTER(TuneResult), _P]),
@@ -342,6 +343,10 @@ class Context:
         _check(lib().fehmm_macro_solve(self._h, _dev(K_vals, torch.float64, "K_vals"), _dev(f, torch.float64, "f"),
                                        _dev(du, torch.float64, "du"), _dev(info, torch.float64, "info", 3),
                                        float(rtol), int(max_it), _stream(stream)), "macro_solve")
+
+    def macro_set_wait_limit(self, cycles):
+        """SM cycles a thread block of macro_solve waits for another before it gives up (info status 3)."""
+        _check(lib().fehmm_macro_set_wait_limit(self._h, int(cycles)), "macro_set_wait_limit")
 
     def macro_csr(self):
         """(rowptr, col, n_rows, nnz); rowptr/col are int32 device views owned by the context."""

@@ -73,6 +73,7 @@ struct fehmm_ctx {
   int32_t* d_halo = nullptr;
   uint16_t* d_lcol = nullptr;
   void* d_pub = nullptr;
+  long long macro_wait = kMacroWaitCycles;
   long long launches = 0;
 };
 
@@ -733,6 +734,7 @@ int fehmm_macro_solve(fehmm_ctx* c, const double* K_vals, const double* f, doubl
   a.halo = c->d_halo;
   a.lcol = c->d_lcol;
   a.pub = c->d_pub;
+  a.wait_limit = c->macro_wait;
   if ((c->resident.lanes
            ? macro_solve_resident_launch(a, c->opt.dim, c->resident, (cudaStream_t)stream)
            : macro_solve_launch(a, macro_solve_blocks(c->num_sms, c->macro_rows), (cudaStream_t)stream)) != cudaSuccess) {
@@ -740,6 +742,12 @@ int fehmm_macro_solve(fehmm_ctx* c, const double* K_vals, const double* f, doubl
     return FEHMM_ERR_CUDA;
   }
   c->launches += 1;
+  return FEHMM_OK;
+}
+
+int fehmm_macro_set_wait_limit(fehmm_ctx* c, long long cycles) {
+  if (!c || cycles < 0) return FEHMM_ERR_ARG;
+  c->macro_wait = cycles;
   return FEHMM_OK;
 }
 

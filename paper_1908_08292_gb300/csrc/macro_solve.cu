@@ -203,7 +203,13 @@ __global__ void __launch_bounds__(kSolveThreads) macro_pcg_kernel(const MacroSol
 
 // ------------------------------------------------------------------ rows resident in registers
 constexpr int kResMaxThreads = 256, kResMaxRows = 128;
-constexpr long long kSpinCycles = 1ll << 32;  // about 2 s: a block that never arrives
+
+__device__ __forceinline__ double fp64_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
+
+// *p = max(*p, v) over the blocks that call it, for values that are not negative; NaN is above every number
+__device__ __forceinline__ void raise_to(double* p, double v) {
+  atomicMax(reinterpret_cast<unsigned long long*>(p), (unsigned long long)__double_as_longlong(v));
+}
 
 // {value, sequence number} as one 16-byte word: a reader sees both or neither
 __device__ __forceinline__ void put(ulonglong2* p, double v, unsigned long long seq) {
@@ -213,9 +219,10 @@ __device__ __forceinline__ void put(ulonglong2* p, double v, unsigned long long 
 }
 
 // Calls take(e, value) for e = t, t + blockDim.x, ... < count with the words at word(e) once they carry seq; four
-// loads are in flight at a time (one after the other their latencies add up).  False if a word never comes.
+// loads are in flight at a time (one after the other their latencies add up).  False if a word has not come within
+// `limit` cycles.
 template <typename Word, typename Take>
-__device__ __forceinline__ bool get_all(int count, unsigned long long seq, Word word, Take take) {
+__device__ __forceinline__ bool get_all(int count, unsigned long long seq, long long limit, Word word, Take take) {
   constexpr int M = 4;
   bool ok = true;
   for (int e0 = threadIdx.x; e0 < count; e0 += M * blockDim.x) {
@@ -236,7 +243,7 @@ __device__ __forceinline__ bool get_all(int count, unsigned long long seq, Word 
 #pragma unroll
       for (int j = 0; j < M; ++j) all = all && s[j] == seq;
       if (all) break;
-      if (clock64() - t0 > kSpinCycles) {
+      if (clock64() - t0 > limit) {
         ok = false;
         break;
       }
@@ -304,6 +311,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
   if (mine && ll == 0) pub[i] = make_ulonglong2(0ull, 0ull);
   if (t < 4) slots[(t >> 1) * 2 * nb + 2 * blockIdx.x + (t & 1)] = make_ulonglong2(0ull, 0ull);
   if (t == 0) action = 0;
+  if (blockIdx.x == 0 && t < 3) a.out[t] = 0.0;
   grid.sync();  // every word carries sequence number 0
   unsigned long long useq = 0, sseq = 0;
   bool lost = false;
@@ -316,9 +324,9 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
     }
   };
   auto product = [&]() {  // the surrounding rows' u, then w = K u (the same in all lanes of a row)
-    lost |= !get_all(nh, useq, [&](int h) { return pub + a.halo[h0 + h]; }, [&](int h, double v) { us[R + h] = v; });
+    lost |= !get_all(nh, useq, a.wait_limit, [&](int h) { return pub + a.halo[h0 + h]; }, [&](int h, double v) { us[R + h] = v; });
     __syncthreads();
-    w = 0.0;
+    w = lost ? fp64_nan() : 0.0;  // a block that gave up spoils the sums it still publishes
 #pragma unroll
     for (int j = 0; j < PER; ++j) w = fma(k[j], us[(j & 1) ? lc[j / 2] >> 16 : lc[j / 2] & 0xffffu], w);
 #pragma unroll
@@ -341,7 +349,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
     }
     if (nb > 1) {
       acc = 0.0;
-      lost |= !get_all(2 * nb, sseq, [&](int e) { return slot + e; }, [&](int, double q) { acc += q; });
+      lost |= !get_all(2 * nb, sseq, a.wait_limit, [&](int e) { return slot + e; }, [&](int, double q) { acc += q; });
 #pragma unroll
       for (int o = 2; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
       if (lane < 2) part[1][2 * warp + lane] = acc;
@@ -362,7 +370,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
   double gamma = 0.0, rgamma = 0.0, den = 0.0, stop = 0.0;
   int it = 0;
   reduce(ll < 2 ? r * (ll ? u : r) : 0.0, [&](double ff, double ru) {
-    a.out[0] = sqrt(ff);
+    if (blockIdx.x == 0) raise_to(a.out, sqrt(ff));
     gamma = ru;
     stop = a.rtol * a.rtol * gamma;
     if (!(gamma > 0.0)) action = 1;
@@ -412,9 +420,17 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
     });
   }
   if (mine && ll == 0) a.du[i] = x;
-  if (blockIdx.x == 0 && t == 0) {
-    a.out[1] = (double)it;
-    a.out[2] = (double)(action - 1);  // 0 converged, 1 cap, 2 breakdown, 3 gave up waiting
+  if (t == 0) {
+    if (blockIdx.x == 0) {
+      a.out[1] = (double)it;
+      raise_to(a.out + 2, (double)(action - 1));  // 0 converged, 1 cap, 2 breakdown
+    }
+    // A block that gave up makes this the outcome, whatever the others made of its words; the norm may be one that
+    // block 0 never formed.
+    if (action == 4) {
+      raise_to(a.out, fp64_nan());
+      raise_to(a.out + 2, 3.0);
+    }
   }
 }
 

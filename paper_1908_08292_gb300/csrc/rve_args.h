@@ -90,12 +90,14 @@ struct MacroSolveArgs {
   const int32_t* halo;      // rows around each block's
   const uint16_t* lcol;     // [nnz] column's place in the block's u
   void* pub;                // 16-byte words: n of u, 4 per block of the partial sums
+  long long wait_limit;     // cycles a block waits for a word of another
 };
 
 struct MacroResident {
   int lanes = 0, rows = 0, blocks = 0;
   size_t smem = 0;
 };
+constexpr long long kMacroWaitCycles = 1ll << 32;  // about 2 s
 MacroResident macro_resident_plan(int dim, int n, int num_sms);
 bool macro_resident_columns(MacroResident& m, int dim, int n, const std::vector<int32_t>& rowptr,
                             const std::vector<int32_t>& col, std::vector<int32_t>& halo_ptr, std::vector<int32_t>& halo,
