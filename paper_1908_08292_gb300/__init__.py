@@ -129,6 +129,15 @@ def _check(rc: int, what: str) -> int:
     return rc
 
 
+def check_macro_info(info):
+    """Host array of a finished macro_solve's info (waits for it) after raising where the solve gave up: its du must
+    not be used."""
+    info = info.cpu().numpy()
+    if info[2] == 3:
+        raise FehmmError("macro_solve: a thread block gave up waiting for another; du is not valid")
+    return info
+
+
 def _dev(t, dtype, name, numel=None):
     """Device pointer of a contiguous CUDA tensor (or None -> NULL)."""
     if t is None:

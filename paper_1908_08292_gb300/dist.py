@@ -24,6 +24,8 @@ from dataclasses import dataclass
 
 import numpy as np
 
+from . import check_macro_info
+
 
 def partition_elements(cost: np.ndarray, world: int) -> list[tuple[int, int]]:
     """Split elements 0..n-1 into `world` contiguous ranges [e0, e1) of nearly equal total cost
@@ -143,6 +145,8 @@ class ShardedIteration:
         if self.shard.rank == 0:
             self.ctx.macro_solve(self.K, self.f, self.du, self.info, rtol=rtol)
         self.shard.share_correction(self.du)
+        self.shard.share_correction(self.info)
+        check_macro_info(self.info)  # every rank holds rank 0's and takes the same way
 
     def __call__(self, u, flags, rtol=1e-10):
         self.solve_local(u, flags)

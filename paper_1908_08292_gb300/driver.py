@@ -25,7 +25,7 @@ import time
 
 import numpy as np
 
-from . import SOLVE_FROM_COMMITTED, Context, FehmmError
+from . import SOLVE_FROM_COMMITTED, Context, FehmmError, check_macro_info
 
 
 class LoadStepDriver:
@@ -158,6 +158,7 @@ class LoadStepDriver:
             passes = 1
         c.macro_dirichlet_load(self.K, new_scale - self.scale, self.g)
         self._solve(self.g)
+        check_macro_info(self.info)
         c.macro_apply_dirichlet(self.u, None, new_scale)  # u[D] = new values; du keeps delta
         return passes
 
@@ -197,7 +198,7 @@ class LoadStepDriver:
         converged = False
         for it in range(self.max_macro + 1):
             self._run(first=(it == 0))
-            info = self.info.cpu().numpy()
+            info = check_macro_info(self.info)
             status = self.st.cpu().numpy()
             if np.any(status > 1):
                 raise FehmmError(f"RVE failure at step {k}, macro iteration {it}: statuses {np.unique(status)}")
