@@ -1829,8 +1829,12 @@ rve2d_kernel(const Rve2dArgs a) {
 // Launch of one instantiation (grid of n_blocks persistent blocks, smem dynamic shared bytes).
 template <typename TA, bool kMG, int LAW, int N = 0>
 inline cudaError_t rve2d_launch_instance(const Rve2dArgs& a, int n_blocks, size_t smem, cudaStream_t stream) {
+  // The limit is one value of the kernel, whoever launches it: set to what the largest grid needs, not to this launch's
+  // share, which another thread's smaller grid would lower between the two calls (129 of 10 000 launches failed with
+  // two threads).
+  constexpr size_t most = offsets2d<TA>(N ? N * N : 2 * kThreads2D).total;
   const cudaError_t err = cudaFuncSetAttribute(rve2d_kernel<TA, kMG, LAW, N>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   if (err != cudaSuccess) return err;
   rve2d_kernel<TA, kMG, LAW, N><<<n_blocks, threads2d<TA>(a.nn_max), smem, stream>>>(a);
   return cudaGetLastError();

@@ -58,6 +58,11 @@ __host__ __device__ constexpr OffsetsD2 offsets_d2(int NN, bool mg) {
   o.total = off;
   return o;
 }
+__host__ __device__ constexpr size_t most_smem_d2(bool mg) {  // over the grids
+  size_t most = 0;
+  for (int n = 2; n <= 32; n += 2) most = offsets_d2(n * n, mg).total > most ? offsets_d2(n * n, mg).total : most;
+  return most;
+}
 // Block scratch (doubles): staged element tangents [36][NN], the stencil [18][2 NN] (grids that do not hold it in
 // registers), then the multigrid: fast region (where not in shared memory) and slow region.  The slow region takes the
 // stencil's place where that is in registers: it has a third of its size.
@@ -1016,8 +1021,9 @@ __global__ void __launch_bounds__(kThreadsD2, 1) rve2d_fp64_kernel(const Rve2dAr
 template <bool kFixed, bool kMG, int LAW, int DPT>
 inline cudaError_t rve2d_launch_fp64(const Rve2dArgs& a, int n_blocks, cudaStream_t stream) {
   const size_t smem = offsets_d2(a.nn_max, kMG).total;
+  constexpr size_t most = most_smem_d2(kMG);  // the kernel's limit for every thread that launches it
   const cudaError_t err = cudaFuncSetAttribute(rve2d_fp64_kernel<kFixed, kMG, LAW, DPT>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   if (err != cudaSuccess) return err;
   rve2d_fp64_kernel<kFixed, kMG, LAW, DPT><<<n_blocks, threads_d2(a.nn_max), smem, stream>>>(a);
   return cudaGetLastError();

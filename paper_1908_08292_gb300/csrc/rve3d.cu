@@ -2061,8 +2061,9 @@ int rve3d_blocks_per_sm(int nn, bool mixed, int count, int num_sms) {
 
 template <typename TA, int LAW>
 cudaError_t rve3d_launch_instance(const Rve2dArgs& a, int n_blocks, int threads, size_t smem, cudaStream_t stream) {
-  const cudaError_t err =
-      cudaFuncSetAttribute(rve3d_kernel<TA, LAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // of the largest grid: the kernel's limit for every thread that launches it
+  const cudaError_t err = cudaFuncSetAttribute(rve3d_kernel<TA, LAW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem3_bytes<TA>(16 * 16 * 16));
   if (err != cudaSuccess) return err;
   rve3d_kernel<TA, LAW><<<n_blocks, threads, smem, stream>>>(a);
   return cudaGetLastError();
