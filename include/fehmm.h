@@ -452,9 +452,10 @@ const char* fehmm_status_str(int code);
  *   w       device double [n_qp][grid_n*grid_n][2]: fluctuation start values in, results
  *           out (the value at node 0 is taken as zero)
  *   F, P, A, status, iters: as in fehmm_rve_solve (A may be NULL: no tangent)
- *   opt     host; dim must be 2 and precision FEHMM_PREC_FP64; tolerances, caps, bc and precond
- *           (anything but FEHMM_PRECOND_BLOCK_JACOBI: multigrid on the grids that have it, and
- *           block-Jacobi where its PCG breaks down) used; law must be FEHMM_LAW_NEO_HOOKE (else
+ *   opt     host; dim must be 2 and precision FEHMM_PREC_FP64; tolerances, caps, bc, precond,
+ *           mg_omega and mg_reuse used (multigrid on the grids that have it, and block-Jacobi where
+ *           its PCG breaks down; block-Jacobi with FEHMM_PRECOND_BLOCK_JACOBI, and with an mg_omega
+ *           outside (0, 1), which is not refused here); law must be FEHMM_LAW_NEO_HOOKE (else
  *           FEHMM_ERR_UNSUPPORTED)
  * The first call on a device looks up the device address of the static array (with that
  * device current); make that first call before any stream capture.  All calls share the

@@ -116,14 +116,16 @@ extern "C" int fehmm_rve2d_solve_fp64_noalloc(int n_qp, int grid_n, int phase_pe
   a.max_cg = opt->max_cg;
   a.max_cond_cg = opt->max_cond_cg;
   a.retry_stages = opt->retry_stages;
-  // Multigrid for the grids that have a hierarchy (6, 8, 12, 16) unless block-Jacobi is asked for: its levels live in
-  // shared memory, its coarse element matrices in the part of the scratch that larger grids use for the stencil.
-  // 150 RVEs of 16 x 16: 5.1 -> 3.3 ms, 200 of 8 x 8: 1.45 -> 1.24 ms.
-  a.mg = opt->precond != FEHMM_PRECOND_BLOCK_JACOBI ? 1 : 0;
+  // Multigrid for the grids that have a hierarchy (6, 8, 12, 16) unless block-Jacobi is asked for, with the smoother's
+  // damping and the reuse of levels of the options: its levels live in shared memory, its coarse element matrices in the
+  // part of the scratch that larger grids use for the stencil.  150 RVEs of 16 x 16: 5.1 -> 3.3 ms, 200 of 8 x 8:
+  // 1.45 -> 1.24 ms.  Options without a damping in (0, 1) are accepted here, where a context refuses them, and take
+  // block-Jacobi.
+  a.mg = opt->precond != FEHMM_PRECOND_BLOCK_JACOBI && opt->mg_omega > 0.0 && opt->mg_omega < 1.0 ? 1 : 0;
   a.bc = opt->bc == FEHMM_BC_KUBC ? 1 : 0;
   a.law = 0;
-  a.mg_omega = 0.7f;
-  a.mg_reuse = 1;
+  a.mg_omega = (float)opt->mg_omega;
+  a.mg_reuse = opt->mg_reuse != 0;
   a.X_in = nullptr;  // no kept transfer solutions: every transfer solve starts from zero
   a.X_out = nullptr;
   a.scratch_stride = 72LL * a.nn_max;
