@@ -142,12 +142,29 @@ __device__ __forceinline__ int block_dot2(T a, T b, double* buf, double stop, T&
   return *flags;
 }
 
-// 1/J for the FP64 neo-Hookean stress of the residuals: the FP32 approximate reciprocal (rcp.approx, relative error
-// below 2^-22) refined by one third-order step in FP64, x <- x + x (e + e^2) with e = 1 - J x, which cubes the
-// relative error (below FP64 rounding).  Conversions are FP64-pipe instructions too, so J's FP32 value and the
-// reciprocal's FP64 value are put together from their bits where both are normal FP32 numbers: three FP64
-// instructions in all.  J below FP32's normal range (a collapsed element) gives a non-finite result, which the Newton
-// loop treats like J <= 0.
+// FP64 reciprocals without the FP64 instructions of a division (about nine; an FP64 instruction holds an SM
+// sub-partition for 64 cycles): the hardware's FP32 approximation x0 (rcp.approx, error at most one FP32 ulp), then one
+// step of the hyperpower iteration of order 3, x = x0 + x0 (e + e^2) with e = 1 - a x0.  Its error is e^3, below 2^-65
+// of the result, so what is left is the rounding of the last operation: within one ulp of 1 / a.
+
+// 1 / x for every x: normal positive x below 2^1018 with its exponent split off, which keeps the mantissa in FP32's
+// range; any other (zero, subnormal, negative, infinite, NaN) by the division.
+__device__ __forceinline__ double recip_d(double x) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (e == 0 || e > 2040 || hi < 0) return 1.0 / x;
+  const double m = __hiloint2double((hi & 0xfffff) | (1023 << 20), __double2loint(x));
+  float f;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"((float)m));
+  double q = (double)f;
+  const double err = fma(-m, q, 1.0);
+  q = fma(q, fma(err, err, err), q);
+  return __hiloint2double(__double2hiint(q) + ((1023 - e) << 20), __double2loint(q));
+}
+
+// 1/J for the FP64 stress of the residuals, J in FP32's normal range: 2^-126 <= J < 2^126.  Conversions are FP64-pipe
+// instructions too, so J's FP32 value and the reciprocal's FP64 value are put together from their bits there: three
+// FP64 instructions in all.  Negative J of that range by conversions, as accurate.  A smaller |J| (a collapsed element)
+// gives a non-finite result, which the Newton loop treats like J <= 0, a larger one zero.
 __device__ __forceinline__ double recip_fp64(double J) {
   float r;
   double x;

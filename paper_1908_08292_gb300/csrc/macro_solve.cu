@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "fehmm_device.cuh"
 #include "rve_args.h"
 
 namespace cg = cooperative_groups;
@@ -255,20 +256,6 @@ __device__ __forceinline__ bool get_all(int count, unsigned long long seq, long 
   return ok;
 }
 
-// 1 / x for positive normal x: the FP32 reciprocal of the mantissa refined by two Newton steps in FP64 (within an
-// ulp or so; a division takes about four times the FP64 instructions, and the iteration waits for this one).
-__device__ __forceinline__ double recip(double x) {
-  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
-  if (e == 0 || e > 2040 || hi < 0) return 1.0 / x;
-  const double m = __hiloint2double((hi & 0xfffff) | (1023 << 20), __double2loint(x));
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"((float)m));
-  double q = (double)r;
-  q = fma(q, fma(-m, q, 1.0), q);
-  q = fma(q, fma(-m, q, 1.0), q);
-  return __hiloint2double(__double2hiint(q) + ((1023 - e) << 20), __double2loint(q));
-}
-
 // L lanes per row, at most PER nonzeros per lane.
 template <int L, int PER>
 __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(const MacroSolveArgs a) {
@@ -384,7 +371,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
         return;
       }
       den = delta;
-      total[0] = gamma * recip(delta);
+      total[0] = gamma * recip_d(delta);
       total[1] = 0.0;
     });
   }
@@ -396,7 +383,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
     publish();
     p = fma(beta, p, u_old);  // off the path of u: while it travels
     x = fma(alpha, p, x);
-    if (t == 0) rgamma = recip(gamma);
+    if (t == 0) rgamma = recip_d(gamma);
     product();
     reduce(ll < 2 ? u * (ll ? w : r) : 0.0, [&](double g, double dl) {
       ++it;
@@ -414,7 +401,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
         action = 3;
         return;
       }
-      total[0] = g * recip(den);
+      total[0] = g * recip_d(den);
       total[1] = b;
       gamma = g;
     });

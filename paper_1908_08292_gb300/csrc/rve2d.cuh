@@ -899,19 +899,6 @@ __device__ __forceinline__ void mg_stencil_block(const TA* ke, int n, int i, int
     }
 }
 
-// 1 / x for finite positive normal x (exponent split off, FP32 reciprocal of the mantissa refined twice); else 1 / x
-__device__ __forceinline__ double recip_d(double x) {
-  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
-  if (e == 0 || e > 2040 || hi < 0) return 1.0 / x;
-  const double m = __hiloint2double((hi & 0xfffff) | (1023 << 20), __double2loint(x));
-  float f;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"((float)m));
-  double q = (double)f;
-  const double err = fma(-m, q, 1.0);
-  q = fma(q, fma(err, err, err), q);
-  return __hiloint2double(__double2hiint(q) + ((1023 - e) << 20), __double2loint(q));
-}
-
 // One entry of a Gauss-Jordan step: a - aik akj ip, in the pivot's column (own) -aik ip.  In FP64 with the pivot
 // row's kj = akj ip formed once, one FP64 instruction an entry.
 __device__ __forceinline__ float dense_update(float a, float aik, float akj, float ip, float, bool own) {
