@@ -31,10 +31,11 @@ from .rve import STATUS_J_NONPOS, STATUS_NEWTON_CAP, STATUS_NONFINITE, STATUS_OK
 
 class DirichletRVE:
     """One microstructure on an n^d element grid of the unit cell, (n+1)^d nodes, w = 0 on the
-    boundary nodes."""
+    boundary nodes; law "nh" (neo-Hookean) or "svk" (St. Venant-Kirchhoff), see material.LAWS."""
 
-    def __init__(self, n, dim, phase, E, nu):
+    def __init__(self, n, dim, phase, E, nu, law="nh"):
         self.n, self.d = int(n), int(dim)
+        self.psi_law, self.P_law, self.A_law = mat.LAWS[law]
         d, n = self.d, self.n
         self.phase = np.asarray(phase, dtype=np.int64).reshape(-1)
         assert self.phase.size == n ** d
@@ -61,7 +62,7 @@ class DirichletRVE:
 
     def residual(self, w, Fbar):
         F = self.F_at_qps(w, Fbar)
-        P = mat.P_of_F(F, self.lam_e[:, None], self.mu_e[:, None])
+        P = self.P_law(F, self.lam_e[:, None], self.mu_e[:, None])
         Re = self.wdet * np.einsum("eqiJ,qaJ->eai", P, self.G)
         R = np.zeros((self.n_nodes, self.d))
         np.add.at(R, self.conn, Re)
@@ -69,7 +70,7 @@ class DirichletRVE:
 
     def tangent(self, w, Fbar):
         F = self.F_at_qps(w, Fbar)
-        A = mat.A_of_F(F, self.lam_e[:, None], self.mu_e[:, None])
+        A = self.A_law(F, self.lam_e[:, None], self.mu_e[:, None])
         ke = self.wdet * np.einsum("qaJ,eqiJkL,qbL->eaibk", self.G, A, self.G)
         nen, d = self.G.shape[1], self.d
         dofs = (self.conn[:, :, None] * d + np.arange(d)[None, None, :]).reshape(self.conn.shape[0], -1)
@@ -105,15 +106,15 @@ class DirichletRVE:
         F = self.F_at_qps(w, Fbar)
         lam, mu = self.lam_e[:, None], self.mu_e[:, None]
         s = self.wdet
-        return (s * mat.P_of_F(F, lam, mu).sum(axis=(0, 1)), s * F.sum(axis=(0, 1)),
-                s * mat.psi(F, lam, mu).sum(), s * mat.A_of_F(F, lam, mu).sum(axis=(0, 1)))
+        return (s * self.P_law(F, lam, mu).sum(axis=(0, 1)), s * F.sum(axis=(0, 1)),
+                s * self.psi_law(F, lam, mu).sum(), s * self.A_law(F, lam, mu).sum(axis=(0, 1)))
 
     def condensed_tangent(self, w, Fbar):
         """Abar = <A> - L_f^T K_ff^-1 L_f over the interior dofs, L = dR/dFbar."""
         d = self.d
         _, _, _, Am = self.averages(w, Fbar)
         F = self.F_at_qps(w, Fbar)
-        A = mat.A_of_F(F, self.lam_e[:, None], self.mu_e[:, None])
+        A = self.A_law(F, self.lam_e[:, None], self.mu_e[:, None])
         Le = self.wdet * np.einsum("qaJ,eqiJkL->eaikL", self.G, A)
         L = np.zeros((self.n_nodes, d, d, d))
         np.add.at(L, self.conn, Le)
