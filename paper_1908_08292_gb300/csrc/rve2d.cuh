@@ -802,8 +802,6 @@ __device__ __forceinline__ void mg_coarse_element(const TA* kf, int nf, int E, T
   for (int q = 0; q < 36; ++q) kc[(size_t)q * nnc + E] = acc[q];
 }
 
-// Periodic neighbours without integer division.
-
 // y = K_l z at node v = (i, j) of a coarse level (zero at the pinned node).
 template <typename TA>
 __device__ __forceinline__ vec2_t<TA> mg_apply(const MgLevel<TA>& L, const vec2_t<TA>* z, int i, int j) {

@@ -10,8 +10,9 @@
 //
 // GB300 layout:
 //  * One block per RVE, up to 512 threads and one block per SM, or several of up to 256 (rve3d_threads,
-//    rve3d_blocks_per_sm); the points of each grid size are a launch of their own.  The apply's vectors, in mixed mode also the FP32 fluctuation, the
-//    residual and the coarse vectors, live in shared memory; the other PCG vectors stream from per-block scratch.
+//    rve3d_blocks_per_sm); the points of each grid size are a launch of their own.  The apply's vectors, in mixed
+//    mode also the FP32 fluctuation, the residual and the coarse vectors, live in shared memory; the other PCG vectors
+//    stream from per-block scratch.
 //  * Residual and tangent apply: two lanes per element, one for each plane of four Gauss points (Cell3).  The FP64
 //    residual stages element forces in global scratch and gathers them per node; the apply, matrix-free in TA
 //    (FP32 in mixed mode), evaluates F again and adds corner by corner without atomics (deterministic sums).
@@ -591,8 +592,6 @@ struct Ctx3 {
   Mg3<TA> mg;
   const uint8_t* phase;
   const double* lame;  // shared [kMaxPhase][2]
-  const TA* lame_t;    // the same in the arithmetic type (a conversion from FP64 costs an FP64 instruction),
-  TA* Fb_t;            // and Fbar of the current stage, both shared
   Scratch3<TA> sc;
   TA* vin;   // shared [3][NN]
   TA* vout;  // shared [3][NN]
@@ -1078,8 +1077,9 @@ __device__ __noinline__ void unit_gradient3(const Ctx3<TA>& c, int cidx) {
 //                 w [mu d_ik g_a.g_b + gm v_a,i v_b,k - hb v_b,i v_a,k],  v = Fit g,
 // with g the gradients of E's trilinear shape functions — the fine bilinear form evaluated on
 // the coarse functions, i.e. P^T K P.  Deeper levels follow from the element blocks with the
-// trilinear weights.  All multigrid data live in the block's global scratch; coarse applies
-// gather per node (no atomics).
+// trilinear weights.  Element blocks, stencils, smoother blocks and the coarsest inverse live in the
+// block's global scratch; the vectors r, z and t of the levels in shared memory in mixed mode, in the
+// scratch in FP64 mode.  Coarse applies gather per node (no atomics).
 // The smoother must contract in the energy norm for the V-cycle to stay positive definite:
 // omega < 2 / lambda_max(D^-1 K).  For Hex8 elasticity lambda_max is about 3.0 (measured on the
 // 8^3 two-sphere RVE), so omega = 0.7 (used in 2D, where lambda_max is about 2.3) is too large
@@ -1738,9 +1738,10 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
   double* lame_s = c.red + 2 * 512;
   double* misc = lame_s + 2 * kMaxPhase;
   c.lame = lame_s;
+  // in the arithmetic type for the apply (a conversion from FP64 costs an FP64 instruction): the Lame table, and Fbar of
+  // the current stage
   TA* lame_t = reinterpret_cast<TA*>(smem + kSmem3LameT);
-  c.lame_t = lame_t;
-  c.Fb_t = lame_t + 2 * kMaxPhase;
+  TA* Fb_t = lame_t + 2 * kMaxPhase;
   c.vin = reinterpret_cast<TA*>(smem + kSmem3Fixed);
   c.vout = c.vin + 3 * NN;
   c.w32 = nullptr;
@@ -1765,7 +1766,7 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
   }
 #pragma unroll
   for (int k = 0; k < 9; ++k) c.Fb[k] = a.F[(size_t)qp * 9 + k];
-  if (threadIdx.x < 9) c.Fb_t[threadIdx.x] = (TA)a.F[(size_t)qp * 9 + threadIdx.x];
+  if (threadIdx.x < 9) Fb_t[threadIdx.x] = (TA)a.F[(size_t)qp * 9 + threadIdx.x];
   const double* w_in = a.w_in + a.qp_w_off[qp];
   double* w = a.w_out + a.qp_w_off[qp];
   c.w = w;
@@ -1896,7 +1897,7 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
       c.Fb[k] = stage == stages ? Ft[k] : (k % 4 == 0 ? 1.0 : 0.0) + (Ft[k] - (k % 4 == 0 ? 1.0 : 0.0)) * stage / stages;
     if (threadIdx.x == 0)
 #pragma unroll
-      for (int k = 0; k < 9; ++k) c.Fb_t[k] = (TA)c.Fb[k];
+      for (int k = 0; k < 9; ++k) Fb_t[k] = (TA)c.Fb[k];
     __syncthreads();
   }
   const int it = it_total;

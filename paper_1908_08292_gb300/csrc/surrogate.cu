@@ -699,7 +699,8 @@ extern "C" int fehmm_surrogate_eval(fehmm_mlp* mlp, const fehmm_surrogate_params
   if (!mlp || !sp || !F || !P || !inside || !work || n <= 0) return FEHMM_ERR_ARG;
   if (!(sp->sx > 0) || !(sp->sg > 0) || !(sp->radius >= 0)) return FEHMM_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  float* x = work + 2 * kPolyTerms;  // [n][6], behind a region that is not used any more
+  // work keeps the size and the alignment that callers know, although nothing is stored in its first part
+  float* x = work + 2 * kPolyTerms;  // [n][6]
   float* y = x + (size_t)n * 6;      // [n]
   float* g = y + n;                  // [n][6]
   float* H = g + (size_t)n * 6;      // [n][36]
