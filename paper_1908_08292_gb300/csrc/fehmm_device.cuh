@@ -161,6 +161,14 @@ __device__ __forceinline__ double recip_d(double x) {
   return __hiloint2double(__double2hiint(q) + ((1023 - e) << 20), __double2loint(q));
 }
 
+// a / x by recip_d.  A subnormal x, whose reciprocal may overflow where the quotient does not (a CG that started from
+// sums of 1e-300), takes the division, as do the others that recip_d divides for.
+__device__ __forceinline__ double div_d(double a, double x) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (e == 0 || e > 2040 || hi < 0) return a / x;
+  return a * recip_d(x);
+}
+
 // 1/J for the FP64 stress of the residuals, J in FP32's normal range: 2^-126 <= J < 2^126.  Conversions are FP64-pipe
 // instructions too, so J's FP32 value and the reciprocal's FP64 value are put together from their bits there: three
 // FP64 instructions in all.  Negative J of that range by conversions, as accurate.  A smaller |J| (a collapsed element)

@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
         return;
       }
       den = delta;
-      total[0] = gamma * recip_d(delta);
+      total[0] = div_d(gamma, delta);
       total[1] = 0.0;
     });
   }
@@ -395,13 +395,14 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) macro_pcg_resident_kernel(c
         action = 2;
         return;
       }
-      const double b = g * rgamma;
+      // infinite: gamma is subnormal (g / gamma may be an ordinary number)
+      const double b = __double2hiint(rgamma) == 0x7ff00000 ? g / gamma : g * rgamma;
       den = fma(-b * b, den, dl);  // d - beta g / alpha, with alpha = gamma / (the last) den
       if (!(den > 0.0)) {
         action = 3;
         return;
       }
-      total[0] = g * recip_d(den);
+      total[0] = div_d(g, den);
       total[1] = b;
       gamma = g;
     });

@@ -588,7 +588,7 @@ __device__ int pcg_d2(const D2<DPT, LAW>& s, const Row<DPT>& R, const double (&M
           out[0] = g / -d;
         } else {
           den = d;
-          out[0] = g * recip_d(d);
+          out[0] = div_d(g, d);
           out[1] = 0.0;
           if (it >= max_it) code = 2;
         }
@@ -597,12 +597,12 @@ __device__ int pcg_d2(const D2<DPT, LAW>& s, const Row<DPT>& R, const double (&M
       } else if (g <= stop) {
         code = 1;
       } else {
-        const double beta = g * recip_d(gamma), dn = fma(-beta * beta, den, d);  // p_new^T K p_new
+        const double beta = div_d(g, gamma), dn = fma(-beta * beta, den, d);  // p_new^T K p_new
         if (!(dn > 0.0)) {
           code = truncate && dn < 0.0 ? 4 : 3;
         } else {
           den = dn;
-          out[0] = g * recip_d(dn);
+          out[0] = div_d(g, dn);
           out[1] = beta;
           if (it + 1 >= max_it) code = 2;
         }
