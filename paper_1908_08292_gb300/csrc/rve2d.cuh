@@ -1705,23 +1705,31 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
           b[3] = b1.y;
         }
         int pst = kStatusOk, ci = 0;
+        bool kept = warm;
         for (;;) {  // as for the Newton corrections: a breakdown is retried with half the damping
-          if (warm && o.active) {
+          if (kept && o.active) {
 #pragma unroll
             for (int s = 0; s < 2; ++s)
               X[c * NN + o.node[s]] = o.pin[s] ? mk2<TA>(TA(0), TA(0)) : X0[c * NN + o.node[s]];
           }
           ci += pcg_pair<TA, kMG>(S, o, Minv, mg, b, X + c * NN, (TA)a.cond_rtol, a.max_cond_cg, sm.p, redD,
-                                       &pst, false, warm);
+                                       &pst, false, kept);
           __syncthreads();
           if (reuse_t && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap)) {
             redo = true;
             break;
           }
-          if (!(kMG && mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) &&
-                mg.omega > TA(0.2) * omega0))
+          if (kMG && mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) &&
+              mg.omega > TA(0.2) * omega0) {
+            mg.omega *= TA(0.5);
+          } else if (kept && pst == kStatusPcgBreakdown) {
+            // A right-hand side far below the kept solution's (zero or rounding in a homogeneous RVE): the tolerance
+            // is relative to it and out of reach from there.  From zero it is not.
+            kept = false;
+            mg.omega = omega0;
+          } else {
             break;
-          mg.omega *= TA(0.5);
+          }
           pst = kStatusOk;
         }
         mg.omega = omega0;

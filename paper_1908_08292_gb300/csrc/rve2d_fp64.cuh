@@ -925,22 +925,28 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
 #pragma unroll
         for (int q = 0; q < DPT; ++q) b[q] = s.act[q] ? Lb[(size_t)k * ND + s.dof[q]] : 0.0;
         int pst = kStatusOk, ci = 0;
+        bool kept = warm;
         for (;;) {
-          if (warm) {
+          if (kept) {
 #pragma unroll
             for (int q = 0; q < DPT; ++q)
               if (s.act[q]) Xs[(size_t)k * ND + s.dof[q]] = s.pin[q] ? 0.0 : X0[(size_t)k * ND + s.dof[q]];
           }
-          ci += pcg_d2<DPT, LAW, kMG>(s, R, Mi, b, Xs + (size_t)k * ND, a.cond_rtol, a.max_cond_cg, &pst, false, warm);
+          ci += pcg_d2<DPT, LAW, kMG>(s, R, Mi, b, Xs + (size_t)k * ND, a.cond_rtol, a.max_cond_cg, &pst, false, kept);
           __syncthreads();
           if (reuse_t && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap)) {
             redo = true;
             break;
           }
-          if (!(kMG && s.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap))) break;
-          if (s.mg.omega > 0.2 * omega0) s.mg.omega *= 0.5;
-          else if (kFixed) s.mg.levels = 0;
-          else break;
+          if (kMG && s.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) && (kFixed || s.mg.omega > 0.2 * omega0)) {
+            if (s.mg.omega > 0.2 * omega0) s.mg.omega *= 0.5;
+            else s.mg.levels = 0;
+          } else if (kept && pst == kStatusPcgBreakdown) {  // from zero (see solve_item_2d)
+            kept = false;
+            s.mg.omega = omega0;
+          } else {
+            break;
+          }
           pst = kStatusOk;
         }
         s.mg.omega = omega0;

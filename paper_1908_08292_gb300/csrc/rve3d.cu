@@ -1950,22 +1950,30 @@ __device__ void solve_item_3d(const Rve2dArgs& a, int qp, unsigned char* smem, u
     const TA omega0 = c.mg.omega;
     for (int cp = 0; cp < 9; ++cp) {
       int pst = kStatusOk, ci = 0;
+      bool kept = warm;
       for (;;) {  // as for the Newton corrections: a breakdown is retried with half the damping
         for (int v = threadIdx.x; v < 3 * NN; v += blockDim.x) {
           c.sc.r[v] = -c.sc.L[(size_t)cp * 3 * NN + v];
-          if (warm) c.sc.x[v] = X0[(size_t)cp * 3 * NN + v];
+          if (kept) c.sc.x[v] = X0[(size_t)cp * 3 * NN + v];
         }
         __syncthreads();
-        ci += pcg3<TA, LAW>(c, (TA)a.cond_rtol, a.max_cond_cg, false, &pst, warm);
+        ci += pcg3<TA, LAW>(c, (TA)a.cond_rtol, a.max_cond_cg, false, &pst, kept);
         if (reuse_t && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap)) {
           mg3_build<TA, LAW>(c);
           reuse_t = false;
           pst = kStatusOk;
           continue;
         }
-        if (!(c.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) && c.mg.omega > TA(0.2) * omega0))
+        if (c.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) && c.mg.omega > TA(0.2) * omega0) {
+          c.mg.omega *= TA(0.5);
+        } else if (kept && pst == kStatusPcgBreakdown) {
+          // a right-hand side far below the kept solution's (zero or rounding in a homogeneous RVE): the tolerance is
+          // relative to it and out of reach from there, but not from zero
+          kept = false;
+          c.mg.omega = omega0;
+        } else {
           break;
-        c.mg.omega *= TA(0.5);
+        }
         pst = kStatusOk;
       }
       c.mg.omega = omega0;
