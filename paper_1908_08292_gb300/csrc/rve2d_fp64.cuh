@@ -724,6 +724,17 @@ __device__ __forceinline__ void transfer_d2(const D2<DPT, LAW>& s, const double*
   }
 }
 
+// Whether a PCG that ended so is tried again with another preconditioner (fresh levels, less damping, block-Jacobi): a
+// breakdown, and a cap that tells of one.  The no-allocation entry's callers may cap the PCG to truncate it: multigrid
+// takes 10 to 25 iterations to the default tolerances (stiffness ratios up to 1000), so a cap below kTellingCap that
+// binds is a truncation, whose step is taken as it is.  (Tried six times, 40 RVEs of 6^2 to 16^2 with caps of 2 to 20
+// took 6.0 to 10.8 times as long as with block-Jacobi, which that entry ran before it had multigrid.)
+constexpr int kTellingCap = 64;
+template <bool kFixed>
+__device__ __forceinline__ bool mends(int pst, int cap) {
+  return pst == kStatusPcgBreakdown || (pst == kStatusPcgCap && (!kFixed || cap >= kTellingCap));
+}
+
 template <bool kFixed, bool kMG, int LAW, int DPT>
 __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, double* scr) {
   const int tid = threadIdx.x;
@@ -846,11 +857,12 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
         build_d2<DPT, LAW, kMG>(s, R, Mi, false, nullptr, !reuse);
         cg_total += pcg_d2<DPT, LAW, kMG>(s, R, Mi, b, s.x, a.cg_rtol, a.max_cg, &pst, true, false);
         __syncthreads();
-        if (reuse && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap || pst == kStatusNegCurv)) {
+        const bool mended = mends<kFixed>(pst, a.max_cg);
+        if (reuse && (mended || pst == kStatusNegCurv)) {
           reuse = false;
-        } else if (kMG && s.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) && s.mg.omega > 0.2 * omega0) {
+        } else if (kMG && s.mg.levels && mended && s.mg.omega > 0.2 * omega0) {
           s.mg.omega *= 0.5;
-        } else if (kFixed && kMG && s.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap)) {
+        } else if (kFixed && kMG && s.mg.levels && mended) {
           s.mg.levels = 0;  // block-Jacobi, the entry's preconditioner for grids without a hierarchy
         } else {
           break;
@@ -934,11 +946,12 @@ __device__ void solve_item_d2(const Rve2dArgs& a, int qp, unsigned char* smem, d
           }
           ci += pcg_d2<DPT, LAW, kMG>(s, R, Mi, b, Xs + (size_t)k * ND, a.cond_rtol, a.max_cond_cg, &pst, false, kept);
           __syncthreads();
-          if (reuse_t && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap)) {
+          const bool mended = mends<kFixed>(pst, a.max_cond_cg);
+          if (reuse_t && mended) {
             redo = true;
             break;
           }
-          if (kMG && s.mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) && (kFixed || s.mg.omega > 0.2 * omega0)) {
+          if (kMG && s.mg.levels && mended && (kFixed || s.mg.omega > 0.2 * omega0)) {
             if (s.mg.omega > 0.2 * omega0) s.mg.omega *= 0.5;
             else s.mg.levels = 0;
           } else if (kept && pst == kStatusPcgBreakdown) {  // from zero (see solve_item_2d)

@@ -70,17 +70,30 @@ def test_no_damping_is_block_jacobi(omega):
 
 
 def test_multigrid_gives_way_to_block_jacobi():
-    """A cap of three PCG iterations, which no solve meets at these tolerances: every Newton correction is tried with the
-    levels kept from the last tangent (from the second on), with fresh ones at the damping 0.7, 0.35, 0.175 and 0.0875,
-    and then with block-Jacobi, whose truncated step is taken.  Newton still converges to the oracle's solution.  With
-    the cap on the transfer instead, its four solves go the same way (the first once more, for the kept levels), and the
-    point is reported."""
+    """A cap of 64 PCG iterations and a tolerance of 1e-150, which none of them meets: every Newton correction is tried
+    with the levels kept from the last tangent (from the second on), with fresh ones at the damping 0.7, 0.35, 0.175 and
+    0.0875, and then with block-Jacobi, whose step is taken.  Newton converges to the oracle's solution.  So do the
+    transfer's four solves with that cap and tolerance (the first once more, for the kept levels), which the status
+    reports."""
     phases, Fs = problem(8, 3, 0.02)
-    got = noalloc(8, phases, Fs, max_cg=3, max_newton=2000)
+    capped = noalloc(8, phases, Fs, max_cg=64, cg_rtol=1e-150)
+    transfer = noalloc(8, phases, Fs, max_cond_cg=64, cond_rtol=1e-150)
+    assert np.all(capped["status"] == 0) and np.all(transfer["status"] == 5)
+    np.testing.assert_array_equal(capped["iters"][:, 1], 64 * (5 + 6 * (capped["iters"][:, 0] - 1)))
+    assert np.all(transfer["iters"][:, 2] == 64 * (1 + 4 * 5)) and np.all(transfer["iters"][:, 3] == 64 * 5)
     for q in range(3):
-        assert got["status"][q] == 0 and got["iters"][q, 0] > 4
-        assert got["iters"][q, 1] == 3 * (5 + 6 * (got["iters"][q, 0] - 1))
         ref = PeriodicRVE(8, 2, phases[q], E, NU).solve(Fs[q], rtol=1e-14, atol=1e-16)
-        assert rel_err(got["P"][q], ref["P"], 1e-3) < TOL and rel_err(got["A"][q], ref["A"], 1e-3) < TOL
-    got = noalloc(8, phases, Fs, max_cond_cg=3)
-    assert np.all(got["status"] == 5) and np.all(got["iters"][:, 2] == 3 + 4 * 5 * 3) and np.all(got["iters"][:, 3] == 15)
+        for got in (capped, transfer):
+            assert rel_err(got["P"][q], ref["P"], 1e-3) < TOL and rel_err(got["A"][q], ref["A"], 1e-3) < TOL
+
+
+@pytest.mark.parametrize("cap", [1, 3, 12, 63])
+def test_a_low_cap_truncates(cap):
+    """Below 64 a cap that binds is the caller's truncation: no correction and no transfer solve takes more iterations
+    than it, as with block-Jacobi."""
+    phases, Fs = problem(8, 3, 0.02)
+    for precond in (0, 1):
+        newton = noalloc(8, phases, Fs, max_cg=cap, cg_rtol=1e-150, max_newton=5, precond=precond)
+        transfer = noalloc(8, phases, Fs, max_cond_cg=cap, cond_rtol=1e-150, precond=precond)
+        np.testing.assert_array_equal(newton["iters"][:, 1], cap * newton["iters"][:, 0])
+        assert np.all(transfer["status"] == 5) and np.all(transfer["iters"][:, 2] == 4 * cap)
