@@ -254,6 +254,7 @@ int fehmm_bind_qps(fehmm_ctx* c, int n_qp, const int32_t* rve_of_qp) {
   const int n_rve = (int)c->rve_n.size(), d = c->opt.dim;
   for (int q = 0; q < n_qp; ++q)
     if (rve_of_qp[q] < 0 || rve_of_qp[q] >= n_rve) return FEHMM_ERR_ARG;
+  c->n_qp = 0;  // until every array is of the new binding: a call that fails on the way leaves the context unbound
   int rc;
   if ((rc = dupload(c->d_rve_n, c->rve_n.data(), c->rve_n.size())) ||
       (rc = dupload(c->d_rve_phase_off, c->rve_phase_off.data(), c->rve_phase_off.size())) ||
@@ -287,7 +288,6 @@ int fehmm_bind_qps(fehmm_ctx* c, int n_qp, const int32_t* rve_of_qp) {
     cudaGetLastError();
     dfree(c->d_w_cur);
     dfree(c->d_w_comm);
-    c->n_qp = 0;
     return FEHMM_ERR_OOM;
   }
   if (cudaMemset(c->d_w_cur, 0, sizeof(double) * total) != cudaSuccess ||
@@ -305,7 +305,6 @@ int fehmm_bind_qps(fehmm_ctx* c, int n_qp, const int32_t* rve_of_qp) {
       if (c->d_x_cur) cudaFree(c->d_x_cur);
       if (c->d_x_comm) cudaFree(c->d_x_comm);
       c->d_x_cur = c->d_x_comm = nullptr;
-      c->n_qp = 0;
       return FEHMM_ERR_OOM;
     }
     if (cudaMemset(c->d_x_cur, 0, xb) != cudaSuccess || cudaMemset(c->d_x_comm, 0, xb) != cudaSuccess)
@@ -331,13 +330,11 @@ int fehmm_bind_qps(fehmm_ctx* c, int n_qp, const int32_t* rve_of_qp) {
     if ((!c->fork && cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess) ||
         cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
       cudaGetLastError();
-      c->n_qp = 0;
       return FEHMM_ERR_CUDA;
     }
     if (cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking) != cudaSuccess) {
       cudaEventDestroy(e);
       cudaGetLastError();
-      c->n_qp = 0;
       return FEHMM_ERR_CUDA;
     }
     c->side.push_back(t);
@@ -580,6 +577,7 @@ int fehmm_macro_create(fehmm_ctx* c, const int32_t* n_el) {
         blk_base[((size_t)e * nen + I) * nen + J] = node_base[nI] + rank * d;
       }
     }
+  c->has_macro = false;  // until every array is of the new mesh
   int rc;
   if ((rc = dupload(c->d_rowptr, rowptr.data(), rowptr.size())) || (rc = dupload(c->d_col, col.data(), col.size())) ||
       (rc = dupload(c->d_blk_base, blk_base.data(), blk_base.size())) ||
