@@ -578,6 +578,10 @@ int fehmm_macro_create(fehmm_ctx* c, const int32_t* n_el) {
       }
     }
   c->has_macro = false;  // until every array is of the new mesh
+  c->n_fixed = 0;        // the old mesh's Dirichlet data number its dofs
+  dfree(c->d_fixed_dofs);
+  dfree(c->d_fixed_vals);
+  dfree(c->d_dir_full);
   int rc;
   if ((rc = dupload(c->d_rowptr, rowptr.data(), rowptr.size())) || (rc = dupload(c->d_col, col.data(), col.size())) ||
       (rc = dupload(c->d_blk_base, blk_base.data(), blk_base.size())) ||

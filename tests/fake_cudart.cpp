@@ -1,14 +1,15 @@
 // A stand-in for the CUDA runtime on the CPU, for tests of the library's host code: device memory is host memory,
 // kernels are not run, and one call can be made to fail.  fake_fail(k): the k-th call from now of those that can fail
 // for want of memory or resources returns an error (0: none does); it returns the number of such calls since the last
-// fake_fail.  fake_blocks: allocations not yet freed.
+// fake_fail.  fake_blocks: allocations not yet freed.  fake_watch(a): remember the int that is argument a of the launches
+// that follow; it returns the last one.
 #include <cuda_runtime_api.h>
 #include <stdlib.h>
 #include <string.h>
 
 #include <set>
 
-static int g_fail = 0, g_calls = 0;
+static int g_fail = 0, g_calls = 0, g_arg = -1, g_seen = 0;
 static std::set<void*> g_blocks;
 static bool fails() { return ++g_calls == g_fail; }
 
@@ -18,6 +19,11 @@ int fake_fail(int k) {
   g_fail = k;
   g_calls = 0;
   return n;
+}
+int fake_watch(int arg) {
+  const int seen = g_seen;
+  g_arg = arg;
+  return seen;
 }
 int fake_blocks() { return (int)g_blocks.size(); }
 
@@ -91,7 +97,10 @@ cudaError_t cudaLaunchCooperativeKernel(const void*, dim3, dim3, void**, size_t,
 unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, void*) { return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3*, dim3*, size_t*, void*) { return cudaSuccess; }
 cudaError_t __cudaGetKernel(cudaKernel_t*, const void*) { return cudaSuccess; }
-cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void**, size_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void** args, size_t, cudaStream_t) {
+  if (g_arg >= 0) g_seen = *(int*)args[g_arg];
+  return cudaSuccess;
+}
 void** __cudaRegisterFatBinary(void*) { return nullptr; }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
