@@ -77,8 +77,8 @@ FP64_PEAK_TFLOPS = 1.25                              # GB300 nominal FP64
 # DRAM bytes per RVE solve of the dominant kernel from an ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum of one launch / RVEs in that launch), with the profile summary it comes
 # from; scaled to a launch of the bench by the RVEs it solves.  Only for a capture of the kernel
-# build the bench runs; the 3D capture (23.9 MB per RVE) predates the kernel that reads the
-# fluctuation in place of stored Gauss-point data, so it has no entry.
+# build the bench runs and of its mix of states; the 3D capture is of 64 RVEs, whose scratch stays
+# in the L2 (1.4 MB per RVE), so it has no entry.
 TRAFFIC_PER_LAUNCH = {("c2", "mg"): (125.4e3, "profiles/rve2d_kernel_mg_c2_macro16.md")}
 
 
