@@ -1690,10 +1690,11 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
     // all) are kept for the transfer too, as for the later Newton iterations: its fine level is
     // the converged tangent.  A transfer PCG that breaks down or hits its cap with kept levels
     // rebuilds the whole tangent with fresh levels and starts the transfer again.
-    bool reuse_t = kMG && mg.levels && a.mg_reuse && it > 0;
+    bool reuse_t = kMG && mg.levels && a.mg_reuse && it > 0, from_zero = false;
     for (;;) {
       build_tangent<TA, kMG, LAW>(o, sm, stage_k, Fb, phase, S, Minv, true, Lb, mg, !reuse_t);
       bool redo = false;
+      const bool kept = warm && !from_zero;
       int t_total = 0, t_max = 0, t_status = kStatusOk;
       for (int c = 0; c < 4; ++c) {
         TA b[4] = {TA(0), TA(0), TA(0), TA(0)};
@@ -1705,7 +1706,6 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
           b[3] = b1.y;
         }
         int pst = kStatusOk, ci = 0;
-        bool kept = warm;
         for (;;) {  // as for the Newton corrections: a breakdown is retried with half the damping
           if (kept && o.active) {
 #pragma unroll
@@ -1719,22 +1719,20 @@ __device__ __forceinline__ void solve_item_2d(const Rve2dArgs& a, int qp, const 
             redo = true;
             break;
           }
-          if (kMG && mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) &&
-              mg.omega > TA(0.2) * omega0) {
-            mg.omega *= TA(0.5);
-          } else if (kept && pst == kStatusPcgBreakdown) {
-            // A right-hand side far below the kept solution's (zero or rounding in a homogeneous RVE): the tolerance
-            // is relative to it and out of reach from there.  From zero it is not.
-            kept = false;
-            mg.omega = omega0;
-          } else {
+          if (!(kMG && mg.levels && (pst == kStatusPcgBreakdown || pst == kStatusPcgCap) &&
+                mg.omega > TA(0.2) * omega0))
             break;
-          }
+          mg.omega *= TA(0.5);
           pst = kStatusOk;
         }
         mg.omega = omega0;
         t_total += ci;
         t_max = ci > t_max ? ci : t_max;
+        if (kept && !redo && pst == kStatusPcgBreakdown) {
+          // A right-hand side far below the kept solution's (zero or rounding in a homogeneous RVE): the tolerance is
+          // relative to it and out of reach from there.  From zero it is not: the transfer once more.
+          redo = from_zero = true;
+        }
         if (redo) break;
         if (pst != kStatusOk && t_status == kStatusOk) t_status = pst;
       }
