@@ -454,7 +454,8 @@ const char* fehmm_status_str(int code);
  *   F, P, A, status, iters: as in fehmm_rve_solve (A may be NULL: no tangent)
  *   opt     host; dim must be 2 and precision FEHMM_PREC_FP64; tolerances, caps, bc, precond,
  *           mg_omega and mg_reuse used (multigrid on the grids that have it, and block-Jacobi where
- *           its PCG breaks down; block-Jacobi with FEHMM_PRECOND_BLOCK_JACOBI, and with an mg_omega
+ *           its PCG breaks down or meets a cap of 64 iterations or more; a lower cap truncates the
+ *           PCG and its step is taken; block-Jacobi with FEHMM_PRECOND_BLOCK_JACOBI, and with an mg_omega
  *           outside (0, 1), which is not refused here); law must be FEHMM_LAW_NEO_HOOKE (else
  *           FEHMM_ERR_UNSUPPORTED)
  * The first call on a device looks up the device address of the static array (with that
